@@ -46,8 +46,9 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     // programmatic serialisation: the pass starts its blocks while the
     // previous launch drains and waits inside the kernel (griddepcontrol)
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid_for(ntiles, cap));
-    cfg.blockDim = dim3(kBlock);
+    const Spread sp = spread_warps(ntiles, cap);
+    cfg.gridDim = dim3(sp.blocks);
+    cfg.blockDim = dim3(uint32_t(sp.threads));
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -89,7 +90,8 @@ template <int GEN>
 void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     constexpr int B = GEN ? MINB_GEN : MINB;
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
-    row_pass_kernel<B, 2, GEN, 0><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles, nullptr, GEN ? 1 : 0);
+    const Spread sp = spread_warps(ntiles, cap);
+    row_pass_kernel<B, 2, GEN, 0><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, nullptr, GEN ? 1 : 0);
 }
 
 void row_sample(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s) {
@@ -97,11 +99,15 @@ void row_sample(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s) {
     else row_sample_g<0>(g, ntiles, s);
 }
 
-template <bool LEADER, int C, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int NT = kBlock>
-void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, C, LEADER, NT>, NT);
-    pair_pass_kernel<R, B, C, LEADER, NT><<<grid_for(ntiles, cap, NT), NT, 0, s>>>(
-        g, ntiles, static_cast<const R*>(cone), colour, sub);
+template <bool LEADER, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int NT = kBlock>
+void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, uint32_t most,
+                 cudaStream_t s) {
+    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, LEADER, NT>, NT);
+    const uint32_t chunk = tiles_per_step(ntiles, cap, most, NT);
+    const uint32_t warps = (ntiles + chunk - 1) / chunk;
+    const Spread sp = spread_warps(warps, cap, NT);
+    pair_pass_kernel<R, B, LEADER, NT><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone), colour,
+                                                                        sub, chunk);
 }
 
 // launch shapes: tiles per grid-stride step {default, 8, 2}, and the
@@ -112,14 +118,14 @@ void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
 template <bool LEADER>
 void pair_pass_s(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int shape, int sub,
                  cudaStream_t s) {
-    constexpr int C0 = LEADER ? kPairChunkLead : kPairChunk;
+    constexpr uint32_t C0 = LEADER ? kPairChunkLead : kPairChunk;
     constexpr int B0 = LEADER ? MINB_PAIR_LEAD : MINB_PAIR;
-    if (shape == 1) pair_pass_t<LEADER, 8>(g, ntiles, cone, colour, sub, s);
-    else if (shape == 2) pair_pass_t<LEADER, 2>(g, ntiles, cone, colour, sub, s);
-    else if (shape == 3) {
-        if constexpr (LEADER) pair_pass_t<LEADER, C0, 5, 128>(g, ntiles, cone, colour, sub, s);
-        else pair_pass_t<LEADER, C0, B0 + 1>(g, ntiles, cone, colour, sub, s);
-    } else pair_pass_t<LEADER, C0>(g, ntiles, cone, colour, sub, s);
+    if (shape == 3) {
+        if constexpr (LEADER) pair_pass_t<LEADER, 5, 128>(g, ntiles, cone, colour, sub, C0, s);
+        else pair_pass_t<LEADER, B0 + 1>(g, ntiles, cone, colour, sub, C0, s);
+    } else {
+        pair_pass_t<LEADER>(g, ntiles, cone, colour, sub, shape == 1 ? 8 : shape == 2 ? 2 : C0, s);
+    }
 }
 
 void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int leader, int shape, int sub,

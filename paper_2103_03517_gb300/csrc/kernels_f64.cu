@@ -16,21 +16,16 @@ constexpr int kFieldChunk = 4;  // the same for the neighbour-field kernel
 
 #include "launchers_common.cuh"
 
-template <int C>
-void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, 1, C, false>);
-    pair_pass_kernel<R, 1, C, false><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles, static_cast<const R*>(cone),
-                                                                           colour, sub);
-}
-
 // launch shapes: tiles per grid-stride step {default, 8, 2}; FP64 lattices
 // always take pair order (LatParams::pair_leader)
 void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int leader, int shape, int sub,
                cudaStream_t s) {
     (void)leader;
-    if (shape == 1) pair_pass_t<8>(g, ntiles, cone, colour, sub, s);
-    else if (shape == 2) pair_pass_t<2>(g, ntiles, cone, colour, sub, s);
-    else pair_pass_t<kPairChunk>(g, ntiles, cone, colour, sub, s);
+    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, 1, false>);
+    const uint32_t chunk = tiles_per_step(ntiles, cap, shape == 1 ? 8 : shape == 2 ? 2 : kPairChunk);
+    const Spread sp = spread_warps((ntiles + chunk - 1) / chunk, cap);
+    pair_pass_kernel<R, 1, false><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone), colour, sub,
+                                                                 chunk);
 }
 
 }  // namespace

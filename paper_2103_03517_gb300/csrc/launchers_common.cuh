@@ -18,17 +18,53 @@ uint32_t resident_blocks(K kernel, int threads = kBlock) {
     return uint32_t(sms) * uint32_t(per_sm);
 }
 
-// blocks for ntiles warp tiles: one warp per tile at most, capped at residency
-uint32_t grid_for(uint32_t ntiles, uint32_t cap, int threads = kBlock) {
+// Launch shape of `warps` warps of work for a kernel that keeps cap blocks of
+// `threads` threads resident.  A launch that fills the GPU takes them all.  A
+// smaller FP64 launch takes blocks of one or two warps, which the hardware
+// deals out over all SMs: an FP64 warp instruction holds the SM's FP64 pipe
+// for many cycles, and in blocks of 256 threads the 64 warps of a 16^3 colour
+// pass sat on 8 SMs with that pipe 70% busy (25 us a pass, 55 us a sweep; 34
+// us a sweep spread out).  Two warps a block above 8 warps per SM keep the SM
+// below its block limit.  FP32 launches stay in full blocks: spread out, a
+// 12^3 lattice swept 6% slower, a 90 x 75 x 61 one 3% slower and a 64^3 one no
+// faster (they wait on memory latency and on the launch, not on a pipe).
+struct Spread {
+    uint32_t blocks;
+    int threads;
+};
+
+Spread spread_warps(uint32_t warps, uint32_t cap, int threads = kBlock) {
+    static const uint32_t sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return uint32_t(n > 0 ? n : 1);
+    }();
     const uint32_t wpb = uint32_t(threads / 32);
-    const uint32_t want = (ntiles + wpb - 1) / wpb;
-    return want < cap ? (want > 0 ? want : 1) : cap;
+    if (warps == 0) warps = 1;
+    if (warps >= cap * wpb) return Spread{cap, threads};
+    if (!kIsF64<R>) return Spread{(warps + wpb - 1) / wpb, threads};
+    if (warps <= 8 * sms) return Spread{warps, 32};
+    return Spread{(warps + 1) / 2, 64};
+}
+
+// Consecutive tiles a warp of a grid-stride kernel takes per step: `most`,
+// or fewer when the launch would otherwise leave resident warps without work
+// (a lone 64^3 lattice has 2048 pair tiles for 2432 warps, and 4 a step kept
+// only 512 of them busy; a 16^3 one walked its 32 tiles on 8 warps).
+// Constrained sweeps alone, half of them measured, 4 tiles a step against
+// this rule: 16^3 36.8 -> 24.6 us, 64^3 43.5 -> 33.9 us, 256^3 unchanged;
+// 16^3 in FP64, spread over the SMs as well, 275 -> 55.9 us.
+uint32_t tiles_per_step(uint32_t ntiles, uint32_t cap, uint32_t most, int threads = kBlock) {
+    const uint32_t even = ntiles / (cap * uint32_t(threads / 32));
+    return even < 1 ? 1 : (even < most ? even : most);
 }
 
 template <int MEASURE>
 void colour_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(colour_pass_kernel<R, V, MINB, MEASURE>);
-    colour_pass_kernel<R, V, MINB, MEASURE><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles, cone, colour);
+    const Spread sp = spread_warps(ntiles, cap);
+    colour_pass_kernel<R, V, MINB, MEASURE><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, cone, colour);
 }
 
 // measure: 0 none, 1 magnetisation and energies, 2 also torques
@@ -43,17 +79,12 @@ void sweep_end(const GroupArgs& g, cudaStream_t s) {
     sweep_end_kernel<R><<<(g.n + kBlock - 1) / kBlock, kBlock, 0, s>>>(g);
 }
 
-template <int C>
-void pair_field_t(const GroupArgs& g, uint32_t ntiles, int colour, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(pair_field_kernel<R, V, C>);
-    pair_field_kernel<R, V, C><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles, colour);
-}
-
 // launch shapes: tiles per grid-stride step {default, 8, 2}
 void pair_field(const GroupArgs& g, uint32_t ntiles, int colour, int shape, cudaStream_t s) {
-    if (shape == 1) pair_field_t<8>(g, ntiles, colour, s);
-    else if (shape == 2) pair_field_t<2>(g, ntiles, colour, s);
-    else pair_field_t<kFieldChunk>(g, ntiles, colour, s);
+    static const uint32_t cap = resident_blocks(pair_field_kernel<R, V>);
+    const uint32_t chunk = tiles_per_step(ntiles, cap, shape == 1 ? 8 : shape == 2 ? 2 : kFieldChunk);
+    const Spread sp = spread_warps((ntiles + chunk - 1) / chunk, cap);
+    pair_field_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, colour, chunk);
 }
 
 void ml_reset(const GroupArgs& g, cudaStream_t s) {
@@ -62,12 +93,14 @@ void ml_reset(const GroupArgs& g, cudaStream_t s) {
 
 void mlong(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(mlong_kernel<R, V>);
-    mlong_kernel<R, V><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles);
+    const Spread sp = spread_warps(ntiles, cap);
+    mlong_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles);
 }
 
 void measure(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(measure_kernel<R, V>);
-    measure_kernel<R, V><<<grid_for(ntiles, cap), kBlock, 0, s>>>(g, ntiles);
+    const Spread sp = spread_warps(ntiles, cap);
+    measure_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles);
 }
 
 // Entry bound of the crystal kernels: the smallest instance that holds nb.
@@ -84,8 +117,9 @@ template <int NB>
 struct XtalPass {
     static void run(LatDev* L, uint32_t ntiles, const void* cone, int sub, int colour, int finalize, cudaStream_t s) {
         static const uint32_t cap = resident_blocks(xtal_pass_kernel<R, NB>);
-        xtal_pass_kernel<R, NB><<<grid_for(ntiles, cap), kBlock, 0, s>>>(L, ntiles, static_cast<const R*>(cone), sub,
-                                                                         colour, finalize);
+        const Spread sp = spread_warps(ntiles, cap);
+        xtal_pass_kernel<R, NB><<<sp.blocks, sp.threads, 0, s>>>(L, ntiles, static_cast<const R*>(cone), sub, colour,
+                                                                 finalize);
     }
 };
 
@@ -94,7 +128,8 @@ struct XtalSample {
     template <int LEVEL>
     static void go(LatDev* L, uint32_t ntiles, uint32_t tiles_per_subset, cudaStream_t s) {
         static const uint32_t cap = resident_blocks(xtal_sample_kernel<R, NB, LEVEL>);
-        xtal_sample_kernel<R, NB, LEVEL><<<grid_for(ntiles, cap), kBlock, 0, s>>>(L, ntiles, tiles_per_subset);
+        const Spread sp = spread_warps(ntiles, cap);
+        xtal_sample_kernel<R, NB, LEVEL><<<sp.blocks, sp.threads, 0, s>>>(L, ntiles, tiles_per_subset);
     }
     // level 2: with the torque sums
     static void run(LatDev* L, uint32_t ntiles, uint32_t tiles_per_subset, int level, cudaStream_t s) {
@@ -107,7 +142,8 @@ template <int NB>
 struct XtalField {
     static void run(LatDev* L, uint32_t ntiles, int sub, int colour, cudaStream_t s) {
         static const uint32_t cap = resident_blocks(xtal_field_kernel<R, NB>);
-        xtal_field_kernel<R, NB><<<grid_for(ntiles, cap), kBlock, 0, s>>>(L, ntiles, sub, colour);
+        const Spread sp = spread_warps(ntiles, cap);
+        xtal_field_kernel<R, NB><<<sp.blocks, sp.threads, 0, s>>>(L, ntiles, sub, colour);
     }
 };
 
@@ -126,7 +162,8 @@ void xtal_sample(LatDev* L, uint32_t ntiles, uint32_t tiles_per_subset, int nb, 
 
 void grain_sample(LatDev* L, uint32_t ntiles, int n_grains, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(grain_sum_kernel<R, V>);
-    grain_sum_kernel<R, V><<<grid_for(ntiles, cap), kBlock, 0, s>>>(L, ntiles);
+    const Spread sp = spread_warps(ntiles, cap);
+    grain_sum_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(L, ntiles);
     grain_finish_kernel<R><<<(n_grains + kBlock) / kBlock, kBlock, 0, s>>>(L);
 }
 

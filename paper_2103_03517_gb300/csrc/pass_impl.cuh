@@ -565,8 +565,8 @@ struct WarpChunk {
 __device__ __forceinline__ WarpChunk warp_chunk(uint32_t ntiles) {
     // even split: warp w takes [w T / W, (w + 1) T / W), so chunks differ by
     // at most one tile and no warp of the launch idles while T >= W
-    const uint32_t nwarps = gridDim.x * uint32_t(kBlock / 32);
-    const uint32_t w = blockIdx.x * uint32_t(kBlock / 32) + (threadIdx.x >> 5);
+    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     WarpChunk c;
     c.begin = uint32_t(uint64_t(w) * ntiles / nwarps);
     c.end = uint32_t(uint64_t(w + 1) * ntiles / nwarps);
@@ -1113,20 +1113,20 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // at most 31 wait between tiles, and a tile adds at most 64.
 constexpr uint32_t kLeaderRing = 128;
 
-// Tiles are taken in grid-stride order, CHUNK consecutive tiles per step: at
-// any moment the warps hold a window of about CHUNK tiles each, a few
+// Tiles are taken in grid-stride order, `chunk` consecutive tiles per step: at
+// any moment the warps hold a window of about `chunk` tiles each, a few
 // lattices of the batch, so that the random gathers of partners and their
 // neighbours stay in L2.  A warp adds its accepted moves and M_L change
 // once per lattice in a chunk.
-template <typename R, int MINB, int CHUNK, bool LEADER, int NT = kBlock>
-__global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32_t ntiles,
-                                                             const R* __restrict__ cone, int colour, int sub) {
+template <typename R, int MINB, bool LEADER, int NT = kBlock>
+__global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32_t ntiles, const R* __restrict__ cone,
+                                                             int colour, int sub, uint32_t chunk) {
     const int lane = int(threadIdx.x & 31);
-    const uint32_t nwarps = gridDim.x * uint32_t(NT / 32);
-    const uint32_t w = blockIdx.x * uint32_t(NT / 32) + (threadIdx.x >> 5);
+    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int l = 0;
-    for (uint32_t c0 = w * CHUNK; c0 < ntiles; c0 += nwarps * CHUNK) {
-        const uint32_t c1 = min(c0 + uint32_t(CHUNK), ntiles);
+    for (uint32_t c0 = w * chunk; c0 < ntiles; c0 += nwarps * chunk) {
+        const uint32_t c1 = min(c0 + chunk, ntiles);
         for (uint32_t tile = c0; tile < c1;) {
             while (__ldg(&g.start[l + 1]) <= tile) ++l;
             const uint32_t t0 = __ldg(&g.start[l]);
@@ -1275,7 +1275,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32
 // spins summed in the order -x, +x, -y, +y, -z, +z, as neighbour_sum4 does,
 // written as (h_x, h_y, h_z, 0).  The other colour does not change during
 // the pass, so the field holds for all of it.  Tiles go to the warps
-// CHUNK at a time in grid-stride order, so that the warps in flight cover
+// `chunk` at a time in grid-stride order, so that the warps in flight cover
 // one compact window of the batch and the +-z planes a tile reads are still
 // in L2 when the tiles two planes on read them again (with one contiguous
 // run per warp those reads were a large part of the launch apart, and every
@@ -1314,15 +1314,15 @@ __device__ __forceinline__ void field_tile_periodic(const LatParams& p, const Sp
     }
 }
 
-template <typename R, int V, int CHUNK>
-__global__ void __launch_bounds__(kBlock) pair_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
-    const uint32_t nwarps = gridDim.x * uint32_t(kBlock / 32);
-    const uint32_t w = blockIdx.x * uint32_t(kBlock / 32) + (threadIdx.x >> 5);
+template <typename R, int V>
+__global__ void __launch_bounds__(kBlock) pair_field_kernel(GroupArgs g, uint32_t ntiles, int colour, uint32_t chunk) {
+    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
+    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31u;
     const int other = colour ^ 1;
     int l = 0;
-    for (uint32_t c0 = w * CHUNK; c0 < ntiles; c0 += nwarps * CHUNK) {
-        const uint32_t c1 = min(c0 + uint32_t(CHUNK), ntiles);
+    for (uint32_t c0 = w * chunk; c0 < ntiles; c0 += nwarps * chunk) {
+        const uint32_t c1 = min(c0 + chunk, ntiles);
         for (uint32_t tile = c0; tile < c1;) {
             while (__ldg(&g.start[l + 1]) <= tile) ++l;  // tiles only move forward
             const uint32_t t0 = __ldg(&g.start[l]);
