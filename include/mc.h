@@ -46,8 +46,8 @@ typedef enum mc_status {
     MC_ERR_ARG = -1,        /* invalid argument (checked on the host)            */
     MC_ERR_NOMEM = -2,      /* device memory exhausted / job can never fit       */
     MC_ERR_CUDA = -3,       /* a CUDA call failed (message in mc_last_error)     */
-    MC_ERR_TIMEOUT = -4,    /* a bounded device wait gave up (the wavefront and  */
-                            /* resident kernels' waits, about one second each;   */
+    MC_ERR_TIMEOUT = -4,    /* a bounded device wait gave up (the wavefront,     */
+                            /* resident and brick kernels' waits, about one second each;   */
                             /* MC_WAVE_INJECT_TIMEOUT=1 or                       */
                             /* MC_RESIDENT_INJECT_TIMEOUT=1 in the environment   */
                             /* when a lattice is created makes its first wait    */
@@ -72,9 +72,13 @@ typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIP
  * passes where the row layout applies (Lh = Lx/2 a power of two <= 64 or a
  * multiple of 64, Nc a multiple of 64) and the general kernel otherwise,
  * and walks the constrained pairs in site order (each pair led by the
- * member whose shuffled position is even); an all-periodic lattice with
- * Lx = 128 and no film tables whose rows fit the SMs' shared memory sweeps
- * resident when it runs alone (see RESIDENT).  GENERAL always takes the
+ * member whose shuffled position is even); a lattice without film tables
+ * whose rows fit the SMs' shared memory (up to about 2.8 million spins) runs
+ * its unconstrained sweeps held there when it runs alone, in calls of at least
+ * 3 sweeps: a 128-wide all-periodic one of 1.5 million spins and more resident
+ * (see RESIDENT), any other as brick sweeps, one cooperative launch per call of
+ * up to 2048 sweeps (512 measured), for which it takes 16 bytes per spin of
+ * device memory on first use (without them it sweeps by launches).  GENERAL always takes the
  * general colour-pass kernel and the pairs in pair order.  ROW is AUTO
  * without the resident sweeps: the row kernels for every colour pass.
  * WAVE is ROW, except that on an all-periodic lattice with Lx = 128 and
@@ -82,7 +86,7 @@ typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIP
  * call run two at a time as single wavefront launches (red and black pass
  * fused, each spin read and written once per sweep; the lattice then holds
  * a second spin buffer, and an odd last sweep of a call runs as two row
- * passes).  RESIDENT is AUTO, named: an all-periodic lattice with Lx = 128
+ * passes).  RESIDENT is AUTO, except that an all-periodic lattice with Lx = 128
  * (no film tables) whose rows fit the SMs' shared memory (about 30 MB of
  * spins on 152 SMs, e.g. 128^3) sweeps, when it runs alone (mc_sweep, or a
  * group of that one lattice), held in shared memory: one cooperative launch

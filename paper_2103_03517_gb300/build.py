@@ -27,6 +27,7 @@ COMMON = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC,-fvisibility=hi
 SOURCES = {
     "kernels_f64.cu": ["-fmad=false", "-prec-div=true", "-prec-sqrt=true"],
     "kernels_f32.cu": ["--use_fast_math"],
+    "kernels_brick.cu": ["--use_fast_math"],
     "runtime.cpp": [],
     "groups.cpp": [],
     "tune.cpp": [],

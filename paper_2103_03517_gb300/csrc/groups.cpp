@@ -137,6 +137,10 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
         g->ls.res = g->res_plans.data();
         g->ls.n_res = n;
     }
+    if (n == 1) {
+        g->ls.brick = lattices[0]->brick;
+        g->ls.brick_lh = uint32_t(lattices[0]->hp.Lh);
+    }
     g->ls.sample_level = 1;
     for (int i = 0; i < n; ++i)
         if (lattices[i]->hp.sample_torque) g->ls.sample_level = 2;

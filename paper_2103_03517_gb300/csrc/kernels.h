@@ -137,6 +137,10 @@ struct LaunchSet {
     // plans, owned by the lattices (none: n_res = 0)
     ResidentPlan* const* res = nullptr;
     int n_res = 0;
+    // a lattice alone whose unconstrained sweeps run as brick launches, else
+    // null; its Lh
+    BrickArgs* brick = nullptr;
+    uint32_t brick_lh = 0;
     int sample_level = 2;  // sample of a measured colour pass: 1 or 2 (torques)
     // a bcc / fcc lattice alone: its descriptor and sub-lattice count, else null
     LatDev* xtal = nullptr;
@@ -144,6 +148,14 @@ struct LaunchSet {
     int xnb_max = 0;  // most neighbour entries of its sub-lattices
     LaunchShape shape;  // autotuned launch shapes
 };
+
+// Brick sweeps (brick_pass.cuh; FP32 simple cubic lattices without film
+// tables): the split of lattice p (host copy) over the current device's SMs,
+// everything of out but its pointers and key; false when its rows do not fit
+// their shared memory.  Then n sweeps of a plan in cooperative launches of at
+// most kResMaxSweeps, measure as for colour_pass.
+bool brick_plan(const LatParams& p, BrickArgs* out);
+cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, cudaStream_t s);
 
 const KernelSet& kernels_f64();
 const KernelSet& kernels_f32();

@@ -99,18 +99,15 @@ void row_sample(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s) {
     else row_sample_g<0>(g, ntiles, s);
 }
 
-template <bool LEADER, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int NT = kBlock>
-void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, uint32_t most,
-                 cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, LEADER, NT>, NT);
-    const uint32_t chunk = tiles_per_step(ntiles, cap, most, NT);
-    const uint32_t warps = (ntiles + chunk - 1) / chunk;
-    const Spread sp = spread_warps(warps, cap, NT);
-    pair_pass_kernel<R, B, LEADER, NT><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone), colour,
-                                                                        sub, chunk);
+template <bool LEADER, int C, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int NT = kBlock>
+void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, cudaStream_t s) {
+    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, C, LEADER, NT>, NT);
+    const Spread sp = spread_warps((ntiles + C - 1) / C, cap, NT);
+    pair_pass_kernel<R, B, C, LEADER, NT><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone),
+                                                                           colour, sub);
 }
 
-// launch shapes: tiles per grid-stride step {default, 8, 2}, and the
+// launch shapes: at most {default, 8, 2} tiles per grid-stride step, and the
 // default step with more resident warps per SM: pair order one more block
 // of 256 threads (fewer registers, some spilled), site order blocks of 128
 // threads, five per SM (20 warps at up to 102 registers, against 16 warps
@@ -118,14 +115,17 @@ void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
 template <bool LEADER>
 void pair_pass_s(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int shape, int sub,
                  cudaStream_t s) {
-    constexpr uint32_t C0 = LEADER ? kPairChunkLead : kPairChunk;
+    constexpr int C0 = LEADER ? kPairChunkLead : kPairChunk;
     constexpr int B0 = LEADER ? MINB_PAIR_LEAD : MINB_PAIR;
-    if (shape == 3) {
-        if constexpr (LEADER) pair_pass_t<LEADER, 5, 128>(g, ntiles, cone, colour, sub, C0, s);
-        else pair_pass_t<LEADER, B0 + 1>(g, ntiles, cone, colour, sub, C0, s);
-    } else {
-        pair_pass_t<LEADER>(g, ntiles, cone, colour, sub, shape == 1 ? 8 : shape == 2 ? 2 : C0, s);
-    }
+    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B0, C0, LEADER>);
+    const int c = tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : C0);
+    if (c == 1) pair_pass_t<LEADER, 1>(g, ntiles, cone, colour, sub, s);
+    else if (c == 2) pair_pass_t<LEADER, 2>(g, ntiles, cone, colour, sub, s);
+    else if (c == 8) pair_pass_t<LEADER, 8>(g, ntiles, cone, colour, sub, s);
+    else if (shape == 3) {
+        if constexpr (LEADER) pair_pass_t<LEADER, C0, 5, 128>(g, ntiles, cone, colour, sub, s);
+        else pair_pass_t<LEADER, C0, B0 + 1>(g, ntiles, cone, colour, sub, s);
+    } else pair_pass_t<LEADER, C0>(g, ntiles, cone, colour, sub, s);
 }
 
 void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int leader, int shape, int sub,

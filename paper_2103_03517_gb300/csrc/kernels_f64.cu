@@ -16,16 +16,25 @@ constexpr int kFieldChunk = 4;  // the same for the neighbour-field kernel
 
 #include "launchers_common.cuh"
 
-// launch shapes: tiles per grid-stride step {default, 8, 2}; FP64 lattices
-// always take pair order (LatParams::pair_leader)
+template <int C>
+void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, int sub, uint32_t cap,
+                 cudaStream_t s) {
+    const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
+    pair_pass_kernel<R, 1, C, false><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, cone, colour, sub);
+}
+
+// launch shapes: at most {default, 8, 2} tiles per grid-stride step; FP64
+// lattices always take pair order (LatParams::pair_leader)
 void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int leader, int shape, int sub,
                cudaStream_t s) {
     (void)leader;
-    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, 1, false>);
-    const uint32_t chunk = tiles_per_step(ntiles, cap, shape == 1 ? 8 : shape == 2 ? 2 : kPairChunk);
-    const Spread sp = spread_warps((ntiles + chunk - 1) / chunk, cap);
-    pair_pass_kernel<R, 1, false><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone), colour, sub,
-                                                                 chunk);
+    static const uint32_t cap = resident_blocks(pair_pass_kernel<R, 1, kPairChunk, false>);
+    const R* c64 = static_cast<const R*>(cone);
+    const int c = tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : kPairChunk);
+    if (c == 8) pair_pass_t<8>(g, ntiles, c64, colour, sub, cap, s);
+    else if (c == 4) pair_pass_t<4>(g, ntiles, c64, colour, sub, cap, s);
+    else if (c == 2) pair_pass_t<2>(g, ntiles, c64, colour, sub, cap, s);
+    else pair_pass_t<1>(g, ntiles, c64, colour, sub, cap, s);
 }
 
 }  // namespace

@@ -48,16 +48,17 @@ Spread spread_warps(uint32_t warps, uint32_t cap, int threads = kBlock) {
     return Spread{(warps + 1) / 2, 64};
 }
 
-// Consecutive tiles a warp of a grid-stride kernel takes per step: `most`,
-// or fewer when the launch would otherwise leave resident warps without work
-// (a lone 64^3 lattice has 2048 pair tiles for 2432 warps, and 4 a step kept
-// only 512 of them busy; a 16^3 one walked its 32 tiles on 8 warps).
-// Constrained sweeps alone, half of them measured, 4 tiles a step against
-// this rule: 16^3 36.8 -> 24.6 us, 64^3 43.5 -> 33.9 us, 256^3 unchanged;
-// 16^3 in FP64, spread over the SMs as well, 275 -> 55.9 us.
-uint32_t tiles_per_step(uint32_t ntiles, uint32_t cap, uint32_t most, int threads = kBlock) {
-    const uint32_t even = ntiles / (cap * uint32_t(threads / 32));
-    return even < 1 ? 1 : (even < most ? even : most);
+// Consecutive tiles a warp of a grid-stride kernel takes per step (an instance
+// each): `most` (2, 4 or 8), or 2 or 1 when the launch would otherwise leave
+// resident warps without work (a lone 64^3 lattice has 2048 pair tiles for
+// 2432 warps, and 4 a step kept only 512 of them busy; a 16^3 one walked its
+// 32 tiles on 8 warps).  Constrained sweeps alone, half of them measured, 4
+// tiles a step against this rule: 16^3 36.8 -> 24.6 us, 64^3 43.5 -> 33.9 us,
+// 256^3 unchanged; 16^3 in FP64, spread over the SMs as well, 275 -> 55.9 us.
+int tiles_per_step(uint32_t ntiles, uint32_t warps, int most) {
+    const uint32_t even = ntiles / warps;
+    if (even >= uint32_t(most)) return most;
+    return even >= 2 ? 2 : 1;
 }
 
 template <int MEASURE>
@@ -79,12 +80,20 @@ void sweep_end(const GroupArgs& g, cudaStream_t s) {
     sweep_end_kernel<R><<<(g.n + kBlock - 1) / kBlock, kBlock, 0, s>>>(g);
 }
 
-// launch shapes: tiles per grid-stride step {default, 8, 2}
+template <int C>
+void pair_field_t(const GroupArgs& g, uint32_t ntiles, int colour, uint32_t cap, cudaStream_t s) {
+    const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
+    pair_field_kernel<R, V, C><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, colour);
+}
+
+// launch shapes: at most {default, 8, 2} tiles per grid-stride step
 void pair_field(const GroupArgs& g, uint32_t ntiles, int colour, int shape, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(pair_field_kernel<R, V>);
-    const uint32_t chunk = tiles_per_step(ntiles, cap, shape == 1 ? 8 : shape == 2 ? 2 : kFieldChunk);
-    const Spread sp = spread_warps((ntiles + chunk - 1) / chunk, cap);
-    pair_field_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, colour, chunk);
+    static const uint32_t cap = resident_blocks(pair_field_kernel<R, V, kFieldChunk>);
+    const int c = tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : kFieldChunk);
+    if (c == 8) pair_field_t<8>(g, ntiles, colour, cap, s);
+    else if (c == 4) pair_field_t<4>(g, ntiles, colour, cap, s);
+    else if (c == 2) pair_field_t<2>(g, ntiles, colour, cap, s);
+    else pair_field_t<1>(g, ntiles, colour, cap, s);
 }
 
 void ml_reset(const GroupArgs& g, cudaStream_t s) {

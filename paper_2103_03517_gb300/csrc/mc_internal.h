@@ -243,4 +243,41 @@ struct ResidentArgs {
     uint32_t key0, key1;  // the lattice's Philox key, a launch constant
 };
 
+// Brick sweeps (brick_pass.cuh): control words of one lattice, in device
+// memory.  Zeroed before every launch but the epoch, which the launch counts
+// up (1 at create): the abort flag; the blocks of brick_close_kernel that are
+// done; by the sweep's parity, running totals of the blocks done (bits 40 up)
+// and of their accepted moves.
+constexpr int kBrickMaxBlocks = 256;
+struct BrickCtl {
+    int abort;
+    unsigned int closed;
+    unsigned long long count[2];
+    uint32_t epoch;
+};
+
+// What a measured sweep of a brick launch leaves behind: its fixed-point
+// sample sums, cone angle and accepted count, in whose place brick_close_kernel
+// puts what each moment word grows by.
+constexpr int kBrickRecord = 28;        // 8-byte words, at least kMomentWords
+constexpr int kBrickRecTheta = kNumSums, kBrickRecAcc = kNumSums + 1;
+constexpr int kBrickMaxMeasured = 512;  // measured sweeps per launch
+
+// A brick launch: nyc x nzc bricks of rows (odd Lh: nyc blocks, runs of
+// rows), at most `rows` rows in a block; packets: 16 bytes per site, [2]
+// [stride]; inject as in ResidentArgs.
+struct BrickArgs {
+    LatDev* lat;
+    BrickCtl* ctl;
+    void* packets;
+    long long* record;    // [kBrickMaxMeasured][kBrickRecord]
+    uint32_t nyc, nzc, rows, smem;
+    FastDiv div_half;     // by Lh / 2
+    size_t bytes;         // of the lattice's brick memory: ctl (null until it is allocated), record, packets
+    int law, faces;       // kernel instance: packed or scalar law, any boundaries
+    int n_sweeps;
+    int inject;
+    uint32_t key0, key1;  // the lattice's Philox key, a launch constant
+};
+
 }  // namespace mcgb

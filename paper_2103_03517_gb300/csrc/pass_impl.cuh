@@ -359,6 +359,20 @@ struct Sums {
     R v[kNumSums];
 };
 
+// a b - c d and a^2 + b^2: in FP64 one IEEE operation at a time, in FP32 with
+// the second product rounded and the first fused into the sum.
+template <typename R>
+__device__ __forceinline__ R diff_of_products(R a, R b, R c, R d) {
+    if constexpr (kIsF64<R>) return a * b - c * d;
+    else return __fmaf_rn(a, b, -__fmul_rn(c, d));
+}
+
+template <typename R>
+__device__ __forceinline__ R sum_of_squares(R a, R b) {
+    if constexpr (kIsF64<R>) return a * a + b * b;
+    else return __fmaf_rn(a, a, __fmul_rn(b, b));
+}
+
 // Sample sums of one site: LEVEL 1 = magnetisation and the single-site
 // energy sums, LEVEL 2 = also the torque sums.  FP32 skips the uniaxial or
 // cubic sum when its constant is zero (its energy is zero whatever the sum).
@@ -371,14 +385,17 @@ __device__ __forceinline__ void add_site(Sums<R>& s, V3<R> S, V3<R> e, bool need
     if (kIsF64<R> || need_u) s.v[kSumU] += pe * pe;
     if (kIsF64<R> || need_c) s.v[kSumC] += cubic_q(S);
     if constexpr (LEVEL >= 2) {
-        s.v[kSumTux] += pe * (S.y * e.z - S.z * e.y);
-        s.v[kSumTuy] += pe * (S.z * e.x - S.x * e.z);
-        s.v[kSumTuz] += pe * (S.x * e.y - S.y * e.x);
-        const R x2 = S.x * S.x, y2 = S.y * S.y, z2 = S.z * S.z;
-        const R c0 = S.x * (y2 + z2), c1 = S.y * (x2 + z2), c2 = S.z * (x2 + y2);
-        s.v[kSumTcx] += S.y * c2 - S.z * c1;
-        s.v[kSumTcy] += S.z * c0 - S.x * c2;
-        s.v[kSumTcz] += S.x * c1 - S.y * c0;
+        // differences of products with the second product rounded first, in so
+        // many words: left to the compiler, the choice differs between kernels
+        // and with it the last bits of a torque
+        s.v[kSumTux] += pe * diff_of_products(S.y, e.z, S.z, e.y);
+        s.v[kSumTuy] += pe * diff_of_products(S.z, e.x, S.x, e.z);
+        s.v[kSumTuz] += pe * diff_of_products(S.x, e.y, S.y, e.x);
+        const R c0 = S.x * sum_of_squares(S.y, S.z), c1 = S.y * sum_of_squares(S.x, S.z),
+                c2 = S.z * sum_of_squares(S.x, S.y);
+        s.v[kSumTcx] += diff_of_products(S.y, c2, S.z, c1);
+        s.v[kSumTcy] += diff_of_products(S.z, c0, S.x, c2);
+        s.v[kSumTcz] += diff_of_products(S.x, c1, S.y, c0);
     }
 }
 
@@ -442,6 +459,85 @@ __device__ inline long long close_counts(const LatParams& p, LatState& st, int m
 __device__ inline void finalize_sweep_unmeasured(const LatParams& p, LatState& st) {
     close_counts(p, st, 0, p.n_mov);
     st.sweep += 1;
+}
+
+// The sample of Sec. 3 from the fixed-point sums (lane i holds sum i):
+// *inc receives what moment word `lane` grows by and *y the quotient that ring
+// word `lane` holds (lanes 3-12).  For the samples of a whole run at once
+// (brick_close_kernel); finalize_sweep below evaluates the same expressions in
+// line, since calling this there made a resident sweep 1% and a small batch 3%
+// slower.
+__device__ __forceinline__ void sample_words(const LatParams& p, long long sum, bool torque, int lane, long long N, double* inc,
+                                    double* y) {
+    constexpr unsigned kAll = 0xffffffffu;
+    // the scales are powers of two, so the products are the quotients
+    const double inv_scale = p.precision == 1 ? 1.0 / kFixScale : 1.0 / kFixScaleF32;
+    double mine = 0.0;
+    if (lane < kNumSums) mine = double(sum) * inv_scale;
+    // the sums each numerator needs, fetched by per-lane shuffles: lanes
+    // 0-2 m_a; 3-5 the exchange, uniaxial and cubic sums; 6 the three m
+    // components (Zeeman); 7 + a the torque sums of axis a and the two
+    // other m components (their field cross product)
+    const int a = lane - 7;  // torque axis of lanes 7-9
+    const int a1 = a == 0 ? 1 : (a == 1 ? 2 : 0), a2 = a == 0 ? 2 : (a == 1 ? 0 : 1);
+    const int i1 = lane < 3 ? kSumMx + lane
+                   : lane == 3 ? kSumEx
+                   : lane == 4 ? kSumU
+                   : lane == 5 ? kSumC
+                   : lane == 6 ? kSumMx
+                   : lane < 10 ? kSumTux + a
+                               : 0;
+    const int i2 = lane == 6 ? kSumMy : (lane >= 7 && lane < 10 ? kSumTcx + a : 0);
+    const int i3 = lane == 6 ? kSumMz : (lane >= 7 && lane < 10 ? kSumMx + a1 : 0);
+    const int i4 = lane >= 7 && lane < 10 ? kSumMx + a2 : 0;
+    const double s1 = __shfl_sync(kAll, mine, i1), s2 = __shfl_sync(kAll, mine, i2);
+    const double s3 = __shfl_sync(kAll, mine, i3), s4 = __shfl_sync(kAll, mine, i4);
+    double num = 0.0;
+    if (lane < 3) num = s1;
+    else if (lane == 3) num = -p.J * s1;
+    else if (lane == 4) num = -p.Ku * s1;
+    else if (lane == 5) num = p.Kc * s1;
+    else if (lane == 6) num = -(p.H[0] * s1 + p.H[1] * s2 + p.H[2] * s3);
+    else if (lane < 10 && torque) num = 2.0 * p.Ku * s1 - 2.0 * p.Kc * s2 + (s3 * p.H[a2] - s4 * p.H[a1]);
+    const double quo = num / double(N);
+    // lanes 0-2: m; 3-6: the energy parts E_ex, E_u, E_c, E_Z; 7-9: tau
+    const double m0 = __shfl_sync(kAll, quo, 0), m1 = __shfl_sync(kAll, quo, 1), m2 = __shfl_sync(kAll, quo, 2);
+    const double e_ex = __shfl_sync(kAll, quo, 3), e_u = __shfl_sync(kAll, quo, 4);
+    const double e_c = __shfl_sync(kAll, quo, 5), e_z = __shfl_sync(kAll, quo, 6);
+    const double ml2 = m0 * m0 + m1 * m1 + m2 * m2;
+    const double ml = sqrt(ml2);
+    const double e = e_ex + e_u + e_c + e_z;
+    // moment word `lane`, in the order of the enum: N, m_a, m_a^2, |m_a|,
+    // |m|, |m|^2, |m|^4, E, E^2, the four parts, tau_a, tau_a^2; x is the
+    // quotient the word is built from (m_a, a part or tau_a)
+    const int src = lane < kMomM2     ? lane - kMomM
+                    : lane < kMomMabs ? lane - kMomM2
+                    : lane < kMomMl   ? lane - kMomMabs
+                    : lane < kMomParts ? 0
+                    : lane < kMomTq   ? 3 + lane - kMomParts
+                    : lane < kMomTq2  ? 7 + lane - kMomTq
+                    : lane < kMomTq2 + 3 ? 7 + lane - kMomTq2
+                                      : 0;
+    const double x = __shfl_sync(kAll, quo, src < 0 ? 0 : src);
+    *inc = lane == kMomN      ? 1.0
+                       : lane < kMomM2    ? x
+                       : lane < kMomMabs  ? x * x
+                       : lane < kMomMl    ? fabs(x)
+                       : lane == kMomMl   ? ml
+                       : lane == kMomMl2  ? ml2
+                       : lane == kMomMl4  ? ml2 * ml2
+                       : lane == kMomE    ? e
+                       : lane == kMomE2   ? e * e
+                       : lane < kMomTq    ? x
+                       : lane < kMomTq2   ? x
+                                          : x * x;
+    // ring word `lane`: sweep, theta, accepted, m, the four parts, tau, 0
+    *y = __shfl_sync(kAll, quo, lane >= 3 && lane < 13 ? lane - 3 : 0);
+}
+
+// Ring word `lane` of a sample (lanes below kRingWords).
+__device__ __forceinline__ double ring_word(int lane, uint32_t sweep, int theta, long long acc, double y) {
+    return lane == 0 ? double(sweep) : lane == 1 ? double(theta) : lane == 2 ? double(acc) : lane < 13 ? y : 0.0;
 }
 
 // End of a sweep on all 32 lanes of the warp that completed the lattice's
@@ -1113,20 +1209,21 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // at most 31 wait between tiles, and a tile adds at most 64.
 constexpr uint32_t kLeaderRing = 128;
 
-// Tiles are taken in grid-stride order, `chunk` consecutive tiles per step: at
-// any moment the warps hold a window of about `chunk` tiles each, a few
+// Tiles are taken in grid-stride order, CHUNK consecutive tiles per step: at
+// any moment the warps hold a window of about CHUNK tiles each, a few
 // lattices of the batch, so that the random gathers of partners and their
 // neighbours stay in L2.  A warp adds its accepted moves and M_L change
 // once per lattice in a chunk.
-template <typename R, int MINB, bool LEADER, int NT = kBlock>
-__global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32_t ntiles, const R* __restrict__ cone,
-                                                             int colour, int sub, uint32_t chunk) {
+template <typename R, int MINB, int CHUNK, bool LEADER, int NT = kBlock>
+__global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32_t ntiles,
+                                                             const R* __restrict__ cone, int colour, int sub) {
     const int lane = int(threadIdx.x & 31);
-    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
-    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const uint32_t wpb = kIsF64<R> ? blockDim.x >> 5 : uint32_t(NT / 32);  // FP64: spread_warps
+    const uint32_t nwarps = gridDim.x * wpb;
+    const uint32_t w = blockIdx.x * wpb + (threadIdx.x >> 5);
     int l = 0;
-    for (uint32_t c0 = w * chunk; c0 < ntiles; c0 += nwarps * chunk) {
-        const uint32_t c1 = min(c0 + chunk, ntiles);
+    for (uint32_t c0 = w * CHUNK; c0 < ntiles; c0 += nwarps * CHUNK) {
+        const uint32_t c1 = min(c0 + uint32_t(CHUNK), ntiles);
         for (uint32_t tile = c0; tile < c1;) {
             while (__ldg(&g.start[l + 1]) <= tile) ++l;
             const uint32_t t0 = __ldg(&g.start[l]);
@@ -1275,7 +1372,7 @@ __global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32
 // spins summed in the order -x, +x, -y, +y, -z, +z, as neighbour_sum4 does,
 // written as (h_x, h_y, h_z, 0).  The other colour does not change during
 // the pass, so the field holds for all of it.  Tiles go to the warps
-// `chunk` at a time in grid-stride order, so that the warps in flight cover
+// CHUNK at a time in grid-stride order, so that the warps in flight cover
 // one compact window of the batch and the +-z planes a tile reads are still
 // in L2 when the tiles two planes on read them again (with one contiguous
 // run per warp those reads were a large part of the launch apart, and every
@@ -1314,15 +1411,16 @@ __device__ __forceinline__ void field_tile_periodic(const LatParams& p, const Sp
     }
 }
 
-template <typename R, int V>
-__global__ void __launch_bounds__(kBlock) pair_field_kernel(GroupArgs g, uint32_t ntiles, int colour, uint32_t chunk) {
-    const uint32_t nwarps = gridDim.x * (blockDim.x >> 5);
-    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+template <typename R, int V, int CHUNK>
+__global__ void __launch_bounds__(kBlock) pair_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
+    const uint32_t wpb = kIsF64<R> ? blockDim.x >> 5 : uint32_t(kBlock / 32);  // FP64: spread_warps
+    const uint32_t nwarps = gridDim.x * wpb;
+    const uint32_t w = blockIdx.x * wpb + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31u;
     const int other = colour ^ 1;
     int l = 0;
-    for (uint32_t c0 = w * chunk; c0 < ntiles; c0 += nwarps * chunk) {
-        const uint32_t c1 = min(c0 + chunk, ntiles);
+    for (uint32_t c0 = w * CHUNK; c0 < ntiles; c0 += nwarps * CHUNK) {
+        const uint32_t c1 = min(c0 + uint32_t(CHUNK), ntiles);
         for (uint32_t tile = c0; tile < c1;) {
             while (__ldg(&g.start[l + 1]) <= tile) ++l;  // tiles only move forward
             const uint32_t t0 = __ldg(&g.start[l]);

@@ -204,15 +204,46 @@ bool wave_desc(const mc_desc* d) {
 
 // Lattices whose sweeps may run held in shared memory (resident_pass.cuh):
 // FP32 simple cubic, every axis periodic, no film tables, rows of 64 sites
-// per colour (Lx = 128), not a slab, the automatic or resident kernel path;
-// whether its rows fit is decided on the device (KernelSet::resident_plan).
+// per colour (Lx = 128), not a slab, and either the resident kernel path or
+// the automatic one and kResAutoSpins spins; whether its rows fit is decided
+// on the device (KernelSet::resident_plan).  Below that size the brick sweeps
+// (brick_desc) are faster, their exchange between blocks being shorter: us a
+// sweep resident / brick 10.3 / 5.9 for 128 x 64 x 64, 15.9 / 17.5 for 128^3.
+constexpr uint64_t kResAutoSpins = 3ull << 19;
+
 bool resident_desc(const mc_desc* d, bool slab) {
     if (slab || d->precision != MC_FP32 || d->lattice != MC_SC) return false;
     if (d->kernel_path != MC_PATH_AUTO && d->kernel_path != MC_PATH_RESIDENT) return false;
     if (d->bond_mask || d->grain_id) return false;
     for (int a = 0; a < 3; ++a)
         if (d->boundary[a] != MC_PERIODIC) return false;
+    if (d->kernel_path == MC_PATH_AUTO && uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] < kResAutoSpins) return false;
     return d->dims[0] == 2 * kResLh;
+}
+
+// Lattices whose sweeps may run as brick launches (brick_pass.cuh): FP32
+// simple cubic without film tables, not a slab, the automatic or resident
+// kernel path, at most kBrickMaxSpins spins (whether its rows fit is decided
+// on the device, brick_plan); 128-wide periodic lattices take resident_pass.cuh.
+constexpr uint64_t kBrickMaxSpins = 3000000;
+
+bool brick_desc(const mc_desc* d, bool slab) {
+    if (slab || d->precision != MC_FP32 || d->lattice != MC_SC || resident_desc(d, slab)) return false;
+    if (d->kernel_path != MC_PATH_AUTO && d->kernel_path != MC_PATH_RESIDENT) return false;
+    if (d->bond_mask || d->grain_id) return false;
+    return uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] <= kBrickMaxSpins;
+}
+
+// Device memory of the brick sweeps of such a lattice, allocated by its first
+// brick launch (brick_memory): kept out of the lattice's own allocation, which
+// it would half as large again; the 80 lattices of a constrained batch, spread
+// over so much more memory, swept 2% slower.
+constexpr size_t kBrickRecordBytes = size_t(kBrickMaxMeasured) * kBrickRecord * sizeof(long long);
+
+size_t brick_bytes(const mc_desc* d) {
+    if (!brick_desc(d, false)) return 0;
+    const uint64_t stride = (uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] / 2 + 63) / 64 * 64;
+    return align256(sizeof(BrickCtl)) + align256(kBrickRecordBytes) + size_t(32 * stride);
 }
 
 size_t lattice_bytes(const mc_desc* d, bool slab) {
@@ -535,6 +566,18 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
             delete rp;
         }
     }
+    if (brick_desc(d, slab != nullptr)) {
+        BrickArgs b{};
+        if (brick_plan(p, &b)) {
+            b.lat = h->d_lat;
+            b.key0 = p.key0;
+            b.key1 = p.key1;
+            b.bytes = brick_bytes(d);
+            const char* inj = std::getenv("MC_RESIDENT_INJECT_TIMEOUT");  // as for the resident sweeps
+            b.inject = inj && inj[0] == '1' ? 1 : 0;
+            h->brick = new BrickArgs(b);
+        }
+    }
     if (size_t(cur - static_cast<char*>(h->d_base)) > h->bytes) {
         cudaFree(h->d_base);
         if (h->owned_stream) cudaStreamDestroy(h->owned_stream);
@@ -637,6 +680,8 @@ LaunchSet single_launch_set(mc_lattice* h) {
     }
     ls.sample_level = h->hp.sample_torque ? 2 : 1;
     ls.shape = h->shape;
+    ls.brick = h->brick;
+    ls.brick_lh = uint32_t(h->hp.Lh);
     if (h->hp.nsub > 1) {
         ls.xtal = h->d_lat;
         ls.nsub = h->hp.nsub;
@@ -801,6 +846,32 @@ int upload_wave_plan(const WavePlan& pl, const std::vector<LatDev*>& dev_lats, c
     return MC_OK;
 }
 
+// The device memory of a lattice's brick sweeps, on first use; false when it
+// cannot be had (none left, or the stream is being captured), and the sweeps
+// then run as launches.
+static bool brick_memory(BrickArgs* b, cudaStream_t s) {
+    if (b->ctl) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    char* m = nullptr;
+    if (cudaMalloc(reinterpret_cast<void**>(&m), b->bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    // zero, so that no packet of uninitialised memory carries a tag; epoch 1
+    const uint32_t first = 1;
+    BrickCtl* ctl = reinterpret_cast<BrickCtl*>(m);
+    if (cudaMemsetAsync(m, 0, b->bytes, s) != cudaSuccess ||
+        cudaMemcpyAsync(&ctl->epoch, &first, sizeof first, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+        cudaFree(m);
+        return false;
+    }
+    b->ctl = ctl;
+    b->record = reinterpret_cast<long long*>(m + align256(sizeof(BrickCtl)));
+    b->packets = m + align256(sizeof(BrickCtl)) + align256(kBrickRecordBytes);
+    return true;
+}
+
 // Enqueue n sweeps of the lattices of a launch set; with events != nullptr
 // every colour pass or pair pass is bracketed by a pair of events.
 int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, int n, int measure, bool constrained,
@@ -830,6 +901,16 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 });
             }
         if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
+        return MC_OK;
+    }
+    if (!constrained && ls.brick && n >= kResMinSweeps && brick_memory(ls.brick, s)) {
+        cudaError_t e = cudaSuccess;
+        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
+        for (int done = 0; done < n && e == cudaSuccess; done += most)
+            timed_kind(kTimedResident, [&] {
+                e = brick_sweeps(*ls.brick, ls.brick_lh, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
+            });
+        if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
         return MC_OK;
     }
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
@@ -950,7 +1031,7 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
                bool constrained, cudaStream_t s) {
     const KernelSet& k = kernel_set(precision);
     // resident sweeps run many to a launch: nothing to capture
-    if (!constrained && ls.n_res && n >= kResMinSweeps)
+    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && brick_memory(ls.brick, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
     const int reps = n / kGraphSweeps;
     if (reps > 0) {
@@ -1075,6 +1156,7 @@ MC_API int mc_destroy(mc_handle h) {
     cudaFree(h->d_base);
     if (h->d_aos) cudaFree(h->d_aos);
     if (h->d_wave) cudaFree(h->d_wave);
+    if (h->brick && h->brick->ctl) cudaFree(h->brick->ctl);
     if (h->owned_stream) cudaStreamDestroy(h->owned_stream);
     delete h;
     return MC_OK;

@@ -53,6 +53,7 @@ struct mc_lattice {
     mcgb::WaveArgs wave_args = {};
     uint32_t wave_nblocks = 0;
     mcgb::ResidentPlan* res = nullptr;  // resident sweeps of the lattice alone (null: none)
+    mcgb::BrickArgs* brick = nullptr;   // brick sweeps of the lattice alone (null: none)
     mcgb::SweepGraphs graphs;     // sweeps of the lattice alone
     mcgb::LaunchShape shape;      // autotuned launch shapes of the lattice alone
     const void* cone = nullptr;   // c(theta) table of the precision
@@ -65,7 +66,10 @@ struct mc_lattice {
     mc_lattice() = default;
     mc_lattice(const mc_lattice&) = delete;
     mc_lattice& operator=(const mc_lattice&) = delete;
-    ~mc_lattice() { delete res; }
+    ~mc_lattice() {
+        delete res;
+        delete brick;
+    }
 };
 
 namespace mcgb {
@@ -84,6 +88,7 @@ int colour_kernel(const LatParams& p, bool film, int path);
 size_t lattice_bytes(const mc_desc* d, bool slab = false);
 int upload_params(mc_lattice* h);
 size_t aos_bytes(const mc_desc* d);
+size_t brick_bytes(const mc_desc* d);
 int ensure_aos(mc_lattice* h);
 void constraint_frame(double theta_deg, double phi_deg, double R[9]);
 const KernelSet& kernel_set(int precision);
@@ -107,6 +112,7 @@ struct WavePlan {
 };
 bool wave_desc(const mc_desc* d);
 bool resident_desc(const mc_desc* d, bool slab);
+bool brick_desc(const mc_desc* d, bool slab);
 WavePlan plan_wave(const std::vector<const LatParams*>& lats, uint32_t blocks);
 int upload_wave_plan(const WavePlan& pl, const std::vector<LatDev*>& dev_lats, cudaStream_t s, void** d_mem,
                      WaveArgs* out);

@@ -167,6 +167,17 @@ void mc_server::loop() {
                 int rc = create_lattice(&desc, &j->h);
                 release_tables(j);
                 if (rc) { j->h = nullptr; j->t_finish = now(); j->status = rc; continue; }
+                if (j->h->brick) {
+                    // the optional memory of brick sweeps (a lattice swept alone),
+                    // only while it leaves half of the budget to other jobs
+                    const size_t extra = j->job.kind == MC_JOB_SWEEP ? brick_bytes(&desc) : 0;
+                    if (extra && used + j->bytes + extra <= budget / 2) {
+                        j->bytes += extra;
+                    } else {
+                        delete j->h->brick;
+                        j->h->brick = nullptr;
+                    }
+                }
                 used += j->bytes;
                 j->t_admit = now();
                 j->measuring = j->job.n_equilibrate <= 0;
