@@ -182,28 +182,6 @@ __device__ __forceinline__ bool brick_neighbours(const float* oth, const float4*
     }
 }
 
-// The move of the general kernel on a lane's two sites (colour_pass_kernel,
-// V = 2): the same functions in the same order.
-__device__ __forceinline__ unsigned scalar_move(const Par<float>& par, float c, uint4 w, const V3<float> S[2],
-                                                const V3<float> h[2], V3<float> e, const bool mov[2], V3<float> Sf[2]) {
-    float P[2], sd[2], u1[2], u2[2];
-    direct_draw_two(w, P, sd, u1, u2);
-    unsigned n = 0;
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-        Sf[v] = S[v];
-        if (mov[v]) {
-            const V3<float> Sn = cap_point_direct(S[v], c, sd[v], u1[v], u2[v]);
-            const float dE = delta_e(par, S[v], Sn, h[v], e);
-            if (metropolis(dE, par, P[v])) {
-                Sf[v] = Sn;
-                ++n;
-            }
-        }
-    }
-    return n;
-}
-
 // LAW 0: packed pairs (row kernels), 1: the general kernel's scalar law;
 // FACES: any boundaries (0: all periodic); ODD: rows of odd Lh (LAW 1);
 // MEASURE as in the row kernel.
@@ -527,7 +505,8 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                 } else {
                     unpack(S, Sv);
                     unpack(h, hv);
-                    const V3<float> ax{par.e[0], par.e[1], par.e[2]};
+                    const V3<float> ax[2] = {V3<float>{par.e[0], par.e[1], par.e[2]},
+                                             V3<float>{par.e[0], par.e[1], par.e[2]}};
                     n = scalar_move(par, cval, w, Sv, hv, ax, mov, Sn);
                     Sf = pack(Sn);
                 }
@@ -564,22 +543,11 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                                 const P3 ea{p2(par.e[0]), p2(par.e[1]), p2(par.e[2])};
                                 pair_tile_parts<MEASURE, NS>(par, Sf, h, ea, O, ea, lf);
                             } else {
-                                Sums<float> sums;
-#pragma unroll
-                                for (int i = 0; i < kNumSums; ++i) sums.v[i] = 0.0f;
-                                const bool nu = par.Ku != 0.0f, nc = par.Kc != 0.0f;
-                                const V3<float> ax{par.e[0], par.e[1], par.e[2]};
+                                const V3<float> ax[2] = {V3<float>{par.e[0], par.e[1], par.e[2]},
+                                                         V3<float>{par.e[0], par.e[1], par.e[2]}};
                                 V3<float> Ov[2];
                                 unpack(O, Ov);
-#pragma unroll
-                                for (int v = 0; v < 2; ++v) {
-                                    if (v == 1 && !two) continue;
-                                    add_site<float, MEASURE>(sums, Sn[v], ax, nu, nc);
-                                    sums.v[kSumEx] += Sn[v].x * hv[v].x + Sn[v].y * hv[v].y + Sn[v].z * hv[v].z;
-                                    add_site<float, MEASURE>(sums, Ov[v], ax, nu, nc);
-                                }
-#pragma unroll
-                                for (int i = 0; i < NS; ++i) lf[i] += __float2int_rn(sums.v[i] * float(kFixScaleF32));
+                                scalar_tile_parts<MEASURE, NS>(par, Sn, hv, ax, Ov, ax, two ? 2 : 1, lf);
                             }
                         }
                     }

@@ -37,12 +37,13 @@ struct KernelSet {
     void (*colour_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure,
                         cudaStream_t s);
     // FP32 colour pass over lattices in the row layout (adjacent site pairs
-    // per lane); gen = 0: all axes periodic, no film tables; gen = 1: any
-    // boundaries and film tables.  Null in the FP64 set.  After an
+    // per lane; law = 0) or outside it with rows of even Lh (law = 1: the
+    // general kernel's arithmetic); gen = 0: all axes periodic, no film tables;
+    // gen = 1: any boundaries and film tables.  Null in the FP64 set.  After an
     // unmeasured black pass (colour 1) it also launches the close of the
     // lattices' sweeps (row_close_kernel).  Returns the status of the
     // launches (made with programmatic serialisation).
-    cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure,
+    cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law,
                             int gen, int shape, cudaStream_t s);
     // Table A2 pair pass over sub-set (sub, colour) (sub = 0 for simple cubic
     // lattices); leader != 0 takes the pairs in site order
@@ -120,9 +121,10 @@ struct LaunchSet {
     GroupArgs all, pairs, pairs_lead;
     uint32_t nt_all = 0, nt_pairs = 0, nt_pairs_lead = 0;  // pair tiles: pair order, site order
     // colour passes: row kernel, row kernel with boundaries and films, the
-    // general kernel (tiles)
-    GroupArgs row, rowx, rest;
-    uint32_t nt_row = 0, nt_rowx = 0, nt_rest = 0;
+    // same two for rows of even Lh outside the row layout, the general kernel
+    // (tiles)
+    GroupArgs row, rowx, even, evenx, rest;
+    uint32_t nt_row = 0, nt_rowx = 0, nt_even = 0, nt_evenx = 0, nt_rest = 0;
     // wavefront lattices (LatParams::wave): their work-unit plan (nb_wave
     // blocks; 0 = none), and the row-kernel list without them, which runs
     // beside a wavefront launch (row above keeps them, for sweeps that run

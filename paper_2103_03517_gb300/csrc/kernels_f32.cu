@@ -40,9 +40,9 @@ constexpr int V = kSitesPerThreadF32;
 
 #include "launchers_common.cuh"
 
-template <int B, int MEASURE, int GEN>
+template <int B, int MEASURE, int GEN, int LAW>
 cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN>);
+    static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN, 1, LAW>);
     // programmatic serialisation: the pass starts its blocks while the
     // previous launch drains and waits inside the kernel (griddepcontrol)
     cudaLaunchConfig_t cfg = {};
@@ -55,7 +55,7 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN>, g, ntiles, cone, colour);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN, 1, LAW>, g, ntiles, cone, colour);
     if (e != cudaSuccess || colour != 1 || MEASURE > 0) return e;  // the unmeasured sweep's end
     cudaLaunchConfig_t cc = cfg;
     cc.gridDim = dim3(uint32_t(g.n));
@@ -64,24 +64,28 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
 }
 
 // launch shape 0: the default blocks per SM of the instance; 1: the other candidate
-template <int GEN, int B0, int B1>
+template <int GEN, int B0, int B1, int LAW>
 cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape,
                        cudaStream_t s) {
     if (shape == 1) {
-        if (measure >= 2) return row_pass_t<B1, 2, GEN>(g, ntiles, c, colour, s);
-        if (measure == 1) return row_pass_t<B1, 1, GEN>(g, ntiles, c, colour, s);
-        return row_pass_t<B1, 0, GEN>(g, ntiles, c, colour, s);
+        if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, s);
+        if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, s);
+        return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, s);
     }
-    if (measure >= 2) return row_pass_t<B0, 2, GEN>(g, ntiles, c, colour, s);
-    if (measure == 1) return row_pass_t<B0, 1, GEN>(g, ntiles, c, colour, s);
-    return row_pass_t<B0, 0, GEN>(g, ntiles, c, colour, s);
+    if (measure >= 2) return row_pass_t<B0, 2, GEN, LAW>(g, ntiles, c, colour, s);
+    if (measure == 1) return row_pass_t<B0, 1, GEN, LAW>(g, ntiles, c, colour, s);
+    return row_pass_t<B0, 0, GEN, LAW>(g, ntiles, c, colour, s);
 }
 
-cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int gen,
+cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law, int gen,
                      int shape, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
-    if (gen) return row_pass_g<1, MINB_GEN, MINB_GEN + 1>(g, ntiles, c, colour, measure, shape, s);
-    return row_pass_g<0, MINB, MINB - 1>(g, ntiles, c, colour, measure, shape, s);
+    if (law) {
+        if (gen) return row_pass_g<1, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, s);
+        return row_pass_g<0, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, s);
+    }
+    if (gen) return row_pass_g<1, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, s);
+    return row_pass_g<0, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, s);
 }
 
 // the all-periodic instance samples red sites first and stores their field

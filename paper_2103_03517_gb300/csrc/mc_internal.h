@@ -65,7 +65,7 @@ inline FastDiv make_fastdiv(uint32_t d) {
     return f;
 }
 
-enum { kColourGeneral = 0, kColourRow = 1, kColourRowGen = 2 };
+enum { kColourGeneral = 0, kColourRow = 1, kColourRowGen = 2, kColourEven = 3, kColourEvenGen = 4 };
 
 // One neighbour entry of a bcc / fcc / hcp sub-lattice: the neighbour's
 // sub-lattice, its cell offset and its coupling (J1 or J2), with what the
@@ -106,8 +106,10 @@ struct LatParams {
     int xnb_n[kXtalMaxSub]; // bcc / fcc: neighbour entries per sub-lattice
     const void* xnb;        // bcc / fcc: [kXtalMaxSub][kXtalMaxNb] XtalNb, or null
     int colour_kernel;      // colour-pass kernel: kColourGeneral, kColourRow (FP32 row
-                            // layout, all axes periodic, no film tables) or
-                            // kColourRowGen (FP32 row layout, any boundaries and films)
+                            // layout, all axes periodic, no film tables),
+                            // kColourRowGen (FP32 row layout, any boundaries and films);
+                            // kColourEven, kColourEvenGen: the same two for FP32
+                            // lattices outside the row layout with even Lh
     void* spins;
     void* spins_alt;        // wavefront lattices (wave != 0): the second spin buffer
                             // a fused sweep writes (same layout), else null

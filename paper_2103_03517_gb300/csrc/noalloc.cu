@@ -133,6 +133,9 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     if (p.colour_kernel == kColourRow) {  // every axis periodic: the row kernel or the general one
         ls.row = ls.all;
         ls.nt_row = ls.nt_all;
+    } else if (p.colour_kernel == kColourEven) {
+        ls.even = ls.all;
+        ls.nt_even = ls.nt_all;
     } else {
         ls.rest = ls.all;
         ls.nt_rest = ls.nt_all;

@@ -245,4 +245,55 @@ __device__ __forceinline__ long long pair_parts_flush(int lf[NS], int lane) {
     return mine;
 }
 
+// ---------------------------------------- the general kernel's law, in pairs
+// Lattices outside the row layout move by the scalar functions of pass_impl
+// .cuh, whose last bits differ from the packed ones.  These two do the same
+// on a lane's pair for the kernels that take such lattices in pairs (brick
+// sweeps, the row kernel's LAW 1), so that all of them give the same chain.
+//
+// The move of the general kernel on a lane's two sites (colour_pass_kernel,
+// V = 2): the same functions in the same order.
+__device__ __forceinline__ unsigned scalar_move(const Par<float>& par, float c, uint4 w, const V3<float> S[2],
+                                                const V3<float> h[2], const V3<float> e[2],
+                                                const bool mov[2], V3<float> Sf[2]) {
+    float P[2], sd[2], u1[2], u2[2];
+    direct_draw_two(w, P, sd, u1, u2);
+    unsigned n = 0;
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        Sf[v] = S[v];
+        if (mov[v]) {
+            const V3<float> Sn = cap_point_direct(S[v], c, sd[v], u1[v], u2[v]);
+            const float dE = delta_e(par, S[v], Sn, h[v], e[v]);
+            if (metropolis(dE, par, P[v])) {
+                Sf[v] = Sn;
+                ++n;
+            }
+        }
+    }
+    return n;
+}
+
+// The sample parts of a lane's n sites (own sites Sf with fields h and axes e,
+// the other colour's sites O with axes eo), as in colour_pass_kernel, added
+// into the lane's accumulators as pair_tile_parts does.
+template <int MEASURE, int NS>
+__device__ __forceinline__ void scalar_tile_parts(const Par<float>& par, const V3<float> Sf[2], const V3<float> h[2],
+                                                  const V3<float> e[2], const V3<float> O[2], const V3<float> eo[2],
+                                                  int n, int lf[NS]) {
+    Sums<float> sums;
+#pragma unroll
+    for (int i = 0; i < kNumSums; ++i) sums.v[i] = 0.0f;
+    const bool nu = par.Ku != 0.0f, nc = par.Kc != 0.0f;
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+        if (v >= n) continue;
+        add_site<float, MEASURE>(sums, Sf[v], e[v], nu, nc);
+        sums.v[kSumEx] += Sf[v].x * h[v].x + Sf[v].y * h[v].y + Sf[v].z * h[v].z;
+        add_site<float, MEASURE>(sums, O[v], eo[v], nu, nc);
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) lf[i] += __float2int_rn(sums.v[i] * float(kFixScaleF32));
+}
+
 }  // namespace mcgb

@@ -20,6 +20,15 @@
 // neighbour sum keeps the order -x, +x, -y, +y, -z, +z.  In the GEN instance
 // every neighbour enters with a factor 1, -1 (across an anti-periodic face)
 // or 0 (absent: open face or missing bond), an exact product.
+//
+// LAW 1 takes the lattices outside the row layout whose rows hold an even
+// number of sites per colour (96^3, 160^3, ...): the same pairs, loads and
+// neighbour sums, with the fourth x neighbour loaded on its own (rows do not
+// line up with lanes) and a last tile that may be part full; the moves and
+// samples are those of the general kernel (scalar_move), whose chain it gives
+// bit for bit.  In the general kernel each of a lane's two sites found its own
+// neighbours and loaded them one float at a time: 750 warp instructions per 64
+// sites, 46% of them issued per cycle, 47 us a pass of 160^3.
 #pragma once
 #include "pair_math.cuh"
 
@@ -36,14 +45,15 @@ __device__ __forceinline__ float face_factor(int bc) { return bc == 0 ? 1.0f : (
 // packed (site 0 in .x, site 1 in .y, as loaded); returns the lattice index
 // of the pair's first site (its parity is the row's x offset).  GEN:
 // mov[v] = site v is not on a pinned plane.
-template <int GEN>
+template <int GEN, int LAW = 0>
 __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const float* s, int colour, uint32_t q0,
                                                   int lane, P3& S, P3& h, P3& O, bool mov[2]) {
     const uint32_t stride = p.stride;
     const float* own = s + size_t(3 * colour) * stride;
     const float* oth = s + size_t(3 * (colour ^ 1)) * stride;
     const uint32_t Lh = uint32_t(p.Lh), Ly = uint32_t(p.Ly), Lz = uint32_t(p.Lz), plane = Lh * Ly;
-    const uint32_t q = q0 + 2u * uint32_t(lane);
+    uint32_t q = q0 + 2u * uint32_t(lane);
+    if (LAW == 1) q = min(q, p.Nc - 2u);  // lanes past the end repeat the last pair
     const uint32_t row = fast_div(q, p.div_lh);
     const uint32_t k = q - row * Lh;
     const uint32_t z = fast_div(row, p.div_ly);
@@ -58,23 +68,30 @@ __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const floa
 #pragma unroll
         for (int a = 0; a < 3; ++a) v[3 * j + a] = ld2(base + size_t(a) * stride, qn[j]);
     }
-    const int G = p.row_lanes;
-    const int gbase = lane & ~(G - 1);
-    const int left = gbase | ((lane - 1) & (G - 1));
-    const int right = gbase | ((lane + 1) & (G - 1));
-    // other colour at k - 1 (left lane's second) and k + 2 (right lane's first)
-    V3<float> lft{__shfl_sync(0xffffffffu, v[3].y, left), __shfl_sync(0xffffffffu, v[4].y, left),
-                  __shfl_sync(0xffffffffu, v[5].y, left)};
-    V3<float> rgt{__shfl_sync(0xffffffffu, v[3].x, right), __shfl_sync(0xffffffffu, v[4].x, right),
-                  __shfl_sync(0xffffffffu, v[5].x, right)};
-    if (Lh > 64u) {  // ends of a 64-site segment of a longer row
-        if (lane == 0) {
-            const uint32_t qe = k == 0 ? q + Lh - 1 : q - 1;
-            lft = V3<float>{oth[qe], oth[stride + qe], oth[2 * size_t(stride) + qe]};
-        }
-        if (lane == 31) {
-            const uint32_t qe = k + 2 == Lh ? q + 2 - Lh : q + 2;
-            rgt = V3<float>{oth[qe], oth[stride + qe], oth[2 * size_t(stride) + qe]};
+    V3<float> lft, rgt;
+    if constexpr (LAW == 1) {
+        // only one of the two is an x neighbour of the pair
+        const uint32_t qe = xoff ? (k + 2 == Lh ? q - k : q + 2) : (k == 0 ? q + Lh - 1 : q - 1);
+        lft = rgt = V3<float>{oth[qe], oth[stride + qe], oth[2 * size_t(stride) + qe]};
+    } else {
+        const int G = p.row_lanes;
+        const int gbase = lane & ~(G - 1);
+        const int left = gbase | ((lane - 1) & (G - 1));
+        const int right = gbase | ((lane + 1) & (G - 1));
+        // other colour at k - 1 (left lane's second) and k + 2 (right lane's first)
+        lft = V3<float>{__shfl_sync(0xffffffffu, v[3].y, left), __shfl_sync(0xffffffffu, v[4].y, left),
+                        __shfl_sync(0xffffffffu, v[5].y, left)};
+        rgt = V3<float>{__shfl_sync(0xffffffffu, v[3].x, right), __shfl_sync(0xffffffffu, v[4].x, right),
+                        __shfl_sync(0xffffffffu, v[5].x, right)};
+        if (Lh > 64u) {  // ends of a 64-site segment of a longer row
+            if (lane == 0) {
+                const uint32_t qe = k == 0 ? q + Lh - 1 : q - 1;
+                lft = V3<float>{oth[qe], oth[stride + qe], oth[2 * size_t(stride) + qe]};
+            }
+            if (lane == 31) {
+                const uint32_t qe = k + 2 == Lh ? q + 2 - Lh : q + 2;
+                rgt = V3<float>{oth[qe], oth[stride + qe], oth[2 * size_t(stride) + qe]};
+            }
         }
     }
     // the other colour at the pair's own indices: one x neighbour of each
@@ -140,7 +157,7 @@ __device__ __forceinline__ V3<float> grain_axis(const LatParams& p, int colour, 
 // the red sites' neighbour sums as the field of the next sweep's red pair
 // pass: the same terms in the same order as pair_field_kernel's (the -x, +x
 // pair commutes), so the same bits.
-template <int MINB, int MEASURE, int GEN, int MOVE = 1>
+template <int MINB, int MEASURE, int GEN, int MOVE = 1, int LAW = 0>
 __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uint32_t ntiles,
                                                                 const float* __restrict__ cone, int colour) {
     constexpr int NS = MEASURE >= 2 ? kNumSums : kSumTux;  // sums sampled
@@ -188,16 +205,18 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
             const uint32_t q0 = (tile - t0) * 64u;
             P3 S, h, O;
             bool mov[2];
-            const uint32_t site0 = row_pair_sums<GEN>(p, s, colour, q0, lane, S, h, O, mov);
+            const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, S, h, O, mov);
+            const bool valid = LAW == 0 || q0 + 2u * uint32_t(lane) < p.Nc;
             P3 e, eo;  // per-site easy axes (films with grain axes)
             const bool grains = GEN != 0 && p.grain;
             if constexpr (GEN != 0) {
                 if (grains) {
                     V3<float> a[2], b[2];
+                    const uint32_t qa = LAW == 1 ? min(q0 + 2u * uint32_t(lane), p.Nc - 2u) : q0 + 2u * uint32_t(lane);
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
-                        a[v] = grain_axis(p, colour, q0 + 2u * uint32_t(lane) + v);
-                        b[v] = grain_axis(p, colour ^ 1, q0 + 2u * uint32_t(lane) + v);
+                        a[v] = grain_axis(p, colour, qa + v);
+                        b[v] = grain_axis(p, colour ^ 1, qa + v);
                     }
                     e = pack(a);
                     eo = pack(b);
@@ -221,7 +240,19 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
             if constexpr (MOVE != 0) {
                 const uint4 w = MEASURE == 0 ? philox_smem(make_uint4(key_site, sweep, key_tag, 0u), rk)
                                              : philox(make_uint4(key_site, sweep, key_tag, 0u), p.key0, p.key1);
-                const unsigned n = pair_move(par, c, w, S, h, mov, grains ? &e : nullptr, Sf);
+                unsigned n;
+                if constexpr (LAW == 0) {
+                    n = pair_move(par, c, w, S, h, mov, grains ? &e : nullptr, Sf);
+                } else {
+                    V3<float> Sv[2], hv[2], ev[2], Sn[2];
+                    unpack(S, Sv);
+                    unpack(h, hv);
+                    unpack(e, ev);
+                    mov[0] = mov[0] && valid;
+                    mov[1] = mov[1] && valid;
+                    n = scalar_move(par, c, w, Sv, hv, ev, mov, Sn);
+                    Sf = pack(Sn);
+                }
                 nacc += n;
                 any = n != 0;
             }
@@ -239,7 +270,17 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
                 *reinterpret_cast<float2*>(own + 2 * size_t(p.stride)) = Sf.z;
             }
             if constexpr (MEASURE > 0) {
-                if (sampled) pair_tile_parts<MEASURE, NS>(par, Sf, h, e, O, eo, lf);
+                if constexpr (LAW == 0) {
+                    if (sampled) pair_tile_parts<MEASURE, NS>(par, Sf, h, e, O, eo, lf);
+                } else if (valid) {
+                    V3<float> Sv[2], hv[2], ev[2], Ov[2], eov[2];
+                    unpack(Sf, Sv);
+                    unpack(h, hv);
+                    unpack(e, ev);
+                    unpack(O, Ov);
+                    unpack(eo, eov);
+                    scalar_tile_parts<MEASURE, NS>(par, Sv, hv, ev, Ov, eov, 2, lf);
+                }
                 if (++nparts == uint32_t(kPartTiles)) {
                     fix += pair_parts_flush<NS>(lf, lane);
                     nparts = 0;

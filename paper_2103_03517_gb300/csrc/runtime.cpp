@@ -125,8 +125,11 @@ int row_fast(const LatParams& p, bool film) {
 
 // Colour-pass kernel of a lattice (LatParams::colour_kernel).
 int colour_kernel(const LatParams& p, bool film, int path) {
-    if (p.precision != MC_FP32 || path == MC_PATH_GENERAL || !row_layout(p)) return kColourGeneral;
-    return row_fast(p, film) ? kColourRow : kColourRowGen;
+    if (p.precision != MC_FP32 || path == MC_PATH_GENERAL) return kColourGeneral;
+    if (row_layout(p)) return row_fast(p, film) ? kColourRow : kColourRowGen;
+    if (p.Lh % 2) return kColourGeneral;  // a lane's pair may lie in two rows
+    return !film && p.bc[0] == MC_PERIODIC && p.bc[1] == MC_PERIODIC && p.bc[2] == MC_PERIODIC ? kColourEven
+                                                                                               : kColourEvenGen;
 }
 
 // ------------------------------------------------------------- lattices
@@ -703,6 +706,12 @@ LaunchSet single_launch_set(mc_lattice* h) {
     } else if (h->hp.colour_kernel == kColourRowGen) {
         ls.rowx = ls.all;
         ls.nt_rowx = ls.nt_all;
+    } else if (h->hp.colour_kernel == kColourEven) {
+        ls.even = ls.all;
+        ls.nt_even = ls.nt_all;
+    } else if (h->hp.colour_kernel == kColourEvenGen) {
+        ls.evenx = ls.all;
+        ls.nt_evenx = ls.nt_all;
     } else {
         ls.rest = ls.all;
         ls.nt_rest = ls.nt_all;
@@ -916,11 +925,17 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
     auto colour_pass = [&](int colour, int meas) {
         if (ls.nt_row) {
-            const cudaError_t e = k.row_pass(ls.row, ls.nt_row, cone, colour, meas, 0, ls.shape.row, s);
+            const cudaError_t e = k.row_pass(ls.row, ls.nt_row, cone, colour, meas, 0, 0, ls.shape.row, s);
             if (launch_err == cudaSuccess) launch_err = e;
         }
         if (ls.nt_rowx) {
-            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 1, ls.shape.row, s);
+            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 0, 1, ls.shape.row, s);
+            if (launch_err == cudaSuccess) launch_err = e;
+        }
+        for (int gen = 0; gen < 2; ++gen) {
+            const uint32_t nt = gen ? ls.nt_evenx : ls.nt_even;
+            if (!nt) continue;
+            const cudaError_t e = k.row_pass(gen ? ls.evenx : ls.even, nt, cone, colour, meas, 1, gen, ls.shape.row, s);
             if (launch_err == cudaSuccess) launch_err = e;
         }
         if (ls.nt_rest) k.colour_pass(ls.rest, ls.nt_rest, cone, colour, meas, s);
@@ -963,16 +978,22 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     // wavefront lattices, the boundary and general lists
     auto rest_pass = [&](int colour, int meas) {
         if (ls.nt_row_rest) {
-            const cudaError_t e = k.row_pass(ls.row_rest, ls.nt_row_rest, cone, colour, meas, 0, ls.shape.row, s);
+            const cudaError_t e = k.row_pass(ls.row_rest, ls.nt_row_rest, cone, colour, meas, 0, 0, ls.shape.row, s);
             if (launch_err == cudaSuccess) launch_err = e;
         }
         if (ls.nt_rowx) {
-            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 1, ls.shape.row, s);
+            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 0, 1, ls.shape.row, s);
+            if (launch_err == cudaSuccess) launch_err = e;
+        }
+        for (int gen = 0; gen < 2; ++gen) {
+            const uint32_t nt = gen ? ls.nt_evenx : ls.nt_even;
+            if (!nt) continue;
+            const cudaError_t e = k.row_pass(gen ? ls.evenx : ls.even, nt, cone, colour, meas, 1, gen, ls.shape.row, s);
             if (launch_err == cudaSuccess) launch_err = e;
         }
         if (ls.nt_rest) k.colour_pass(ls.rest, ls.nt_rest, cone, colour, meas, s);
     };
-    const bool rest_any = ls.nt_row_rest || ls.nt_rowx || ls.nt_rest;
+    const bool rest_any = ls.nt_row_rest || ls.nt_rowx || ls.nt_even || ls.nt_evenx || ls.nt_rest;
     bool red_field_ready = false;  // the next constrained sweep's red field is stored
     for (int i = 0; i < n; ++i) {
         // wavefront lattices sweep two at a time, spins -> spins_alt -> spins,
@@ -1014,7 +1035,9 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                     if (ls.nt_row) k.row_sample(ls.row, ls.nt_row, 0, s);
                     if (ls.nt_rowx) k.row_sample(ls.rowx, ls.nt_rowx, 1, s);
                     if (ls.nt_rest) k.measure(ls.rest, ls.nt_rest, s);
-                    red_field_ready = ls.nt_row && !ls.nt_rowx && !ls.nt_rest;
+                    if (ls.nt_even) k.measure(ls.even, ls.nt_even, s);
+                    if (ls.nt_evenx) k.measure(ls.evenx, ls.nt_evenx, s);
+                    red_field_ready = ls.nt_row && !ls.nt_rowx && !ls.nt_rest && !ls.nt_even && !ls.nt_evenx;
                 } else {
                     k.measure(ls.all, ls.nt_all, s);
                 }
