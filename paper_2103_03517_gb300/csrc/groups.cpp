@@ -77,9 +77,9 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
     // colour passes: one list per colour-pass kernel (LatParams::colour_kernel);
     // constrained pair passes: one list per pair order (LatParams::pair_leader);
     // each list with its tile starts, in launch order
-    // general, row, row with films, even rows, even rows with films; pairs in
-    // pair order, in site order; row lattices other than the wavefront ones
-    constexpr int kLists = 8;
+    // one per colour-pass kernel; pairs in pair order, in site order; row
+    // lattices other than the wavefront ones
+    constexpr int kPairs = kColourKinds, kRowRest = kColourKinds + 2, kLists = kColourKinds + 3;
     std::vector<LatDev*> sub[kLists];
     std::vector<uint32_t> st[kLists];
     for (int c = 0; c < kLists; ++c) st[c].assign(1, 0);
@@ -87,7 +87,7 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
     std::vector<LatDev*> wave_dev;
     for (int j = 0; j < n; ++j) {
         const LatParams& hp = lattices[order[j]]->hp;
-        const int c = hp.colour_kernel, q = 5 + (hp.pair_leader ? 1 : 0);
+        const int c = hp.colour_kernel, q = kPairs + (hp.pair_leader ? 1 : 0);
         sub[c].push_back(all[j]);
         st[c].push_back(st[c].back() + hp.nblocks_site);
         sub[q].push_back(all[j]);
@@ -96,8 +96,8 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
             wave_hp.push_back(&hp);
             wave_dev.push_back(all[j]);
         } else if (c == kColourRow) {
-            sub[7].push_back(all[j]);
-            st[7].push_back(st[7].back() + hp.nblocks_site);
+            sub[kRowRest].push_back(all[j]);
+            st[kRowRest].push_back(st[kRowRest].back() + hp.nblocks_site);
         }
     }
     cudaSetDevice(g->device);
@@ -115,10 +115,18 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
     std::copy(sa.begin(), sa.end(), reinterpret_cast<uint32_t*>(hb + o0));
     g->ls.all = GroupArgs{reinterpret_cast<LatDev**>(db), reinterpret_cast<uint32_t*>(db + o0), n};
     g->ls.nt_all = sa.back();
-    GroupArgs* lists[kLists] = {&g->ls.rest,  &g->ls.row,   &g->ls.rowx,       &g->ls.even,
-                                &g->ls.evenx, &g->ls.pairs, &g->ls.pairs_lead, &g->ls.row_rest};
-    uint32_t* counts[kLists] = {&g->ls.nt_rest,  &g->ls.nt_row,   &g->ls.nt_rowx,       &g->ls.nt_even,
-                                &g->ls.nt_evenx, &g->ls.nt_pairs, &g->ls.nt_pairs_lead, &g->ls.nt_row_rest};
+    GroupArgs* lists[kLists];
+    uint32_t* counts[kLists];
+    for (int c = 0; c < kColourKinds; ++c) {
+        lists[c] = &g->ls.col[c];
+        counts[c] = &g->ls.nt_col[c];
+    }
+    lists[kPairs] = &g->ls.pairs;
+    counts[kPairs] = &g->ls.nt_pairs;
+    lists[kPairs + 1] = &g->ls.pairs_lead;
+    counts[kPairs + 1] = &g->ls.nt_pairs_lead;
+    lists[kRowRest] = &g->ls.row_rest;
+    counts[kRowRest] = &g->ls.nt_row_rest;
     for (int c = 0; c < kLists; ++c) {
         const size_t op = size_t(1 + c) * b_ptr, oi = o0 + size_t(1 + c) * b_idx;
         std::copy(sub[c].begin(), sub[c].end(), reinterpret_cast<LatDev**>(hb + op));

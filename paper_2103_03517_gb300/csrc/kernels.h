@@ -39,7 +39,7 @@ struct KernelSet {
     // FP32 colour pass over lattices in the row layout (adjacent site pairs
     // per lane; law = 0) or outside it with rows of even Lh (law = 1: the
     // general kernel's arithmetic); gen = 0: all axes periodic, no film tables;
-    // gen = 1: any boundaries and film tables.  Null in the FP64 set.  After an
+    // gen = 1: any boundaries; gen = 2: film tables, any boundaries.  Null in the FP64 set.  After an
     // unmeasured black pass (colour 1) it also launches the close of the
     // lattices' sweeps (row_close_kernel).  Returns the status of the
     // launches (made with programmatic serialisation).
@@ -61,7 +61,7 @@ struct KernelSet {
     void (*mlong)(const GroupArgs& g, uint32_t ntiles, cudaStream_t s);
     // Standalone sample + end of sweep (site tiles).
     void (*measure)(const GroupArgs& g, uint32_t ntiles, cudaStream_t s);
-    // The same over lattices in the row layout (gen as in row_pass); with gen
+    // The same over lattices in the row layout (gen as in row_pass, law 0); with gen
     // = 0 it also stores the red sites' field for the next constrained sweep
     // (LatParams::pfield).  Null in the FP64 set.
     void (*row_sample)(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s);
@@ -120,14 +120,12 @@ struct KernelSet {
 struct LaunchSet {
     GroupArgs all, pairs, pairs_lead;
     uint32_t nt_all = 0, nt_pairs = 0, nt_pairs_lead = 0;  // pair tiles: pair order, site order
-    // colour passes: row kernel, row kernel with boundaries and films, the
-    // same two for rows of even Lh outside the row layout, the general kernel
-    // (tiles)
-    GroupArgs row, rowx, even, evenx, rest;
-    uint32_t nt_row = 0, nt_rowx = 0, nt_even = 0, nt_evenx = 0, nt_rest = 0;
+    // colour passes: lattices and tiles of each colour-pass kernel
+    GroupArgs col[kColourKinds];
+    uint32_t nt_col[kColourKinds] = {};
     // wavefront lattices (LatParams::wave): their work-unit plan (nb_wave
     // blocks; 0 = none), and the row-kernel list without them, which runs
-    // beside a wavefront launch (row above keeps them, for sweeps that run
+    // beside a wavefront launch (col keeps them, for sweeps that run
     // as two row passes)
     WaveArgs wave = {};
     uint32_t nb_wave = 0;

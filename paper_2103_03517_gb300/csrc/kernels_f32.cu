@@ -30,7 +30,8 @@ namespace {
 
 using R = float;
 constexpr int MINB = MC_MINB_F32;  // minimum resident blocks per SM of the colour pass
-constexpr int MINB_GEN = MC_MINB_GEN_F32;  // the same for the row kernel with boundaries and films
+constexpr int MINB_FACES = 3;              // the same for the row kernel with faces
+constexpr int MINB_GEN = MC_MINB_GEN_F32;  // the same for the row kernel with film tables
 constexpr int MINB_PAIR = MC_MINB_PAIR_F32;  // the same for the pair pass
 constexpr int MINB_PAIR_LEAD = 2;            // the same for the pair pass in site order
 constexpr int kPairChunk = MC_PAIR_CHUNK;    // consecutive pair tiles per grid-stride step
@@ -81,10 +82,12 @@ cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int 
                      int shape, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
     if (law) {
-        if (gen) return row_pass_g<1, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, s);
+        if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, s);
+        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, s);
         return row_pass_g<0, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, s);
     }
-    if (gen) return row_pass_g<1, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, s);
+    if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, s);
+    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, s);
     return row_pass_g<0, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, s);
 }
 
@@ -92,14 +95,15 @@ cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int 
 // (the next constrained sweep's red field); the other keeps black
 template <int GEN>
 void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
-    constexpr int B = GEN ? MINB_GEN : MINB;
+    constexpr int B = GEN == 2 ? MINB_GEN : (GEN == 1 ? MINB_FACES : MINB);
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
     const Spread sp = spread_warps(ntiles, cap);
     row_pass_kernel<B, 2, GEN, 0><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, nullptr, GEN ? 1 : 0);
 }
 
 void row_sample(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s) {
-    if (gen) row_sample_g<1>(g, ntiles, s);
+    if (gen == 2) row_sample_g<2>(g, ntiles, s);
+    else if (gen == 1) row_sample_g<1>(g, ntiles, s);
     else row_sample_g<0>(g, ntiles, s);
 }
 

@@ -65,7 +65,16 @@ inline FastDiv make_fastdiv(uint32_t d) {
     return f;
 }
 
-enum { kColourGeneral = 0, kColourRow = 1, kColourRowGen = 2, kColourEven = 3, kColourEvenGen = 4 };
+// Colour-pass kernels.  General: any lattice.  The others are FP32 lattices on
+// the row kernel: Row* in the row layout (its LAW 0), Even* outside it with
+// even Lh (LAW 1), each with all axes periodic, with open, pinned or
+// anti-periodic faces, or with film tables and any faces (its GEN 0, 1, 2).
+enum {
+    kColourGeneral = 0,
+    kColourRow, kColourRowFaces, kColourRowFilm,
+    kColourEven, kColourEvenFaces, kColourEvenFilm,
+    kColourKinds
+};
 
 // One neighbour entry of a bcc / fcc / hcp sub-lattice: the neighbour's
 // sub-lattice, its cell offset and its coupling (J1 or J2), with what the
@@ -105,11 +114,7 @@ struct LatParams {
     int pair_leader;        // constrained pass in site order (FP32, automatic kernel path)
     int xnb_n[kXtalMaxSub]; // bcc / fcc: neighbour entries per sub-lattice
     const void* xnb;        // bcc / fcc: [kXtalMaxSub][kXtalMaxNb] XtalNb, or null
-    int colour_kernel;      // colour-pass kernel: kColourGeneral, kColourRow (FP32 row
-                            // layout, all axes periodic, no film tables),
-                            // kColourRowGen (FP32 row layout, any boundaries and films);
-                            // kColourEven, kColourEvenGen: the same two for FP32
-                            // lattices outside the row layout with even Lh
+    int colour_kernel;      // colour-pass kernel (kColourGeneral, ...)
     void* spins;
     void* spins_alt;        // wavefront lattices (wave != 0): the second spin buffer
                             // a fused sweep writes (same layout), else null

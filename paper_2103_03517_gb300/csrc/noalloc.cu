@@ -130,16 +130,8 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     ls.nt_all = p.nblocks_site;
     ls.nt_pairs = p.nblocks_pair;
     ls.sample_level = 2;
-    if (p.colour_kernel == kColourRow) {  // every axis periodic: the row kernel or the general one
-        ls.row = ls.all;
-        ls.nt_row = ls.nt_all;
-    } else if (p.colour_kernel == kColourEven) {
-        ls.even = ls.all;
-        ls.nt_even = ls.nt_all;
-    } else {
-        ls.rest = ls.all;
-        ls.nt_rest = ls.nt_all;
-    }
+    ls.col[p.colour_kernel] = ls.all;
+    ls.nt_col[p.colour_kernel] = ls.nt_all;
     rc = enqueue_sweeps(kernels_f32(), ls, base + kOffCone, n_sweeps, samples ? 1 : 0, false, s, nullptr);
     if (rc) return rc;
     if (samples) {

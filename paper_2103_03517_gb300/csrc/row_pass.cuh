@@ -1,12 +1,12 @@
 // row_pass.cuh -- FP32 colour pass (Table A1) over lattices in the row layout:
 // Lx even, rows of Lh = Lx/2 sites per colour a power of two <= 64 or a
 // multiple of 64, and Nc a multiple of 64, so that every warp tile is full
-// and its rows split evenly over the lanes.  Two instances: GEN = 0 for
+// and its rows split evenly over the lanes.  Three instances: GEN = 0 for
 // lattices with every axis periodic and no film tables (the batched m(T)
-// workload), GEN = 1 for any boundary modes (open, pinned, anti-periodic),
-// bond masks and per-grain easy axes (walls, granular films).  Neither holds
-// the general-geometry code of the general colour pass, so that they run in
-// fewer registers.
+// workload), GEN = 1 for any boundary modes (open, pinned, anti-periodic:
+// walls, particles), GEN = 2 for bond masks and per-grain easy axes as well
+// (granular films).  None holds the general-geometry code of the general
+// colour pass, so that they run in fewer registers.
 //
 // Lane L of a tile of 64 colour indices q0 .. q0 + 63 takes the adjacent pair
 // q = q0 + 2L, q + 1 of one row, so that every spin is read as a float2 (one
@@ -17,8 +17,10 @@
 // of the pair; the fourth, at k-1 or k+2, is the neighbouring lane's pair,
 // taken by a warp shuffle inside the row group (wrapping the row) or, at the
 // ends of a 64-site segment of a longer row, loaded on its own.  The
-// neighbour sum keeps the order -x, +x, -y, +y, -z, +z.  In the GEN instance
-// every neighbour enters with a factor 1, -1 (across an anti-periodic face)
+// neighbour sum keeps the order -x, +x, -y, +y, -z, +z.  In the GEN 1 instance
+// the bonds across x faces enter with their factor, and the factors of y and z
+// only in tiles with a row on such a face; in GEN 2 every neighbour enters with
+// a factor 1, -1 (across an anti-periodic face)
 // or 0 (absent: open face or missing bond), an exact product.
 //
 // LAW 1 takes the lattices outside the row layout whose rows hold an even
@@ -43,7 +45,7 @@ __device__ __forceinline__ float face_factor(int bc) { return bc == 0 ? 1.0f : (
 
 // Spins and neighbour sums of lane L's pair in the tile starting at q0,
 // packed (site 0 in .x, site 1 in .y, as loaded); returns the lattice index
-// of the pair's first site (its parity is the row's x offset).  GEN:
+// of the pair's first site (its parity is the row's x offset).  GEN 1, 2:
 // mov[v] = site v is not on a pinned plane.
 template <int GEN, int LAW = 0>
 __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const float* s, int colour, uint32_t q0,
@@ -97,16 +99,42 @@ __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const floa
     // the other colour at the pair's own indices: one x neighbour of each
     // site (and the site of the other colour the sample pairs with it)
     O = P3{v[3], v[4], v[5]};
-    if constexpr (GEN == 0) {
+    if constexpr (GEN <= 1) {
+        const int bx = p.bc[0], by = p.bc[1], bz = p.bc[2];
+        if constexpr (GEN == 1) {
+            // a bond across an x face enters with the face's factor
+            const float fl = k == 0 ? face_factor(bx) : 1.0f, fr = k + 2 == Lh ? face_factor(bx) : 1.0f;
+            lft = V3<float>{fl * lft.x, fl * lft.y, fl * lft.z};
+            rgt = V3<float>{fr * rgt.x, fr * rgt.y, fr * rgt.z};
+        }
         // the other x neighbour: site 0 has (xoff ? o1 : lft), site 1 has
         // (xoff ? rgt : o0); the -x + +x sum is the same either way round
         const P3 a{make_float2(xoff ? v[3].y : lft.x, xoff ? rgt.x : v[3].x),
                    make_float2(xoff ? v[4].y : lft.y, xoff ? rgt.y : v[4].x),
                    make_float2(xoff ? v[5].y : lft.z, xoff ? rgt.z : v[5].x)};
-        h.x = p2add(p2add(p2add(p2add(p2add(O.x, a.x), v[6]), v[9]), v[12]), v[15]);
-        h.y = p2add(p2add(p2add(p2add(p2add(O.y, a.y), v[7]), v[10]), v[13]), v[16]);
-        h.z = p2add(p2add(p2add(p2add(p2add(O.z, a.z), v[8]), v[11]), v[14]), v[17]);
+        h = P3{p2add(O.x, a.x), p2add(O.y, a.y), p2add(O.z, a.z)};
+        // rows on a y or z face whose bonds do not simply wrap: factors (no
+        // lane's, in most tiles)
+        const bool edge = GEN == 1 && ((by != 0 && (y == 0 || y + 1 == Ly)) || (bz != 0 && (z == 0 || z + 1 == Lz)));
+        if (GEN == 1 && __any_sync(0xffffffffu, edge)) {
+            const float f[4] = {y > 0 ? 1.0f : face_factor(by), y + 1 < Ly ? 1.0f : face_factor(by),
+                                z > 0 ? 1.0f : face_factor(bz), z + 1 < Lz ? 1.0f : face_factor(bz)};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                h = P3{p2fma(p2(f[j]), v[6 + 3 * j], h.x), p2fma(p2(f[j]), v[7 + 3 * j], h.y),
+                       p2fma(p2(f[j]), v[8 + 3 * j], h.z)};
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                h = P3{p2add(h.x, v[6 + 3 * j]), p2add(h.y, v[7 + 3 * j]), p2add(h.z, v[8 + 3 * j])};
+        }
         mov[0] = mov[1] = true;
+        if constexpr (GEN == 1) {
+            const uint32_t x0 = xoff + 2u * k;
+            const bool row_pinned = edge && ((by == 2 && (y == 0 || y + 1 == Ly)) || (bz == 2 && (z == 0 || z + 1 == Lz)));
+            mov[0] = !row_pinned && !(bx == 2 && x0 == 0);
+            mov[1] = !row_pinned && !(bx == 2 && x0 + 3 == uint32_t(p.Lx));
+        }
     } else {
         const int bx = p.bc[0], by = p.bc[1], bz = p.bc[2];
         const uint32_t x0 = xoff + 2u * k;  // x of site 0; site 1 is at x0 + 2
@@ -208,8 +236,8 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
             const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, S, h, O, mov);
             const bool valid = LAW == 0 || q0 + 2u * uint32_t(lane) < p.Nc;
             P3 e, eo;  // per-site easy axes (films with grain axes)
-            const bool grains = GEN != 0 && p.grain;
-            if constexpr (GEN != 0) {
+            const bool grains = GEN == 2 && p.grain;
+            if constexpr (GEN == 2) {
                 if (grains) {
                     V3<float> a[2], b[2];
                     const uint32_t qa = LAW == 1 ? min(q0 + 2u * uint32_t(lane), p.Nc - 2u) : q0 + 2u * uint32_t(lane);

@@ -126,10 +126,10 @@ int row_fast(const LatParams& p, bool film) {
 // Colour-pass kernel of a lattice (LatParams::colour_kernel).
 int colour_kernel(const LatParams& p, bool film, int path) {
     if (p.precision != MC_FP32 || path == MC_PATH_GENERAL) return kColourGeneral;
-    if (row_layout(p)) return row_fast(p, film) ? kColourRow : kColourRowGen;
-    if (p.Lh % 2) return kColourGeneral;  // a lane's pair may lie in two rows
-    return !film && p.bc[0] == MC_PERIODIC && p.bc[1] == MC_PERIODIC && p.bc[2] == MC_PERIODIC ? kColourEven
-                                                                                               : kColourEvenGen;
+    const bool faces = p.bc[0] != MC_PERIODIC || p.bc[1] != MC_PERIODIC || p.bc[2] != MC_PERIODIC;
+    const int gen = film ? 2 : (faces ? 1 : 0);
+    if (row_layout(p)) return kColourRow + gen;
+    return p.Lh % 2 ? kColourGeneral : kColourEven + gen;  // odd: a lane's pair may lie in two rows
 }
 
 // ------------------------------------------------------------- lattices
@@ -689,9 +689,9 @@ LaunchSet single_launch_set(mc_lattice* h) {
         ls.xtal = h->d_lat;
         ls.nsub = h->hp.nsub;
         for (int i = 0; i < h->hp.nsub; ++i) ls.xnb_max = std::max(ls.xnb_max, h->hp.xnb_n[i]);
-    } else if (h->hp.colour_kernel == kColourRow) {
-        ls.row = ls.all;
-        ls.nt_row = ls.nt_all;
+    } else {
+        ls.col[h->hp.colour_kernel] = ls.all;
+        ls.nt_col[h->hp.colour_kernel] = ls.nt_all;
         if (h->res) {
             ls.res = &h->res;
             ls.n_res = 1;
@@ -699,22 +699,10 @@ LaunchSet single_launch_set(mc_lattice* h) {
         if (h->hp.wave) {
             ls.wave = h->wave_args;
             ls.nb_wave = h->wave_nblocks;
-        } else {
+        } else if (h->hp.colour_kernel == kColourRow) {
             ls.row_rest = ls.all;
             ls.nt_row_rest = ls.nt_all;
         }
-    } else if (h->hp.colour_kernel == kColourRowGen) {
-        ls.rowx = ls.all;
-        ls.nt_rowx = ls.nt_all;
-    } else if (h->hp.colour_kernel == kColourEven) {
-        ls.even = ls.all;
-        ls.nt_even = ls.nt_all;
-    } else if (h->hp.colour_kernel == kColourEvenGen) {
-        ls.evenx = ls.all;
-        ls.nt_evenx = ls.nt_all;
-    } else {
-        ls.rest = ls.all;
-        ls.nt_rest = ls.nt_all;
     }
     return ls;
 }
@@ -923,22 +911,19 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         return MC_OK;
     }
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
+    auto kind_pass = [&](int kind, const GroupArgs& ga, uint32_t nt, int colour, int meas) {
+        if (!nt) return;
+        if (kind == kColourGeneral) {
+            k.colour_pass(ga, nt, cone, colour, meas, s);
+            return;
+        }
+        const cudaError_t e = k.row_pass(ga, nt, cone, colour, meas, kind >= kColourEven ? 1 : 0,
+                                         (kind - kColourRow) % 3, ls.shape.row, s);
+        if (launch_err == cudaSuccess) launch_err = e;
+    };
     auto colour_pass = [&](int colour, int meas) {
-        if (ls.nt_row) {
-            const cudaError_t e = k.row_pass(ls.row, ls.nt_row, cone, colour, meas, 0, 0, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        if (ls.nt_rowx) {
-            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 0, 1, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        for (int gen = 0; gen < 2; ++gen) {
-            const uint32_t nt = gen ? ls.nt_evenx : ls.nt_even;
-            if (!nt) continue;
-            const cudaError_t e = k.row_pass(gen ? ls.evenx : ls.even, nt, cone, colour, meas, 1, gen, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        if (ls.nt_rest) k.colour_pass(ls.rest, ls.nt_rest, cone, colour, meas, s);
+        for (int c = kColourRow; c < kColourKinds; ++c) kind_pass(c, ls.col[c], ls.nt_col[c], colour, meas);
+        kind_pass(kColourGeneral, ls.col[kColourGeneral], ls.nt_col[kColourGeneral], colour, meas);
     };
     if (ls.xtal) {  // bcc / fcc / hcp: the 2 nsub sub-sets in turn, then the sample
         for (int i = 0; i < n; ++i) {
@@ -975,25 +960,14 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         return MC_OK;
     }
     // the lattices beside a wavefront launch: the row list without the
-    // wavefront lattices, the boundary and general lists
+    // wavefront lattices, and every other list
     auto rest_pass = [&](int colour, int meas) {
-        if (ls.nt_row_rest) {
-            const cudaError_t e = k.row_pass(ls.row_rest, ls.nt_row_rest, cone, colour, meas, 0, 0, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        if (ls.nt_rowx) {
-            const cudaError_t e = k.row_pass(ls.rowx, ls.nt_rowx, cone, colour, meas, 0, 1, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        for (int gen = 0; gen < 2; ++gen) {
-            const uint32_t nt = gen ? ls.nt_evenx : ls.nt_even;
-            if (!nt) continue;
-            const cudaError_t e = k.row_pass(gen ? ls.evenx : ls.even, nt, cone, colour, meas, 1, gen, ls.shape.row, s);
-            if (launch_err == cudaSuccess) launch_err = e;
-        }
-        if (ls.nt_rest) k.colour_pass(ls.rest, ls.nt_rest, cone, colour, meas, s);
+        kind_pass(kColourRow, ls.row_rest, ls.nt_row_rest, colour, meas);
+        for (int c = kColourRow + 1; c < kColourKinds; ++c) kind_pass(c, ls.col[c], ls.nt_col[c], colour, meas);
+        kind_pass(kColourGeneral, ls.col[kColourGeneral], ls.nt_col[kColourGeneral], colour, meas);
     };
-    const bool rest_any = ls.nt_row_rest || ls.nt_rowx || ls.nt_even || ls.nt_evenx || ls.nt_rest;
+    bool rest_any = ls.nt_row_rest != 0;
+    for (int c = 0; c < kColourKinds; ++c) rest_any = rest_any || (c != kColourRow && ls.nt_col[c]);
     bool red_field_ready = false;  // the next constrained sweep's red field is stored
     for (int i = 0; i < n; ++i) {
         // wavefront lattices sweep two at a time, spins -> spins_alt -> spins,
@@ -1032,12 +1006,13 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
             red_field_ready = false;
             if (measure) {
                 if (k.row_sample) {  // row-layout lattices sample in the row kernels
-                    if (ls.nt_row) k.row_sample(ls.row, ls.nt_row, 0, s);
-                    if (ls.nt_rowx) k.row_sample(ls.rowx, ls.nt_rowx, 1, s);
-                    if (ls.nt_rest) k.measure(ls.rest, ls.nt_rest, s);
-                    if (ls.nt_even) k.measure(ls.even, ls.nt_even, s);
-                    if (ls.nt_evenx) k.measure(ls.evenx, ls.nt_evenx, s);
-                    red_field_ready = ls.nt_row && !ls.nt_rowx && !ls.nt_rest && !ls.nt_even && !ls.nt_evenx;
+                    red_field_ready = ls.nt_col[kColourRow] != 0;
+                    for (int c = 0; c < kColourKinds; ++c) {
+                        if (!ls.nt_col[c]) continue;
+                        if (c >= kColourRow && c <= kColourRowFilm) k.row_sample(ls.col[c], ls.nt_col[c], c - kColourRow, s);
+                        else k.measure(ls.col[c], ls.nt_col[c], s);
+                        red_field_ready = red_field_ready && c == kColourRow;
+                    }
                 } else {
                     k.measure(ls.all, ls.nt_all, s);
                 }

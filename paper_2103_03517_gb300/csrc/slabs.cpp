@@ -62,7 +62,7 @@ MC_API int mc_slab_create(const mc_desc* d, int z0, int nz, mc_handle* out) {
     const SlabSpec spec{z0, nz, Lz};
     rc = create_lattice(&ld, out, &spec);
     if (rc) return rc;
-    if ((*out)->hp.colour_kernel != kColourRowGen) {
+    if ((*out)->hp.colour_kernel != kColourRowFaces) {
         mc_destroy(*out);
         *out = nullptr;
         return fail(MC_ERR_ARG, "a slab needs the FP32 row layout (Lx/2 a power of two <= 64 or a multiple of 64, "
@@ -88,7 +88,7 @@ MC_API int mc_slab_pass(mc_handle h, int colour, int measure) {
     cudaSetDevice(h->device);
     const LaunchSet ls = single_launch_set(h);
     const int level = measure ? (h->hp.sample_torque ? 2 : 1) : 0;
-    const cudaError_t e = kernels_f32().row_pass(ls.rowx, ls.nt_rowx, h->cone, colour ^ h->hp.cflip, level, 0, 1,
+    const cudaError_t e = kernels_f32().row_pass(ls.col[kColourRowFaces], ls.nt_col[kColourRowFaces], h->cone, colour ^ h->hp.cflip, level, 0, 1,
                                                  ls.shape.row, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "slab pass");
     return MC_OK;

@@ -59,7 +59,9 @@ int copy_state(const std::vector<mc_lattice*>& lats, Snapshot& snap, bool save, 
 int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats, const void* cone, int sweeps,
              int what, cudaStream_t s, mc_tune_report* out) {
     if (sweeps < 1 || !(what & (MC_TUNE_SWEEP | MC_TUNE_CONSTRAINED))) return fail(MC_ERR_ARG, "invalid argument");
-    const bool tune_free = (what & MC_TUNE_SWEEP) && (ls.nt_row || ls.nt_rowx || ls.nt_even || ls.nt_evenx);
+    bool row_kernel = false;
+    for (int c = kColourRow; c < kColourKinds; ++c) row_kernel = row_kernel || ls.nt_col[c];
+    const bool tune_free = (what & MC_TUNE_SWEEP) && row_kernel;
     const bool tune_cons = (what & MC_TUNE_CONSTRAINED) && (ls.nt_pairs || ls.nt_pairs_lead);
     for (mc_lattice* h : lats) {
         if (h->hp.nsub > 1) return fail(MC_ERR_ARG, "crystal lattices have no tunable launch shape");
