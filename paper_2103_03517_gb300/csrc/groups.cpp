@@ -90,6 +90,7 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
         const int c = hp.colour_kernel, q = kPairs + (hp.pair_leader ? 1 : 0);
         sub[c].push_back(all[j]);
         st[c].push_back(st[c].back() + hp.nblocks_site);
+        g->ls.turns[c] = (sub[c].size() == 1 || g->ls.turns[c]) && long_rows(hp);
         sub[q].push_back(all[j]);
         st[q].push_back(st[q].back() + hp.nblocks_pair);
         if (hp.wave) {

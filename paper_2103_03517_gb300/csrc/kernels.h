@@ -39,12 +39,13 @@ struct KernelSet {
     // FP32 colour pass over lattices in the row layout (adjacent site pairs
     // per lane; law = 0) or outside it with rows of even Lh (law = 1: the
     // general kernel's arithmetic); gen = 0: all axes periodic, no film tables;
-    // gen = 1: any boundaries; gen = 2: film tables, any boundaries.  Null in the FP64 set.  After an
+    // gen = 1: any boundaries; gen = 2: film tables, any boundaries; turns: the
+    // warps of a block share its tiles in turn (LaunchSet::turns).  Null in the FP64 set.  After an
     // unmeasured black pass (colour 1) it also launches the close of the
     // lattices' sweeps (row_close_kernel).  Returns the status of the
     // launches (made with programmatic serialisation).
     cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law,
-                            int gen, int shape, cudaStream_t s);
+                            int gen, int shape, bool turns, cudaStream_t s);
     // Table A2 pair pass over sub-set (sub, colour) (sub = 0 for simple cubic
     // lattices); leader != 0 takes the pairs in site order
     // (LatParams::pair_leader).
@@ -123,6 +124,7 @@ struct LaunchSet {
     // colour passes: lattices and tiles of each colour-pass kernel
     GroupArgs col[kColourKinds];
     uint32_t nt_col[kColourKinds] = {};
+    bool turns[kColourKinds] = {};  // every lattice of the list is large with long rows (long_rows)
     // wavefront lattices (LatParams::wave): their work-unit plan (nb_wave
     // blocks; 0 = none), and the row-kernel list without them, which runs
     // beside a wavefront launch (col keeps them, for sweeps that run

@@ -41,9 +41,9 @@ constexpr int V = kSitesPerThreadF32;
 
 #include "launchers_common.cuh"
 
-template <int B, int MEASURE, int GEN, int LAW>
+template <int B, int MEASURE, int GEN, int LAW, int TURNS = 0>
 cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
-    static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN, 1, LAW>);
+    static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>);
     // programmatic serialisation: the pass starts its blocks while the
     // previous launch drains and waits inside the kernel (griddepcontrol)
     cudaLaunchConfig_t cfg = {};
@@ -56,7 +56,7 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN, 1, LAW>, g, ntiles, cone, colour);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, g, ntiles, cone, colour);
     if (e != cudaSuccess || colour != 1 || MEASURE > 0) return e;  // the unmeasured sweep's end
     cudaLaunchConfig_t cc = cfg;
     cc.gridDim = dim3(uint32_t(g.n));
@@ -66,8 +66,15 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
 
 // launch shape 0: the default blocks per SM of the instance; 1: the other candidate
 template <int GEN, int B0, int B1, int LAW>
-cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape,
+cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape, bool turns,
                        cudaStream_t s) {
+    if constexpr (GEN < 2) {
+        if (turns && shape == 0) {
+            if (measure >= 2) return row_pass_t<B0, 2, GEN, LAW, 1>(g, ntiles, c, colour, s);
+            if (measure == 1) return row_pass_t<B0, 1, GEN, LAW, 1>(g, ntiles, c, colour, s);
+            return row_pass_t<B0, 0, GEN, LAW, 1>(g, ntiles, c, colour, s);
+        }
+    }
     if (shape == 1) {
         if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, s);
         if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, s);
@@ -79,16 +86,16 @@ cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colo
 }
 
 cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law, int gen,
-                     int shape, cudaStream_t s) {
+                     int shape, bool turns, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
     if (law) {
-        if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, s);
-        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, s);
-        return row_pass_g<0, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, s);
+        if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        return row_pass_g<0, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
     }
-    if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, s);
-    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, s);
-    return row_pass_g<0, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, s);
+    if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    return row_pass_g<0, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
 }
 
 // the all-periodic instance samples red sites first and stores their field

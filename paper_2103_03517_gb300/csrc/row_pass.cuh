@@ -177,6 +177,12 @@ __device__ __forceinline__ V3<float> grain_axis(const LatParams& p, int colour, 
     return V3<float>{a.x, a.y, a.z};
 }
 
+// TURNS: the warps of a block take consecutive tiles in turn, so that at any
+// moment they work on neighbouring rows and find each other's rows in L1.  It
+// pays where a row is long (Lh >= 128: the rows a warp alone comes back to have
+// left L1 by then): wall 1024 x 128 x 128 217 -> 186 us a sweep, 256^3 164 ->
+// 158; it does not for the batch of 16^3 ... 128^3 (168 -> 184, where a block
+// also publishes many small lattices once per warp) nor for films (276 -> 286).
 // MOVE = 0: no moves; the sample of the current state, closing the lattice's
 // sweep as the standalone sample does after a constrained sweep: with colour
 // c, each site of colour c, the site of the other colour with its index, and
@@ -185,7 +191,7 @@ __device__ __forceinline__ V3<float> grain_axis(const LatParams& p, int colour, 
 // the red sites' neighbour sums as the field of the next sweep's red pair
 // pass: the same terms in the same order as pair_field_kernel's (the -x, +x
 // pair commutes), so the same bits.
-template <int MINB, int MEASURE, int GEN, int MOVE = 1, int LAW = 0>
+template <int MINB, int MEASURE, int GEN, int MOVE = 1, int LAW = 0, int TURNS = 0>
 __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uint32_t ntiles,
                                                                 const float* __restrict__ cone, int colour) {
     constexpr int NS = MEASURE >= 2 ? kNumSums : kSumTux;  // sums sampled
@@ -195,18 +201,23 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
     // angle and counters) before it reads any of them.  Launched without
     // the attribute, both instructions do nothing.
     asm volatile("griddepcontrol.launch_dependents;");
+    // A warp takes an even share of consecutive tiles, or with TURNS a block does
+    // and its warps take the tiles of it in turn
+    constexpr uint32_t kStep = TURNS ? kBlock / 32 : 1;
     const WarpChunk wc = warp_chunk(ntiles);
     const int lane = wc.lane;
     const uint32_t tag = tag_of(colour, kPurposeMove);
-    uint32_t tile = wc.begin;
-    int l = tile < wc.end ? lattice_of_tile(g, tile) : 0;
+    const uint32_t tend = TURNS ? uint32_t(uint64_t(blockIdx.x + 1) * ntiles / gridDim.x) : wc.end;
+    uint32_t tile = TURNS ? uint32_t(uint64_t(blockIdx.x) * ntiles / gridDim.x) + (threadIdx.x >> 5) : wc.begin;
+    int l = tile < tend ? lattice_of_tile(g, tile) : 0;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    while (tile < wc.end) {
+    for (; tile < tend; ++l) {
+        const uint32_t t0 = __ldg(&g.start[l]);
+        const uint32_t t1 = min(__ldg(&g.start[l + 1]), tend);
+        if (TURNS && tile >= t1) continue;  // a small lattice between two of the warp's tiles
         LatDev* L = g.lats[l];
         const LatParams& p = L->p;
-        const uint32_t t0 = __ldg(&g.start[l]);
-        const uint32_t t1 = min(__ldg(&g.start[l + 1]), wc.end);
-        const uint32_t run = t1 - tile;
+        const uint32_t run = (t1 - tile + kStep - 1) / kStep;
         const Par<float> par = load_par<float>(p);
         const float c = MOVE ? cone[L->st.theta] : 0.0f;
         const uint32_t sweep = L->st.sweep;
@@ -229,7 +240,7 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 #pragma unroll
         for (int i = 0; i < NS; ++i) lf[i] = 0;
         uint32_t nparts = 0;
-        for (; tile < t1; ++tile) {
+        for (; tile < t1; tile += kStep) {
             const uint32_t q0 = (tile - t0) * 64u;
             P3 S, h, O;
             bool mov[2];
@@ -330,7 +341,6 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
             publish(L->st, lane, 0, true, fix, 3, run, p.nblocks_site, true,
                     [&] { finalize_sweep(p, L->st, 1, true, lane); });
         }
-        ++l;
     }
 }
 

@@ -669,6 +669,11 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     return MC_OK;
 }
 
+// Lattices whose row-kernel passes take a block's tiles in turn (TURNS in
+// row_pass.cuh): long rows, and tiles enough that a block lies in one or two
+// lattices.
+bool long_rows(const LatParams& p) { return p.Lh >= 128 && p.nblocks_site >= 1024; }
+
 // Launch tables of the lattice alone (one colour-pass kernel).
 LaunchSet single_launch_set(mc_lattice* h) {
     LaunchSet ls;
@@ -692,6 +697,7 @@ LaunchSet single_launch_set(mc_lattice* h) {
     } else {
         ls.col[h->hp.colour_kernel] = ls.all;
         ls.nt_col[h->hp.colour_kernel] = ls.nt_all;
+        ls.turns[h->hp.colour_kernel] = long_rows(h->hp);
         if (h->res) {
             ls.res = &h->res;
             ls.n_res = 1;
@@ -918,7 +924,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
             return;
         }
         const cudaError_t e = k.row_pass(ga, nt, cone, colour, meas, kind >= kColourEven ? 1 : 0,
-                                         (kind - kColourRow) % 3, ls.shape.row, s);
+                                         (kind - kColourRow) % 3, ls.shape.row, ls.turns[kind], s);
         if (launch_err == cudaSuccess) launch_err = e;
     };
     auto colour_pass = [&](int colour, int meas) {

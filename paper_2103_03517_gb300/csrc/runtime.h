@@ -99,6 +99,7 @@ int observables_from(const mc_lattice* h, const LatState& st, mc_observables* ou
 int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* cone, int n, int measure,
                bool constrained, cudaStream_t s);
 void destroy_graphs(SweepGraphs& gr);
+bool long_rows(const LatParams& p);
 LaunchSet single_launch_set(mc_lattice* h);
 int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats, const void* cone, int sweeps,
              int what, cudaStream_t s, mc_tune_report* out);
