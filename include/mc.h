@@ -371,7 +371,7 @@ MC_API int mc_group_sync(mc_group_handle g);
 /* Launch-shape autotuning of the batched sweeps (the block and tile shapes of
  * a persistent launch).  Candidates, in the order of the report's arrays:
  *   row:   FP32 row kernel, minimum resident blocks per SM (so registers per
- *          thread): all-periodic lattices {3, 2}, boundaries and films {2, 3};
+ *          thread): {3, 2} (boundaries and films: 2 in passes with a sample);
  *          a lattice swept resident (MC_PATH_RESIDENT): threads per block
  *          {512, 640};
  *   field: constrained neighbour-field kernel, tiles per grid-stride step

@@ -4,9 +4,6 @@
 #ifndef MC_MINB_F32
 #define MC_MINB_F32 3
 #endif
-#ifndef MC_MINB_GEN_F32
-#define MC_MINB_GEN_F32 2
-#endif
 #ifndef MC_MINB_PAIR_F32
 #define MC_MINB_PAIR_F32 3
 #endif
@@ -30,8 +27,11 @@ namespace {
 
 using R = float;
 constexpr int MINB = MC_MINB_F32;  // minimum resident blocks per SM of the colour pass
-constexpr int MINB_FACES = 3;              // the same for the row kernel with faces
-constexpr int MINB_GEN = MC_MINB_GEN_F32;  // the same for the row kernel with film tables
+// The same for the row kernel with faces (GEN 1) and with film tables (GEN 2):
+// three blocks without a sample, two with one, whose sums would spill 160 to
+// 380 bytes a thread at 80 registers.  Film 1024 x 1024 x 15, at two / three
+// blocks: 278 / 253 us a sweep unmeasured, 278 / 347 measured.
+constexpr int MINB_FACES = 3, MINB_FACES_M = 2, MINB_FILM = 3, MINB_FILM_M = 2;
 constexpr int MINB_PAIR = MC_MINB_PAIR_F32;  // the same for the pair pass
 constexpr int MINB_PAIR_LEAD = 2;            // the same for the pair pass in site order
 constexpr int kPairChunk = MC_PAIR_CHUNK;    // consecutive pair tiles per grid-stride step
@@ -64,45 +64,48 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     return cudaLaunchKernelEx(&cc, row_close_kernel, g, 0);
 }
 
-// launch shape 0: the default blocks per SM of the instance; 1: the other candidate
-template <int GEN, int B0, int B1, int LAW>
-cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape, bool turns,
+// launch shape 0: the default blocks per SM of the instance (B0 of a pass
+// without a sample, B0M of one with it); 1: the other candidate, B1
+template <int GEN, int B0, int B0M, int B1, int LAW, int TURNS>
+cudaError_t row_pass_s(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape,
                        cudaStream_t s) {
-    if constexpr (GEN < 2) {
-        if (turns && shape == 0) {
-            if (measure >= 2) return row_pass_t<B0, 2, GEN, LAW, 1>(g, ntiles, c, colour, s);
-            if (measure == 1) return row_pass_t<B0, 1, GEN, LAW, 1>(g, ntiles, c, colour, s);
-            return row_pass_t<B0, 0, GEN, LAW, 1>(g, ntiles, c, colour, s);
+    if constexpr (!TURNS) {
+        if (shape == 1) {
+            if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, s);
+            if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, s);
+            return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, s);
         }
     }
-    if (shape == 1) {
-        if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, s);
-        if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, s);
-        return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, s);
-    }
-    if (measure >= 2) return row_pass_t<B0, 2, GEN, LAW>(g, ntiles, c, colour, s);
-    if (measure == 1) return row_pass_t<B0, 1, GEN, LAW>(g, ntiles, c, colour, s);
-    return row_pass_t<B0, 0, GEN, LAW>(g, ntiles, c, colour, s);
+    if (measure >= 2) return row_pass_t<B0M, 2, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
+    if (measure == 1) return row_pass_t<B0M, 1, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
+    return row_pass_t<B0, 0, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
+}
+
+template <int GEN, int B0, int B0M, int B1, int LAW>
+cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape, bool turns,
+                       cudaStream_t s) {
+    if (turns && shape == 0) return row_pass_s<GEN, B0, B0M, B1, LAW, 1>(g, ntiles, c, colour, measure, shape, s);
+    return row_pass_s<GEN, B0, B0M, B1, LAW, 0>(g, ntiles, c, colour, measure, shape, s);
 }
 
 cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law, int gen,
                      int shape, bool turns, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
     if (law) {
-        if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
-        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
-        return row_pass_g<0, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        return row_pass_g<0, MINB, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
     }
-    if (gen == 2) return row_pass_g<2, MINB_GEN, MINB_GEN + 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
-    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
-    return row_pass_g<0, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
 }
 
 // the all-periodic instance samples red sites first and stores their field
 // (the next constrained sweep's red field); the other keeps black
 template <int GEN>
 void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
-    constexpr int B = GEN == 2 ? MINB_GEN : (GEN == 1 ? MINB_FACES : MINB);
+    constexpr int B = GEN == 2 ? MINB_FILM_M : (GEN == 1 ? MINB_FACES_M : MINB);
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
     const Spread sp = spread_warps(ntiles, cap);
     row_pass_kernel<B, 2, GEN, 0><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, nullptr, GEN ? 1 : 0);

@@ -46,10 +46,11 @@ __device__ __forceinline__ float face_factor(int bc) { return bc == 0 ? 1.0f : (
 // Spins and neighbour sums of lane L's pair in the tile starting at q0,
 // packed (site 0 in .x, site 1 in .y, as loaded); returns the lattice index
 // of the pair's first site (its parity is the row's x offset).  GEN 1, 2:
-// mov[v] = site v is not on a pinned plane.
+// mov[v] = site v is not on a pinned plane; GEN 2: mm, the bond bits of the two
+// sites (adjacent bytes).
 template <int GEN, int LAW = 0>
 __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const float* s, int colour, uint32_t q0,
-                                                  int lane, P3& S, P3& h, P3& O, bool mov[2]) {
+                                                  int lane, uint32_t mm, P3& S, P3& h, P3& O, bool mov[2]) {
     const uint32_t stride = p.stride;
     const float* own = s + size_t(3 * colour) * stride;
     const float* oth = s + size_t(3 * (colour ^ 1)) * stride;
@@ -143,10 +144,6 @@ __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const floa
         const float fxp = x0 + 3 == uint32_t(p.Lx) ? face_factor(bx) : 1.0f;
         const float fym = y > 0 ? 1.0f : face_factor(by), fyp = y + 1 < Ly ? 1.0f : face_factor(by);
         const float fzm = z > 0 ? 1.0f : face_factor(bz), fzp = z + 1 < Lz ? 1.0f : face_factor(bz);
-        // bond bits of the two sites (adjacent bytes), all present without a mask
-        const uint32_t mm = p.bonds ? uint32_t(__ldg(reinterpret_cast<const unsigned short*>(
-                                          p.bonds + size_t(colour) * stride + q)))
-                                    : 0x3F3Fu;
         auto fac = [mm](int bit, float base) { return ((mm >> bit) & 1u) ? base : 0.0f; };
         // -x and +x neighbours of the two sites, and each term's factor (an
         // exact 1, -1 or 0), packed (site 0, site 1)
@@ -170,19 +167,38 @@ __device__ __forceinline__ uint32_t row_pair_sums(const LatParams& p, const floa
     return xoff + 2u * k + uint32_t(p.Lx) * row;
 }
 
-// Easy axis of grain table entry g (float4 rows).
-__device__ __forceinline__ V3<float> grain_axis(const LatParams& p, int colour, uint32_t q) {
-    const int32_t g = __ldg(&p.grain[uint32_t(colour) * p.stride + q]);
-    const float4 a = __ldg(static_cast<const float4*>(p.gaxis) + g);
-    return V3<float>{a.x, a.y, a.z};
+// Film tables of a lane's pair at q: its bond bits (all present without a
+// mask), its grains, and those of the other colour's pair (a sample's).
+struct FilmPair {
+    uint32_t bonds;
+    int2 g, go;
+};
+
+template <bool SAMPLE>
+__device__ __forceinline__ FilmPair film_pair(const LatParams& p, int colour, uint32_t q) {
+    FilmPair f{0x3F3Fu, make_int2(0, 0), make_int2(0, 0)};
+    if (p.bonds)
+        f.bonds = __ldg(reinterpret_cast<const unsigned short*>(p.bonds + size_t(colour) * p.stride + q));
+    if (p.grain) {
+        f.g = __ldg(reinterpret_cast<const int2*>(p.grain + size_t(colour) * p.stride + q));
+        if (SAMPLE) f.go = __ldg(reinterpret_cast<const int2*>(p.grain + size_t(colour ^ 1) * p.stride + q));
+    }
+    return f;
+}
+
+// Easy axes of two entries of the grain table (float4 rows), packed.
+__device__ __forceinline__ P3 grain_axes(const LatParams& p, int2 g) {
+    const float4 a = __ldg(static_cast<const float4*>(p.gaxis) + g.x), b = __ldg(static_cast<const float4*>(p.gaxis) + g.y);
+    return P3{make_float2(a.x, b.x), make_float2(a.y, b.y), make_float2(a.z, b.z)};
 }
 
 // TURNS: the warps of a block take consecutive tiles in turn, so that at any
 // moment they work on neighbouring rows and find each other's rows in L1.  It
 // pays where a row is long (Lh >= 128: the rows a warp alone comes back to have
 // left L1 by then): wall 1024 x 128 x 128 217 -> 186 us a sweep, 256^3 164 ->
-// 158; it does not for the batch of 16^3 ... 128^3 (168 -> 184, where a block
-// also publishes many small lattices once per warp) nor for films (276 -> 286).
+// 158, film 1024 x 1024 x 15 267 -> 253; it does not for the batch of 16^3 ...
+// 128^3 (168 -> 184, where a block also publishes many small lattices once per
+// warp).
 // MOVE = 0: no moves; the sample of the current state, closing the lattice's
 // sweep as the standalone sample does after a constrained sweep: with colour
 // c, each site of colour c, the site of the other colour with its index, and
@@ -240,27 +256,30 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 #pragma unroll
         for (int i = 0; i < NS; ++i) lf[i] = 0;
         uint32_t nparts = 0;
+        // films: the tables of a tile are read one tile ahead, since its axes hang
+        // on its grains
+        FilmPair ahead{};
+        auto film_at = [&](uint32_t t) {
+            const uint32_t q = (t - t0) * 64u + 2u * uint32_t(lane);
+            return film_pair<(MEASURE > 0)>(p, colour, LAW == 1 ? min(q, p.Nc - 2u) : q);
+        };
+        if constexpr (GEN == 2) ahead = film_at(tile);
         for (; tile < t1; tile += kStep) {
             const uint32_t q0 = (tile - t0) * 64u;
             P3 S, h, O;
-            bool mov[2];
-            const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, S, h, O, mov);
-            const bool valid = LAW == 0 || q0 + 2u * uint32_t(lane) < p.Nc;
             P3 e, eo;  // per-site easy axes (films with grain axes)
             const bool grains = GEN == 2 && p.grain;
+            const FilmPair film = ahead;
             if constexpr (GEN == 2) {
                 if (grains) {
-                    V3<float> a[2], b[2];
-                    const uint32_t qa = LAW == 1 ? min(q0 + 2u * uint32_t(lane), p.Nc - 2u) : q0 + 2u * uint32_t(lane);
-#pragma unroll
-                    for (int v = 0; v < 2; ++v) {
-                        a[v] = grain_axis(p, colour, qa + v);
-                        b[v] = grain_axis(p, colour ^ 1, qa + v);
-                    }
-                    e = pack(a);
-                    eo = pack(b);
+                    e = grain_axes(p, film.g);
+                    if (MEASURE > 0) eo = grain_axes(p, film.go);
                 }
+                if (tile + kStep < t1) ahead = film_at(tile + kStep);
             }
+            bool mov[2];
+            const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, film.bonds, S, h, O, mov);
+            const bool valid = LAW == 0 || q0 + 2u * uint32_t(lane) < p.Nc;
             if (!grains) e = eo = P3{p2(e_ax.x), p2(e_ax.y), p2(e_ax.z)};
             P3 Sf = S;
             bool any = false;
