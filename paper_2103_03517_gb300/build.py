@@ -28,6 +28,8 @@ SOURCES = {
     "kernels_f64.cu": ["-fmad=false", "-prec-div=true", "-prec-sqrt=true"],
     "kernels_f32.cu": ["--use_fast_math"],
     "kernels_brick.cu": ["--use_fast_math"],
+    "kernels_xtal_f64.cu": ["-fmad=false", "-prec-div=true", "-prec-sqrt=true"],
+    "kernels_xtal_f32.cu": ["--use_fast_math"],
     "runtime.cpp": [],
     "groups.cpp": [],
     "tune.cpp": [],

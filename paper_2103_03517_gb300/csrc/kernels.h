@@ -30,6 +30,23 @@ struct alignas(128) ResidentPlan {
     ResidentArgs args;
 };
 
+// Launchers of a bcc, fcc or hcp lattice (one lattice a launch), a set per
+// precision.
+struct XtalKernels {
+    // pass over sub-set (sub, colour) of ntiles 32-site tiles (finalize != 0
+    // closes the sweep)
+    cudaError_t (*pass)(const XtalArgs& a, uint32_t ntiles, const void* cone, int sub, int colour, int finalize,
+                        cudaStream_t s);
+    // the sample over the 2 nsub sub-sets (ntiles = 2 nsub tiles_per_subset),
+    // which closes the sweep (level 2: with the torques)
+    cudaError_t (*sample)(const XtalArgs& a, uint32_t ntiles, uint32_t tiles_per_subset, int level, cudaStream_t s);
+    // constrained sweeps: the neighbour field of sub-set (sub, colour) into
+    // LatParams::pfield
+    void (*field)(const XtalArgs& a, uint32_t ntiles, int sub, int colour, cudaStream_t s);
+};
+const XtalKernels& xtal_f64();
+const XtalKernels& xtal_f32();
+
 struct KernelSet {
     // Table A1 colour pass over the lattices of g (ntiles = warp tiles of the
     // launch; the launcher sizes a persistent grid from the occupancy).
@@ -66,17 +83,6 @@ struct KernelSet {
     // = 0 it also stores the red sites' field for the next constrained sweep
     // (LatParams::pfield).  Null in the FP64 set.
     void (*row_sample)(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s);
-    // bcc / fcc / hcp lattice L alone: a pass over sub-set (sub, colour) of
-    // ntiles 32-site tiles (finalize != 0 closes the sweep), and the sample
-    // over the 2 nsub sub-sets (ntiles = 2 nsub tiles_per_subset), which
-    // closes it (level 2: with the torques); nb = the most neighbour entries
-    // of a sub-lattice.
-    void (*xtal_pass)(LatDev* L, uint32_t ntiles, const void* cone, int sub, int colour, int finalize, int nb,
-                      cudaStream_t s);
-    void (*xtal_sample)(LatDev* L, uint32_t ntiles, uint32_t tiles_per_subset, int nb, int level, cudaStream_t s);
-    // Constrained sweeps of a crystal L: the neighbour field of sub-set (sub,
-    // colour) into LatParams::pfield (ntiles 32-site tiles).
-    void (*xtal_field)(LatDev* L, uint32_t ntiles, int sub, int colour, int nb, cudaStream_t s);
     // One grain sample of a film lattice (ntiles site tiles, n_grains grains).
     void (*grain_sample)(LatDev* L, uint32_t ntiles, int n_grains, cudaStream_t s);
     // Slice sums for the profile of one lattice.
@@ -144,10 +150,9 @@ struct LaunchSet {
     BrickArgs* brick = nullptr;
     uint32_t brick_lh = 0;
     int sample_level = 2;  // sample of a measured colour pass: 1 or 2 (torques)
-    // a bcc / fcc lattice alone: its descriptor and sub-lattice count, else null
-    LatDev* xtal = nullptr;
+    // a bcc / fcc / hcp lattice alone (xtal.lat, else null) and its sub-lattices
+    XtalArgs xtal = {};
     int nsub = 1;
-    int xnb_max = 0;  // most neighbour entries of its sub-lattices
     LaunchShape shape;  // autotuned launch shapes
 };
 

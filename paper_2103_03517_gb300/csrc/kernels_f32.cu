@@ -17,7 +17,6 @@
 
 #include "kernels.h"
 #include "pass_impl.cuh"
-#include "xtal_pass.cuh"
 #include "row_pass.cuh"
 #include "wave_pass.cuh"
 #include "resident_pass.cuh"
@@ -371,8 +370,8 @@ cudaError_t slab_close_all(LatDev* const* lats, int n, int measure, cudaStream_t
 
 const KernelSet& kernels_f32() {
     static const KernelSet k{colour_pass, row_pass,    pair_pass,   sweep_end,         pair_field,
-                             ml_reset,    mlong,       measure,     row_sample,        xtal_pass,
-                             xtal_sample, xtal_field_launch, grain_sample, profile, "f32",
+                             ml_reset,    mlong,       measure,     row_sample,        grain_sample,
+                             profile,     "f32",
                              wave_sweep,  wave_blocks, slab_export,       slab_close,   slab_halo,
                              slab_close_all, resident_sweeps, resident_plan};
     return k;

@@ -3,7 +3,6 @@
 // expression is evaluated as one IEEE operation at a time, left to right.
 #include "kernels.h"
 #include "pass_impl.cuh"
-#include "xtal_pass.cuh"
 
 namespace mcgb {
 namespace {
@@ -41,8 +40,8 @@ void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour
 
 const KernelSet& kernels_f64() {
     static const KernelSet k{colour_pass, nullptr,     pair_pass,   sweep_end,         pair_field,
-                             ml_reset,    mlong,       measure,     nullptr,           xtal_pass,
-                             xtal_sample, xtal_field_launch, grain_sample, profile, "f64",
+                             ml_reset,    mlong,       measure,     nullptr,           grain_sample,
+                             profile,     "f64",
                              nullptr,     nullptr,     nullptr,           nullptr,      nullptr,
                              nullptr,     nullptr,     nullptr};
     return k;

@@ -76,21 +76,6 @@ enum {
     kColourKinds
 };
 
-// One neighbour entry of a bcc / fcc / hcp sub-lattice: the neighbour's
-// sub-lattice, its cell offset and its coupling (J1 or J2), with what the
-// kernels need precomputed for the lattice's size: the offset taken modulo
-// (Lx, Ly, Lz), the parity of dx + dy + dz (bit 0 of par; bit 1 marks a
-// forward entry, one of each entry and its reverse), and for a site of
-// colour c the element offset of the neighbour's x-component array.
-constexpr int kXtalMaxSub = 4, kXtalMaxNb = 24;
-struct XtalNb {
-    int8_t sub, dx, dy, dz;
-    float fJ;
-    double J;
-    uint32_t dxw, dyw, dzw, par;
-    uint64_t off[2];
-};
-
 struct LatParams {
     int Lx, Ly, Lz, Lh;
     int bc[3];
@@ -112,8 +97,6 @@ struct LatParams {
     int row_lanes;          // FP32 row path: lanes per row group, min(Lh/2, 32)
     int nsub;               // sub-lattices: 1 simple cubic, 2 bcc, 4 fcc
     int pair_leader;        // constrained pass in site order (FP32, automatic kernel path)
-    int xnb_n[kXtalMaxSub]; // bcc / fcc: neighbour entries per sub-lattice
-    const void* xnb;        // bcc / fcc: [kXtalMaxSub][kXtalMaxNb] XtalNb, or null
     int colour_kernel;      // colour-pass kernel (kColourGeneral, ...)
     void* spins;
     void* spins_alt;        // wavefront lattices (wave != 0): the second spin buffer
@@ -248,6 +231,18 @@ struct ResidentArgs {
     int n_sweeps;
     int inject;
     uint32_t key0, key1;  // the lattice's Philox key, a launch constant
+};
+
+// A bcc, fcc or hcp lattice's launches (xtal_pass.cuh): its descriptor, type
+// (1 bcc, 2 fcc, 3 hcp) and couplings, and the spins and stride of its
+// parameters as launch constants.
+struct XtalArgs {
+    LatDev* lat;
+    void* spins;
+    uint32_t stride;
+    int type, j2;  // j2: J2 != 0
+    double J, J2;
+    float fJ, fJ2;
 };
 
 // Brick sweeps (brick_pass.cuh): control words of one lattice, in device

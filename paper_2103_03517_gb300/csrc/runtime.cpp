@@ -142,58 +142,6 @@ static void set_float_params(LatParams& p) {
 
 int sublattices(int lattice) { return lattice == MC_BCC ? 2 : (lattice == MC_FCC || lattice == MC_HCP ? 4 : 1); }
 
-// Neighbour table of a bcc, fcc or hcp lattice from its basis (fractions of
-// the cell; cell lengths ell, a = 1): entry (t, d) of sub-lattice s, d a
-// cell offset in {-1, 0, 1}^3, is a neighbour when |(b_t + d - b_s) ell|^2
-// equals the nearest-neighbour distance^2 (bcc 3/4, fcc 1/2, hcp 1;
-// coupling J) or, for bcc and fcc with J2 != 0, 1 (the same sub-lattice one
-// cell away; coupling J2).  Entries are ordered by t, then d_z, d_y, d_x
-// from -1 to 1: the order in which the field is summed.  hcp: the
-// orthohexagonal cell (1, sqrt 3, sqrt(8/3)) with sub-lattices (0,0,0),
-// (1/2,1/2,0), (1/2,1/6,1/2), (0,2/3,1/2).
-static void xtal_table(int lattice, double J, double J2, const LatParams& p, XtalNb out[kXtalMaxSub][kXtalMaxNb],
-                       int n[kXtalMaxSub]) {
-    const double bcc[2][3] = {{0, 0, 0}, {0.5, 0.5, 0.5}};
-    const double fcc[4][3] = {{0, 0, 0}, {0.5, 0.5, 0}, {0.5, 0, 0.5}, {0, 0.5, 0.5}};
-    const double hcp[4][3] = {{0, 0, 0}, {0.5, 0.5, 0}, {0.5, 1.0 / 6.0, 0.5}, {0, 2.0 / 3.0, 0.5}};
-    const int ns = sublattices(lattice);
-    const double(*b)[3] = lattice == MC_BCC ? bcc : (lattice == MC_FCC ? fcc : hcp);
-    const double ell[3] = {1.0, lattice == MC_HCP ? std::sqrt(3.0) : 1.0, lattice == MC_HCP ? std::sqrt(8.0 / 3.0) : 1.0};
-    const double nn2 = lattice == MC_BCC ? 0.75 : (lattice == MC_FCC ? 0.5 : 1.0);
-    const bool with_j2 = lattice != MC_HCP && J2 != 0.0;
-    for (int s = 0; s < ns; ++s) {
-        n[s] = 0;
-        for (int t = 0; t < ns; ++t)
-            for (int dz = -1; dz <= 1; ++dz)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const double r[3] = {(b[t][0] + dx - b[s][0]) * ell[0], (b[t][1] + dy - b[s][1]) * ell[1],
-                                             (b[t][2] + dz - b[s][2]) * ell[2]};
-                        const double r2 = r[0] * r[0] + r[1] * r[1] + r[2] * r[2];
-                        const bool nn = std::fabs(r2 - nn2) < 1e-9, nnn = with_j2 && std::fabs(r2 - 1.0) < 1e-9;
-                        if (!nn && !nnn) continue;
-                        XtalNb& e = out[s][n[s]++];
-                        e.sub = int8_t(t);
-                        e.dx = int8_t(dx);
-                        e.dy = int8_t(dy);
-                        e.dz = int8_t(dz);
-                        e.J = nn ? J : J2;
-                        e.fJ = float(e.J);
-                        e.dxw = uint32_t((dx + p.Lx) % p.Lx);
-                        e.dyw = uint32_t((dy + p.Ly) % p.Ly);
-                        e.dzw = uint32_t((dz + p.Lz) % p.Lz);
-                        e.par = uint32_t(dx + dy + dz + 4) & 1u;  // + 4 keeps the sum non-negative, parity unchanged
-                        for (int c = 0; c < 2; ++c)
-                            e.off[c] = (uint64_t(t) * 2 + ((uint32_t(c) + e.par) & 1u)) * 3 * uint64_t(p.stride);
-                        // forward entries (bit 1): one of each entry and its reverse
-                        // (sub-lattice t -> s, offset -d), so that summing S_i.S_j over
-                        // them sees every bond once
-                        const bool fwd = t > s || (t == s && (dz > 0 || (dz == 0 && (dy > 0 || (dy == 0 && dx > 0)))));
-                        e.par |= fwd ? 2u : 0u;
-                    }
-    }
-}
-
 // Lattices whose sweeps may run as wavefront launches (wave_pass.cuh):
 // FP32 simple cubic, every axis periodic, no film tables, rows of 64 sites
 // per colour (Lx = 128), Ly >= 16, the wavefront kernel path asked for.
@@ -258,7 +206,6 @@ size_t lattice_bytes(const mc_desc* d, bool slab) {
     size_t b = align256(sizeof(LatDev));
     b += align256(size_t(nsub) * 6 * stride * rs);
     if (wave_desc(d)) b += align256(6 * stride * rs);  // the second spin buffer
-    if (nsub > 1) b += align256(sizeof(XtalNb) * kXtalMaxSub * kXtalMaxNb);
     if (d->bond_mask) b += align256(2 * stride);
     if (d->grain_id) {
         const size_t ng = size_t(std::max(d->n_grains, 1));
@@ -508,11 +455,6 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     p.spins = take(size_t(p.nsub) * 6 * size_t(p.stride) * rs);
     p.wave = wave_desc(d) ? 1 : 0;
     if (p.wave) p.spins_alt = take(6 * size_t(p.stride) * rs);
-    XtalNb xt[kXtalMaxSub][kXtalMaxNb] = {};
-    if (p.nsub > 1) {
-        xtal_table(d->lattice, d->J, d->J2, p, xt, p.xnb_n);
-        p.xnb = take(sizeof xt);
-    }
     std::vector<uint8_t> hb;
     if (din->bond_mask) {
         hb.assign(2 * size_t(p.stride), 0);
@@ -621,7 +563,6 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     up(h->d_lat, &init, sizeof init);
     up(p.spins, hs.data(), hs.size());
     if (!hb.empty()) up(const_cast<uint8_t*>(p.bonds), hb.data(), hb.size());
-    if (p.nsub > 1) up(const_cast<void*>(p.xnb), xt, sizeof xt);
     if (!hg.empty()) {
         up(const_cast<int32_t*>(p.grain), hg.data(), hg.size() * 4);
         up(const_cast<void*>(p.gaxis), hax.data(), hax.size());
@@ -691,9 +632,10 @@ LaunchSet single_launch_set(mc_lattice* h) {
     ls.brick = h->brick;
     ls.brick_lh = uint32_t(h->hp.Lh);
     if (h->hp.nsub > 1) {
-        ls.xtal = h->d_lat;
+        const bool j2 = h->desc.lattice != MC_HCP && h->desc.J2 != 0.0;
+        ls.xtal = XtalArgs{h->d_lat, h->hp.spins, h->hp.stride, h->desc.lattice, j2 ? 1 : 0, h->desc.J, h->desc.J2,
+                           float(h->desc.J), float(h->desc.J2)};
         ls.nsub = h->hp.nsub;
-        for (int i = 0; i < h->hp.nsub; ++i) ls.xnb_max = std::max(ls.xnb_max, h->hp.xnb_n[i]);
     } else {
         ls.col[h->hp.colour_kernel] = ls.all;
         ls.nt_col[h->hp.colour_kernel] = ls.nt_all;
@@ -931,15 +873,18 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         for (int c = kColourRow; c < kColourKinds; ++c) kind_pass(c, ls.col[c], ls.nt_col[c], colour, meas);
         kind_pass(kColourGeneral, ls.col[kColourGeneral], ls.nt_col[kColourGeneral], colour, meas);
     };
-    if (ls.xtal) {  // bcc / fcc / hcp: the 2 nsub sub-sets in turn, then the sample
+    if (ls.xtal.lat) {  // bcc / fcc / hcp: the 2 nsub sub-sets in turn, then the sample
+        const XtalKernels& x = &k == &kernels_f64() ? xtal_f64() : xtal_f32();
+        auto checked = [&](cudaError_t e) {
+            if (launch_err == cudaSuccess) launch_err = e;
+        };
         for (int i = 0; i < n; ++i) {
             if (!constrained) {
                 for (int sub = 0; sub < ls.nsub; ++sub)
                     for (int colour = 0; colour < 2; ++colour) {
                         const bool last = sub == ls.nsub - 1 && colour == 1;
                         timed([&] {
-                            k.xtal_pass(ls.xtal, ls.nt_all, cone, sub, colour, last && !measure ? 1 : 0, ls.xnb_max,
-                                        s);
+                            checked(x.pass(ls.xtal, ls.nt_all, cone, sub, colour, last && !measure ? 1 : 0, s));
                         });
                     }
             } else {  // Table A2 per sub-set, as for the two colours of a simple cubic lattice
@@ -949,7 +894,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
                 for (int sub = 0; sub < ls.nsub; ++sub)
                     for (int colour = 0; colour < 2; ++colour) {
-                        k.xtal_field(ls.xtal, ls.nt_all, sub, colour, ls.xnb_max, s);
+                        x.field(ls.xtal, ls.nt_all, sub, colour, s);
                         timed([&] {
                             if (ls.nt_pairs) k.pair_pass(ls.pairs, ls.nt_pairs, cone, colour, 0, ls.shape.pair, sub, s);
                             if (ls.nt_pairs_lead)
@@ -959,9 +904,10 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 if (!measure) k.sweep_end(ls.all, s);
             }
             if (measure)
-                k.xtal_sample(ls.xtal, uint32_t(2 * ls.nsub) * ls.nt_all, ls.nt_all, ls.xnb_max, ls.sample_level, s);
+                checked(x.sample(ls.xtal, uint32_t(2 * ls.nsub) * ls.nt_all, ls.nt_all, ls.sample_level, s));
         }
         cudaError_t e = cudaGetLastError();
+        if (launch_err != cudaSuccess) e = launch_err;
         if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
         return MC_OK;
     }
