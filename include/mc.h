@@ -539,7 +539,7 @@ MC_API int mc_slab_sweep(const mc_handle* slabs, int n, int n_sweeps, int measur
  * The entry point allocates nothing: no cudaMalloc, no cudaFree, no stream,
  * no library routine that allocates.  The scratch the sweep kernels need
  * (lattice descriptor with its counters and sums, launch tables, cone table,
- * sample ring) is one static 32 KiB device array inside libmc, reserved on
+ * sample ring) is one static 36 KiB device array inside libmc, reserved on
  * every GPU that loads the library until the process exits.  Each call
  * looks up the array's device address in the current device's context (a
  * lookup that allocates nothing); the first call on a device also loads

@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
             }
             __syncwarp();
             if (MEASURE > 0 && ok && blk == 0 && lane < 2)
-                a.record[size_t(sw) * kBrickRecord + kBrickRecTheta + lane] = lane == 0 ? (long long)theta : acc;
+                a.record[size_t(sw) * kRecordWords + kRecTheta + lane] = lane == 0 ? (long long)theta : acc;
         }
         if (ok && blk == 0) {  // the run's end
             if (lane == 0) {
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                             const long long v = *reinterpret_cast<volatile long long*>(&cta_sums[lane]);
                             cta_sums[lane] = 0;
                             if (v)
-                                atomicAdd(reinterpret_cast<unsigned long long*>(&a.record[size_t(sw) * kBrickRecord + lane]),
+                                atomicAdd(reinterpret_cast<unsigned long long*>(&a.record[size_t(sw) * kRecordWords + lane]),
                                           static_cast<unsigned long long>(v));
                         }
                     }
@@ -627,8 +627,8 @@ __global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(LatDev* L, Bric
     if (*reinterpret_cast<volatile int*>(&ctl->abort)) return;
     const long long ring = st.ring_count;
     if (w < n) {
-        long long* r = record + size_t(w) * kBrickRecord;
-        const long long sum = lane < kNumSums ? r[lane] : 0, theta = r[kBrickRecTheta], acc = r[kBrickRecAcc];
+        long long* r = record + size_t(w) * kRecordWords;
+        const long long sum = lane < kNumSums ? r[lane] : 0, theta = r[kRecTheta], acc = r[kRecAcc];
         double inc, y;
         sample_words(p, sum, p.sample_torque != 0, lane, p.N, &inc, &y);  // its shuffles end the reads
         if (lane < kMomentWords) r[lane] = __double_as_longlong(inc);
@@ -650,11 +650,11 @@ __global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(LatDev* L, Bric
         for (; i + 16 <= n; i += 16) {
             double x[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = __ldcg(r + size_t(i + j) * kBrickRecord);
+            for (int j = 0; j < 16; ++j) x[j] = __ldcg(r + size_t(i + j) * kRecordWords);
 #pragma unroll
             for (int j = 0; j < 16; ++j) m += x[j];
         }
-        for (; i < n; ++i) m += __ldcg(r + size_t(i) * kBrickRecord);
+        for (; i < n; ++i) m += __ldcg(r + size_t(i) * kRecordWords);
         st.moments[lane] = m;
     }
     if (lane == 0) st.ring_count = ring + n;

@@ -57,9 +57,10 @@ struct KernelSet {
     // per lane; law = 0) or outside it with rows of even Lh (law = 1: the
     // general kernel's arithmetic); gen = 0: all axes periodic, no film tables;
     // gen = 1: any boundaries; gen = 2: film tables, any boundaries; turns: the
-    // warps of a block share its tiles in turn (LaunchSet::turns).  Null in the FP64 set.  After an
-    // unmeasured black pass (colour 1) it also launches the close of the
-    // lattices' sweeps (row_close_kernel).  Returns the status of the
+    // warps of a block share its tiles in turn (LaunchSet::turns).  Null in the FP64 set.  After a
+    // black pass (colour 1) it also launches the close of the lattices' sweeps
+    // (row_close_kernel); of measured ones the samples are formed by
+    // sample_close.  Returns the status of the
     // launches (made with programmatic serialisation).
     cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law,
                             int gen, int shape, bool turns, cudaStream_t s);
@@ -87,6 +88,10 @@ struct KernelSet {
     void (*grain_sample)(LatDev* L, uint32_t ntiles, int n_grains, cudaStream_t s);
     // Slice sums for the profile of one lattice.
     void (*profile)(LatDev* d, uint32_t Lh, uint32_t rows, cudaStream_t s);
+    // The samples of the measured sweeps of row-kernel lattices since the last
+    // call (at most kSampleRecords), of every lattice of g.  Null in the FP64
+    // set.
+    void (*sample_close)(const GroupArgs& g, cudaStream_t s);
     const char* name;
     // FP32 wavefront sweep (red and black pass in one launch) of the
     // lattices of a, nblocks blocks; dir = 0 reads spins and writes

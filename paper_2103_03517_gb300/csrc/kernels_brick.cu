@@ -104,7 +104,7 @@ cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int 
         a.n_sweeps = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
         cudaError_t e = cudaMemsetAsync(a.ctl, 0, offsetof(BrickCtl, epoch), s);
         if (e == cudaSuccess && measure)
-            e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kBrickRecord * sizeof(long long), s);
+            e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kRecordWords * sizeof(long long), s);
         if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
         if (e == cudaSuccess && measure) {
             brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a.lat, a.ctl, a.record, a.n_sweeps);

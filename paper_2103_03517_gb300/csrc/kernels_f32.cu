@@ -56,11 +56,11 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, g, ntiles, cone, colour);
-    if (e != cudaSuccess || colour != 1 || MEASURE > 0) return e;  // the unmeasured sweep's end
+    if (e != cudaSuccess || colour != 1) return e;  // the sweep's end
     cudaLaunchConfig_t cc = cfg;
     cc.gridDim = dim3(uint32_t(g.n));
     cc.blockDim = dim3(32);
-    return cudaLaunchKernelEx(&cc, row_close_kernel, g, 0);
+    return cudaLaunchKernelEx(&cc, row_close_kernel, g, MEASURE > 0 ? 1 : 0);
 }
 
 // launch shape 0: the default blocks per SM of the instance (B0 of a pass
@@ -98,6 +98,10 @@ cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int 
     if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
     if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
     return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+}
+
+void sample_close(const GroupArgs& g, cudaStream_t s) {
+    sample_close_kernel<<<uint32_t(g.n), 32 * kSampleRecords, 0, s>>>(g);
 }
 
 // the all-periodic instance samples red sites first and stores their field
@@ -371,7 +375,7 @@ cudaError_t slab_close_all(LatDev* const* lats, int n, int measure, cudaStream_t
 const KernelSet& kernels_f32() {
     static const KernelSet k{colour_pass, row_pass,    pair_pass,   sweep_end,         pair_field,
                              ml_reset,    mlong,       measure,     row_sample,        grain_sample,
-                             profile,     "f32",
+                             profile,     sample_close, "f32",
                              wave_sweep,  wave_blocks, slab_export,       slab_close,   slab_halo,
                              slab_close_all, resident_sweeps, resident_plan};
     return k;

@@ -108,6 +108,7 @@ struct LatParams {
     const uint8_t* bonds;   // [2][stride] or null
     const int32_t* grain;   // [2][stride] or null
     const void* gaxis;      // [n_grains][4] in the lattice precision, or null
+    long long* records;     // FP32: [kSampleRecords][kRecordWords]
     double* ring;           // [ring_cap][kRingWords]
     int ring_cap;
     long long* profile;     // [3][Lx] fixed-point sums
@@ -144,7 +145,7 @@ struct LatState {
     int theta;                      // cone half-angle, degrees
     uint32_t sweep;                 // sweeps completed
     int error;                      // sticky mc_status
-    int pad;
+    int nrec;                       // sample records pending (0 between calls)
     long long last_acc;
     long long sums[kNumSums];       // fixed-point lattice sums of this sample
     long long ml_hi, ml_lo;         // exact M_L of this constrained sweep
@@ -245,6 +246,13 @@ struct XtalArgs {
     float fJ, fJ2;
 };
 
+// What a measured sweep leaves behind until its sample is formed: its fixed-
+// point sums, cone angle and accepted count, in whose place the closing kernels
+// (brick_close_kernel, sample_close_kernel) put what each moment word grows by.
+constexpr int kRecordWords = 28;  // 8-byte words, at least kMomentWords
+constexpr int kRecTheta = kNumSums, kRecAcc = kNumSums + 1;
+constexpr int kSampleRecords = 16;  // records a lattice holds for launched sweeps
+
 // Brick sweeps (brick_pass.cuh): control words of one lattice, in device
 // memory.  Zeroed before every launch but the epoch, which the launch counts
 // up (1 at create): the abort flag; the blocks of brick_close_kernel that are
@@ -258,11 +266,6 @@ struct BrickCtl {
     uint32_t epoch;
 };
 
-// What a measured sweep of a brick launch leaves behind: its fixed-point
-// sample sums, cone angle and accepted count, in whose place brick_close_kernel
-// puts what each moment word grows by.
-constexpr int kBrickRecord = 28;        // 8-byte words, at least kMomentWords
-constexpr int kBrickRecTheta = kNumSums, kBrickRecAcc = kNumSums + 1;
 constexpr int kBrickMaxMeasured = 512;  // measured sweeps per launch
 
 // A brick launch: nyc x nzc bricks of rows (odd Lh: nyc blocks, runs of
@@ -272,7 +275,7 @@ struct BrickArgs {
     LatDev* lat;
     BrickCtl* ctl;
     void* packets;
-    long long* record;    // [kBrickMaxMeasured][kBrickRecord]
+    long long* record;    // [kBrickMaxMeasured][kRecordWords]
     uint32_t nyc, nzc, rows, smem;
     FastDiv div_half;     // by Lh / 2
     size_t bytes;         // of the lattice's brick memory: ctl (null until it is allocated), record, packets

@@ -14,7 +14,7 @@ namespace mcgb {
 namespace {
 
 constexpr int kMaxSamples = 256;                     // samples one call can return
-constexpr size_t kScratchBytes = 32 * 1024;          // the whole scratch array
+constexpr size_t kScratchBytes = 36 * 1024;          // the whole scratch array
 
 // Layout of the scratch array (byte offsets, 256-aligned pieces).
 constexpr size_t kOffLat = 0;
@@ -23,7 +23,8 @@ constexpr size_t kOffStartSite = kOffLats + 256;     // uint32_t [2]
 constexpr size_t kOffStartPair = kOffStartSite + 256;
 constexpr size_t kOffCone = kOffStartPair + 256;     // float [181]
 constexpr size_t kOffRing = kOffCone + 1024;         // double [kMaxSamples][kRingWords]
-constexpr size_t kUsed = kOffRing + size_t(kMaxSamples) * kRingWords * sizeof(double);
+constexpr size_t kOffRecords = kOffRing + size_t(kMaxSamples) * kRingWords * sizeof(double);
+constexpr size_t kUsed = kOffRecords + size_t(kSampleRecords) * kRecordWords * sizeof(long long);
 static_assert(sizeof(LatDev) <= kOffLats, "lattice descriptor does not fit its scratch slot");
 static_assert(kUsed <= kScratchBytes, "scratch layout exceeds the array");
 
@@ -100,6 +101,7 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     p.spins = spins;
     p.ring = reinterpret_cast<double*>(base + kOffRing);
     p.ring_cap = kMaxSamples;
+    p.records = reinterpret_cast<long long*>(base + kOffRecords);
     p.J = J; p.Ku = K_u; p.Kc = K_c; p.T = T;
     const double an = std::sqrt(axis[0] * axis[0] + axis[1] * axis[1] + axis[2] * axis[2]);
     for (int a = 0; a < 3; ++a) { p.e[a] = axis[a] / an; p.H[a] = H[a]; }

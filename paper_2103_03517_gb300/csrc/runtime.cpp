@@ -189,7 +189,7 @@ bool brick_desc(const mc_desc* d, bool slab) {
 // brick launch (brick_memory): kept out of the lattice's own allocation, which
 // it would half as large again; the 80 lattices of a constrained batch, spread
 // over so much more memory, swept 2% slower.
-constexpr size_t kBrickRecordBytes = size_t(kBrickMaxMeasured) * kBrickRecord * sizeof(long long);
+constexpr size_t kBrickRecordBytes = size_t(kBrickMaxMeasured) * kRecordWords * sizeof(long long);
 
 size_t brick_bytes(const mc_desc* d) {
     if (!brick_desc(d, false)) return 0;
@@ -213,6 +213,7 @@ size_t lattice_bytes(const mc_desc* d, bool slab) {
         b += align256(3 * ng * 8) + align256(ng * 4) + align256((ng + 1) * 8);  // grain samples
     }
     const int cap = d->ring_capacity > 0 ? d->ring_capacity : 4096;
+    if (rs == 4) b += align256(size_t(kSampleRecords) * kRecordWords * 8);
     b += align256(size_t(cap) * kRingWords * 8);
     b += align256(3 * size_t(d->dims[0]) * 8);
     // launch tables of the lattice alone: lattice pointer, site and pair starts
@@ -487,6 +488,7 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
         h->film_grain.assign(din->grain_id, din->grain_id + p.N);
         h->film_axes.assign(din->grain_axis, din->grain_axis + 3 * size_t(d->n_grains));
     }
+    if (rs == 4) p.records = reinterpret_cast<long long*>(take(size_t(kSampleRecords) * kRecordWords * 8));
     p.ring = reinterpret_cast<double*>(take(size_t(p.ring_cap) * kRingWords * 8));
     p.profile = reinterpret_cast<long long*>(take(3 * size_t(p.Lx) * 8));
     h->d_group_lats = reinterpret_cast<LatDev**>(take(sizeof(void*)));
@@ -970,6 +972,8 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
             }
         }
+        if (!constrained && measure && k.sample_close && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
+            k.sample_close(ls.all, s);
     }
     if (launch_err != cudaSuccess) return cuda_fail(launch_err, "row kernel launch");
     cudaError_t e = cudaGetLastError();
