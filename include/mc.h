@@ -539,9 +539,11 @@ MC_API int mc_slab_sweep(const mc_handle* slabs, int n, int n_sweeps, int measur
  * The entry point allocates nothing: no cudaMalloc, no cudaFree, no stream,
  * no library routine that allocates.  The scratch the sweep kernels need
  * (lattice descriptor with its counters and sums, launch tables, cone table,
- * sample ring) is one static 36 KiB device array inside libmc, reserved on
+ * sample ring) is one static 36 KiB device array inside libmc, and calls of at
+ * least 3 sweeps on a lattice of up to 64^3 spins, which run as brick sweeps
+ * (see MC_PATH_AUTO), use a second one of 4.1 MiB; both are reserved on
  * every GPU that loads the library until the process exits.  Each call
- * looks up the array's device address in the current device's context (a
+ * looks up the arrays' device addresses in the current device's context (a
  * lookup that allocates nothing); the first call on a device also loads
  * libmc's kernels there, so make that first call before any stream
  * capture.  Every call rewrites the whole scratch

@@ -28,9 +28,9 @@
 //
 // Packets.  The packet of a site is rewritten two passes after it was read:
 // by then its writer has read the reader's own packet of the pass between,
-// which the reader stored after its read.  Tags are epoch * 8192 + pass + 1
-// (pass -1: the state at the start), the epoch counted up by every launch, so
-// no packet of an earlier launch can match.
+// which the reader stored after its read.  Tags are (epoch + 1) * 8192 + pass +
+// 1 (pass -1: the state at the start), the epoch counted up by every launch, so
+// no packet of an earlier launch, and none of zeroed memory, can match.
 //
 // Cone angle.  Every block adds its accepted count of a sweep and its arrival
 // to one word (running totals, one word per parity of the sweep: a block adds
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         }
     int theta = L->st.theta;
     const uint32_t sweep0 = L->st.sweep;
-    const uint32_t T0 = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch) << 13;
+    const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch), T0 = (epoch + 1u) << 13;
     const Par<float> par = load_par<float>(p);
     const bool adapt = MEASURE == 0 || p.adapt_in_measure;
     __syncthreads();
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
             atomicExch(&ctl->abort, 1);
             atomicCAS(&st.error, 0, -4);  // MC_ERR_TIMEOUT
         }
-        if (blk == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(&ctl->epoch) = (T0 >> 13) + 1u;
+        if (blk == 0 && lane == 0) *reinterpret_cast<volatile uint32_t*>(&ctl->epoch) = epoch + 1u;
         return;
     }
     // ----------------------------------------------------------- the workers

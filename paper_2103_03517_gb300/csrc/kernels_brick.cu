@@ -90,11 +90,6 @@ bool brick_plan(const LatParams& p, BrickArgs* out) {
     out->div_half = make_fastdiv(std::max(1u, Lh / 2));
     out->law = p.colour_kernel == kColourRow || p.colour_kernel == kColourRowFaces ? 0 : 1;
     out->faces = p.bc[0] || p.bc[1] || p.bc[2] ? 1 : 0;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, brick_sweep_kernel<1, 1, 1, 2>, kBrickThreads, 0) !=
-            cudaSuccess ||
-        per_sm < 1)
-        return false;
     return true;
 }
 

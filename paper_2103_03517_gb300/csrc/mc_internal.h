@@ -255,7 +255,7 @@ constexpr int kSampleRecords = 16;  // records a lattice holds for launched swee
 
 // Brick sweeps (brick_pass.cuh): control words of one lattice, in device
 // memory.  Zeroed before every launch but the epoch, which the launch counts
-// up (1 at create): the abort flag; the blocks of brick_close_kernel that are
+// up: the abort flag; the blocks of brick_close_kernel that are
 // done; by the sweep's parity, running totals of the blocks done (bits 40 up)
 // and of their accepted moves.
 constexpr int kBrickMaxBlocks = 256;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 
 #include "runtime.h"
@@ -31,15 +32,25 @@ static_assert(kUsed <= kScratchBytes, "scratch layout exceeds the array");
 // Shared by every call on a device; contents persist from call to call.
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
+// Memory of the brick sweeps of calls of at least kResMinSweeps sweeps on a
+// lattice of up to kBrickSpins (64^3): control words, records, packets.  Zero at
+// load; the epoch in its control words then counts the calls.
+constexpr long long kBrickSpins = 1 << 18;
+constexpr size_t kBrickOffRecord = 256;
+constexpr size_t kBrickOffPackets = kBrickOffRecord + size_t(kMaxSamples) * kRecordWords * sizeof(long long);
+static __device__ __align__(256) unsigned char g_brick[kBrickOffPackets + 16 * size_t(kBrickSpins)];
+static_assert(sizeof(BrickCtl) <= kBrickOffRecord && kBrickOffPackets % 256 == 0, "brick memory layout");
+
 // Device address of g_scratch in the current device's context (in host code
 // the name is only a stand-in).  Looked up on every call: the lookup
 // allocates nothing and is cheap once the module is loaded, and an address
 // kept from an earlier context would dangle after cudaDeviceReset.  The
 // first call on a device loads the module, so it belongs before any stream
 // capture.
-int scratch_address(char** out) {
+template <typename T>
+int scratch_address(const T& array, char** out) {
     void* p = nullptr;
-    const cudaError_t e = cudaGetSymbolAddress(&p, g_scratch);
+    const cudaError_t e = cudaGetSymbolAddress(&p, array);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(no-allocation scratch)");
     *out = static_cast<char*>(p);
     return MC_OK;
@@ -71,7 +82,7 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     if (n_sweeps == 0) return MC_OK;
 
     char* base = nullptr;
-    rc = scratch_address(&base);
+    rc = scratch_address(g_scratch, &base);
     if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
@@ -111,18 +122,20 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     host.st.theta = *theta_deg;
     host.st.sweep = uint32_t(first_sweep);
 
+    // everything before the ring in one copy
     LatDev* d_lat = reinterpret_cast<LatDev*>(base + kOffLat);
     const uint32_t starts[4] = {0, p.nblocks_site, 0, p.nblocks_pair};
-    float cone[181];
+    alignas(16) char image[kOffRing] = {};
+    std::memcpy(image + kOffLat, &host, sizeof host);
+    std::memcpy(image + kOffLats, &d_lat, sizeof d_lat);
+    std::memcpy(image + kOffStartSite, starts, 2 * sizeof(uint32_t));
+    std::memcpy(image + kOffStartPair, starts + 2, 2 * sizeof(uint32_t));
+    float* cone = reinterpret_cast<float*>(image + kOffCone);
     for (int deg = 0; deg <= 180; ++deg) {
         const double h = std::sin((double)deg * (M_PI / 360.0));
         cone[deg] = (float)(2.0 * (h * h));
     }
-    cudaError_t e = cudaMemcpyAsync(d_lat, &host, sizeof host, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffLats, &d_lat, sizeof d_lat, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffStartSite, starts, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffStartPair, starts + 2, 2 * sizeof(uint32_t), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(base + kOffCone, cone, sizeof cone, cudaMemcpyHostToDevice, s);
+    cudaError_t e = cudaMemcpyAsync(base, image, sizeof image, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "no-allocation scratch set-up");
 
     LaunchSet ls;
@@ -134,6 +147,20 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     ls.sample_level = 2;
     ls.col[p.colour_kernel] = ls.all;
     ls.nt_col[p.colour_kernel] = ls.nt_all;
+    BrickArgs brick{};
+    if (n_sweeps >= kResMinSweeps && p.N <= kBrickSpins && brick_plan(p, &brick)) {
+        char* mem = nullptr;
+        rc = scratch_address(g_brick, &mem);
+        if (rc) return rc;
+        brick.lat = d_lat;
+        brick.ctl = reinterpret_cast<BrickCtl*>(mem);
+        brick.record = reinterpret_cast<long long*>(mem + kBrickOffRecord);
+        brick.packets = mem + kBrickOffPackets;
+        brick.key0 = p.key0;
+        brick.key1 = p.key1;
+        ls.brick = &brick;
+        ls.brick_lh = uint32_t(p.Lh);
+    }
     rc = enqueue_sweeps(kernels_f32(), ls, base + kOffCone, n_sweeps, samples ? 1 : 0, false, s, nullptr);
     if (rc) return rc;
     if (samples) {
@@ -141,10 +168,14 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
                             cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return cuda_fail(e, "copy of the samples");
     }
-    int theta = 0;
-    e = cudaMemcpyAsync(&theta, &d_lat->st.theta, sizeof theta, cudaMemcpyDeviceToHost, s);
+    // theta, the sweep counter and the device error, adjacent words of the state
+    static_assert(offsetof(LatState, error) == offsetof(LatState, theta) + 8, "one copy reads both");
+    int state[3] = {0, 0, 0};
+    e = cudaMemcpyAsync(state, &d_lat->st.theta, sizeof state, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "no-allocation sweep");
+    if (state[2]) return fail(state[2], "device reported error %d", state[2]);
+    const int theta = state[0];
     *theta_deg = theta;
     return MC_OK;
 }

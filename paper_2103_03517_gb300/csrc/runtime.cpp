@@ -805,15 +805,12 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
         cudaGetLastError();
         return false;
     }
-    // zero, so that no packet of uninitialised memory carries a tag; epoch 1
-    const uint32_t first = 1;
-    BrickCtl* ctl = reinterpret_cast<BrickCtl*>(m);
-    if (cudaMemsetAsync(m, 0, b->bytes, s) != cudaSuccess ||
-        cudaMemcpyAsync(&ctl->epoch, &first, sizeof first, cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    // zero, so that no packet of uninitialised memory carries a tag
+    if (cudaMemsetAsync(m, 0, b->bytes, s) != cudaSuccess) {
         cudaFree(m);
         return false;
     }
-    b->ctl = ctl;
+    b->ctl = reinterpret_cast<BrickCtl*>(m);
     b->record = reinterpret_cast<long long*>(m + align256(sizeof(BrickCtl)));
     b->packets = m + align256(sizeof(BrickCtl)) + align256(kBrickRecordBytes);
     return true;
@@ -922,6 +919,8 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     };
     bool rest_any = ls.nt_row_rest != 0;
     for (int c = 0; c < kColourKinds; ++c) rest_any = rest_any || (c != kColourRow && ls.nt_col[c]);
+    bool row_any = false;  // lattices whose samples sample_close forms
+    for (int c = kColourRow; c < kColourKinds; ++c) row_any = row_any || ls.nt_col[c];
     bool red_field_ready = false;  // the next constrained sweep's red field is stored
     for (int i = 0; i < n; ++i) {
         // wavefront lattices sweep two at a time, spins -> spins_alt -> spins,
@@ -972,7 +971,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
             }
         }
-        if (!constrained && measure && k.sample_close && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
+        if (!constrained && measure && row_any && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
             k.sample_close(ls.all, s);
     }
     if (launch_err != cudaSuccess) return cuda_fail(launch_err, "row kernel launch");
