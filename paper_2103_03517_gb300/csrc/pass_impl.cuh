@@ -16,7 +16,7 @@ constexpr bool kIsF64 = std::is_same<R, double>::value;
 template <typename R>
 struct Par {
     R J, Ku, e[3], Kc, H[3], T;
-    R beta2;  // FP32: -log2(e) / T (unused in FP64)
+    R beta2;  // -log2(e) / T in FP32 (FP64: for boltzmann_filter)
     R Rm[9];
 };
 
@@ -25,7 +25,7 @@ __device__ __forceinline__ Par<R> load_par(const LatParams& p) {
     Par<R> q;
     if constexpr (kIsF64<R>) {
         q.J = p.J; q.Ku = p.Ku; q.Kc = p.Kc; q.T = p.T;
-        q.beta2 = 0.0;
+        q.beta2 = p.fBeta2;
         for (int a = 0; a < 3; ++a) { q.e[a] = p.e[a]; q.H[a] = p.H[a]; }
         for (int a = 0; a < 9; ++a) q.Rm[a] = p.R[a];
     } else {
@@ -344,9 +344,31 @@ __device__ __forceinline__ R boltzmann(R dE, const Par<R>& par) {
     else return exp2f(dE * par.beta2);
 }
 
+// FP64: P < f exp(-dE/T) decided in FP32 where FP32 can decide it: 1 yes, 0 no,
+// -1 too close to call (or out of FP32's range) and left to the exact test, so
+// that the decision is the exact test's in every case.  f > 0 is a factor given
+// to 1e-6.  With e = dE and b = -log2(e)/T rounded to FP32, x = e b is
+// off by at most 3 2^-24 |x|, so 2^x by 1.3e-7 |x| relative, exp2f by 2 ulp, and
+// P's rounding by 2^-24; the margin is above their sum.  An exact test costs
+// about 45 FP64 instructions (a division and the degree-13 polynomial) on a unit
+// that takes 64 cycles for a warp's; about one in 10^5 is needed.
+__device__ __forceinline__ int boltzmann_filter(double dE, float b, double P, float f = 1.0f) {
+    const float e = float(dE);
+    if (!(fabsf(e) < 1e30f && b > -1e30f && f > 1e-30f && f < 1e30f)) return -1;
+    const float x = e * b;
+    const float y = f * exp2f(x), tol = 4e-6f + 4e-7f * fabsf(x), p = float(P);
+    if (p < y * (1.0f - tol)) return 1;
+    if (p > y * (1.0f + tol)) return 0;
+    return -1;
+}
+
 template <typename R>
 __device__ __forceinline__ bool metropolis(R dE, const Par<R>& par, R P) {
     if (dE <= R(0)) return true;
+    if constexpr (kIsF64<R>) {
+        const int d = boltzmann_filter(dE, float(par.beta2), P);
+        if (d >= 0) return d != 0;
+    }
     return P < boltzmann(dE, par);
 }
 
@@ -399,6 +421,28 @@ __device__ __forceinline__ void add_site(Sums<R>& s, V3<R> S, V3<R> e, bool need
     }
 }
 
+// The warp's sums of NS <= 16 FP64 values, sum i on lane i: pairs of lanes 16,
+// 8, 4, 2 and 1 apart are added in turn, the lanes of a pair sharing the values
+// between them, so that 16 additions do what a butterfly of every value takes 5
+// NS for, and in the same order (the same bits).
+template <int NS>
+__device__ __forceinline__ double warp_sums_f64(const double* in, int lane) {
+    double v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = i < NS ? in[i] : 0.0;
+#pragma unroll
+    for (int o = 16, h = 8; h > 0; o >>= 1, h >>= 1) {
+        const bool up = lane & o;  // this lane keeps the upper half of its values
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double mine = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+            v[i] = mine + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    const double t = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return __shfl_sync(0xffffffffu, t, (2 * lane) & 31);
+}
+
 // ------------------------------------------------------------------------
 // Measurement sums of one warp tile as fixed point on lane i for sum i.
 // FP64: reduced across the warp in a fixed butterfly order, then rounded at
@@ -412,15 +456,7 @@ __device__ __forceinline__ void add_site(Sums<R>& s, V3<R> S, V3<R> e, bool need
 template <typename R, int NS = kNumSums>
 __device__ __forceinline__ long long warp_tile_fix(const Sums<R>& s, int lane) {
     if constexpr (kIsF64<R>) {
-        R mine = R(0);
-#pragma unroll
-        for (int i = 0; i < NS; ++i) {
-            R v = s.v[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == i) mine = v;
-        }
-        return __double2ll_rn(mine * kFixScale);
+        return __double2ll_rn(warp_sums_f64<NS>(s.v, lane) * kFixScale);
     } else {
         static_assert(kSitesPerThreadF32 <= 2, "a lane's FP32 sample part must stay below 16");
         int mine = 0;
@@ -1148,12 +1184,11 @@ __device__ __forceinline__ unsigned pair_move_with(const LatParams& p, const Par
     R xnj = sqrt(t);
     if (hj.x < R(0)) xnj = -xnj;
     bool ok;
-    R rM;
+    R rM = R(0);
+    double MLn = 0.0;
     if constexpr (kIsF64<R>) {
-        const double MLn = ML + hni.x + xnj - hi.x - hj.x;
+        MLn = ML + hni.x + xnj - hi.x - hj.x;
         ok = MLn > 0.0;
-        const double ratio = MLn / ML;
-        rM = ratio * ratio;
     } else {
         // FP32 spins: the change of M_L is evaluated in FP32 and applied to
         // the FP64 M_L as (1 + delta / M_L)^2.
@@ -1170,10 +1205,22 @@ __device__ __forceinline__ unsigned pair_move_with(const LatParams& p, const Par
     const R dEi = delta_e(par, Si, Sni, h_i, easy_axis(p, par, colour, qi));
     const R dEj = delta_e(par, Sj, Snj, h_j, easy_axis(p, par, colour, qj));
     const R dE = dEi + dEj;
-    R r = rM;
-    r = r * (fabs(hj.x) / fabs(xnj));
-    r = r * boltzmann(dE, par);
-    if (!(P < r)) return 0;
+    int decided = -1;
+    if constexpr (kIsF64<R>) {  // the three divisions and the exponential only where FP32 cannot tell
+        const float fr = float(MLn) / float(ML);
+        decided = boltzmann_filter(dE, float(par.beta2), P, fr * fr * (float(fabs(hj.x)) / float(fabs(xnj))));
+    }
+    if (decided == 0) return 0;
+    if (decided < 0) {
+        if constexpr (kIsF64<R>) {
+            const double ratio = MLn / ML;
+            rM = ratio * ratio;
+        }
+        R r = rM;
+        r = r * (fabs(hj.x) / fabs(xnj));
+        r = r * boltzmann(dE, par);
+        if (!(P < r)) return 0;
+    }
     store_spin(s, p.stride, set, qi, Sni);
     store_spin(s, p.stride, set, qj, Snj);
     own4[qi] = Spin4<R>{Sni.x, Sni.y, Sni.z, R(0)};

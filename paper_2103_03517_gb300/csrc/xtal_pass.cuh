@@ -247,15 +247,7 @@ __global__ void __launch_bounds__(kBlock) xtal_sample_kernel(const __grid_consta
             sums.v[kSumEx] = xtal_dot(S, h);
         }
         if constexpr (kIsF64<R>) {
-            R mine = R(0);
-#pragma unroll
-            for (int i = 0; i < NS; ++i) {
-                R v = sums.v[i];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == i) mine = v;
-            }
-            fix += __double2ll_rn(mine * kFixScale);
+            fix += __double2ll_rn(warp_sums_f64<NS>(sums.v, lane) * kFixScale);
         } else {
             fix += warp_tile_fix<R, NS>(sums, lane);  // per-lane fixed point, integer warp sums
         }
