@@ -88,6 +88,8 @@ struct KernelSet {
     void (*grain_sample)(LatDev* L, uint32_t ntiles, int n_grains, cudaStream_t s);
     // Slice sums for the profile of one lattice.
     void (*profile)(LatDev* d, uint32_t Lh, uint32_t rows, cudaStream_t s);
+    // The spins of a new lattice p (host copy): all along v, or a wall along x.
+    void (*init_spins)(const LatParams& p, int wall, const double v[3], cudaStream_t s);
     // The samples of the measured sweeps of row-kernel lattices since the last
     // call (at most kSampleRecords), of every lattice of g.  Null in the FP64
     // set.

@@ -375,7 +375,7 @@ cudaError_t slab_close_all(LatDev* const* lats, int n, int measure, cudaStream_t
 const KernelSet& kernels_f32() {
     static const KernelSet k{colour_pass, row_pass,    pair_pass,   sweep_end,         pair_field,
                              ml_reset,    mlong,       measure,     row_sample,        grain_sample,
-                             profile,     sample_close, "f32",
+                             profile,     init_spins,  sample_close, "f32",
                              wave_sweep,  wave_blocks, slab_export,       slab_close,   slab_halo,
                              slab_close_all, resident_sweeps, resident_plan};
     return k;

@@ -59,6 +59,12 @@ void measure(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     measure_kernel<R, V><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles);
 }
 
+void init_spins(const LatParams& p, int wall, const double v[3], cudaStream_t s) {
+    static const uint32_t cap = resident_blocks(init_spins_kernel<R>);
+    const uint32_t want = (p.stride + kBlock - 1) / kBlock;
+    init_spins_kernel<R><<<want < cap ? want : cap, kBlock, 0, s>>>(p, wall, V3<R>{R(v[0]), R(v[1]), R(v[2])});
+}
+
 void grain_sample(LatDev* L, uint32_t ntiles, int n_grains, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(grain_sum_kernel<R, V>);
     const Spread sp = spread_warps(ntiles, cap);

@@ -394,17 +394,9 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     p.row_fast = row_fast(p, d->bond_mask != nullptr || d->grain_id != nullptr);
     p.colour_kernel = colour_kernel(p, d->bond_mask != nullptr || d->grain_id != nullptr, d->kernel_path);
     p.row_lanes = p.Lh / 2 < 32 ? (p.Lh / 2 > 0 ? p.Lh / 2 : 1) : 32;
-    long long pinned = 0;
-    for (int z = 0; z < p.Lz; ++z)
-        for (int y = 0; y < p.Ly; ++y)
-            for (int x = 0; x < p.Lx; ++x) {
-                const int c[3] = {x, y, z};
-                const int L[3] = {p.Lx, p.Ly, p.Lz};
-                bool pin = false;
-                for (int a = 0; a < 3; ++a) pin |= p.bc[a] == MC_PINNED && (c[a] == 0 || c[a] == L[a] - 1);
-                pinned += pin;
-            }
-    p.n_mov = p.N - pinned;
+    long long moving = 1;  // sites off every pinned plane
+    for (int a = 0; a < 3; ++a) moving *= p.bc[a] == MC_PINNED ? std::max(d->dims[a] - 2, 0) : d->dims[a];
+    p.n_mov = moving * p.nsub;
     p.adapt_in_measure = d->adapt_in_measure;
     p.sample_torque = d->sample_torque ? 1 : 0;
     p.key0 = uint32_t(d->seed);
@@ -533,23 +525,6 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     }
 
     trace("create: allocated");
-    // initial state
-    std::vector<double> xyz(size_t(p.N) * 3);
-    for (long long i = 0; i < p.N; ++i) {
-        if (d->init == MC_INIT_WALL) {
-            const int x = int((i / p.nsub) % p.Lx);
-            xyz[3 * i] = 0; xyz[3 * i + 1] = 0; xyz[3 * i + 2] = x < p.Lx / 2 ? 1.0 : -1.0;
-        } else {
-            const double n = std::sqrt(d->init_dir[0] * d->init_dir[0] + d->init_dir[1] * d->init_dir[1] +
-                                       d->init_dir[2] * d->init_dir[2]);
-            for (int a = 0; a < 3; ++a) xyz[3 * i + a] = d->init_dir[a] / n;
-        }
-    }
-    std::vector<char> hs(size_t(p.nsub) * 6 * size_t(p.stride) * rs, 0);
-    if (rs == 8) to_device_layout(p, xyz.data(), reinterpret_cast<double*>(hs.data()));
-    else to_device_layout(p, xyz.data(), reinterpret_cast<float*>(hs.data()));
-
-    trace("create: host layout built");
     LatDev init;
     std::memset(&init, 0, sizeof init);
     init.st.theta = d->theta0_deg;
@@ -563,7 +538,14 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     set_float_params(p);
     init.p = p;
     up(h->d_lat, &init, sizeof init);
-    up(p.spins, hs.data(), hs.size());
+    if (rc == MC_OK) {
+        const double* v = d->init_dir;
+        const double n = std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        const double dir[3] = {v[0] / n, v[1] / n, v[2] / n};
+        kernel_set(d->precision).init_spins(p, d->init == MC_INIT_WALL ? 1 : 0, dir, h->stream);
+        const cudaError_t ee = cudaGetLastError();
+        if (ee != cudaSuccess) rc = cuda_fail(ee, "initial spins");
+    }
     if (!hb.empty()) up(const_cast<uint8_t*>(p.bonds), hb.data(), hb.size());
     if (!hg.empty()) {
         up(const_cast<int32_t*>(p.grain), hg.data(), hg.size() * 4);
