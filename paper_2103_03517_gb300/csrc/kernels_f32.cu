@@ -43,24 +43,11 @@ constexpr int V = kSitesPerThreadF32;
 template <int B, int MEASURE, int GEN, int LAW, int TURNS = 0>
 cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>);
-    // programmatic serialisation: the pass starts its blocks while the
-    // previous launch drains and waits inside the kernel (griddepcontrol)
-    cudaLaunchConfig_t cfg = {};
     const Spread sp = spread_warps(ntiles, cap);
-    cfg.gridDim = dim3(sp.blocks);
-    cfg.blockDim = dim3(uint32_t(sp.threads));
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, g, ntiles, cone, colour);
+    const cudaError_t e =
+        launch_chained(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, sp.blocks, sp.threads, s, g, ntiles, cone, colour);
     if (e != cudaSuccess || colour != 1) return e;  // the sweep's end
-    cudaLaunchConfig_t cc = cfg;
-    cc.gridDim = dim3(uint32_t(g.n));
-    cc.blockDim = dim3(32);
-    return cudaLaunchKernelEx(&cc, row_close_kernel, g, MEASURE > 0 ? 1 : 0);
+    return launch_chained(row_close_kernel, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
 }
 
 // launch shape 0: the default blocks per SM of the instance (B0 of a pass
@@ -111,7 +98,8 @@ void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     constexpr int B = GEN == 2 ? MINB_FILM_M : (GEN == 1 ? MINB_FACES_M : MINB);
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
     const Spread sp = spread_warps(ntiles, cap);
-    row_pass_kernel<B, 2, GEN, 0><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, nullptr, GEN ? 1 : 0);
+    launch_chained_if(sp.blocks < cap, row_pass_kernel<B, 2, GEN, 0>, sp.blocks, sp.threads, s, g, ntiles,
+                      static_cast<const R*>(nullptr), GEN ? 1 : 0);
 }
 
 void row_sample(const GroupArgs& g, uint32_t ntiles, int gen, cudaStream_t s) {
@@ -124,8 +112,8 @@ template <bool LEADER, int C, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int N
 void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, C, LEADER, NT>, NT);
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap, NT);
-    pair_pass_kernel<R, B, C, LEADER, NT><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, static_cast<const R*>(cone),
-                                                                           colour, sub);
+    launch_chained_if(sp.blocks < cap, pair_pass_kernel<R, B, C, LEADER, NT>, sp.blocks, sp.threads, s, g, ntiles,
+                      static_cast<const R*>(cone), colour, sub);
 }
 
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step, and the

@@ -19,7 +19,7 @@ template <int C>
 void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, int sub, uint32_t cap,
                  cudaStream_t s) {
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
-    pair_pass_kernel<R, 1, C, false><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, cone, colour, sub);
+    launch_chained_if(sp.blocks < cap, pair_pass_kernel<R, 1, C, false>, sp.blocks, sp.threads, s, g, ntiles, cone, colour, sub);
 }
 
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step; FP64

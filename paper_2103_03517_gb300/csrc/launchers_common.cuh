@@ -24,13 +24,16 @@ void colour_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
 }
 
 void sweep_end(const GroupArgs& g, cudaStream_t s) {
-    sweep_end_kernel<R><<<(g.n + kBlock - 1) / kBlock, kBlock, 0, s>>>(g);
+    launch_chained(sweep_end_kernel<R>, uint32_t(g.n + kBlock - 1) / kBlock, kBlock, s, g);
 }
 
+// The constrained sweeps' launches are chained where they do not fill the GPU
+// (8^3 ... 32^3 alone 10% faster a sweep); a full one's blocks, started early,
+// only take room from the launch that they wait for (80 x 64^3 1.2% slower).
 template <int C>
 void pair_field_t(const GroupArgs& g, uint32_t ntiles, int colour, uint32_t cap, cudaStream_t s) {
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
-    pair_field_kernel<R, V, C><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, colour);
+    launch_chained_if(sp.blocks < cap, pair_field_kernel<R, V, C>, sp.blocks, sp.threads, s, g, ntiles, colour);
 }
 
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step

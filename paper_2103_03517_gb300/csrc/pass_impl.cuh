@@ -1049,6 +1049,8 @@ __global__ void __launch_bounds__(kBlock) mlong_kernel(GroupArgs g, uint32_t nti
 // thread per lattice): cone adaptation, M_L carried, the sweep counter.
 template <typename R>
 __global__ void sweep_end_kernel(GroupArgs g) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int l = int(blockIdx.x * blockDim.x + threadIdx.x);
     if (l >= g.n) return;
     LatDev* L = g.lats[l];
@@ -1264,6 +1266,8 @@ constexpr uint32_t kLeaderRing = 128;
 template <typename R, int MINB, int CHUNK, bool LEADER, int NT = kBlock>
 __global__ void __launch_bounds__(NT, MINB) pair_pass_kernel(GroupArgs g, uint32_t ntiles,
                                                              const R* __restrict__ cone, int colour, int sub) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int lane = int(threadIdx.x & 31);
     const uint32_t wpb = kIsF64<R> ? blockDim.x >> 5 : uint32_t(NT / 32);  // FP64: spread_warps
     const uint32_t nwarps = gridDim.x * wpb;
@@ -1460,6 +1464,8 @@ __device__ __forceinline__ void field_tile_periodic(const LatParams& p, const Sp
 
 template <typename R, int V, int CHUNK>
 __global__ void __launch_bounds__(kBlock) pair_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t wpb = kIsF64<R> ? blockDim.x >> 5 : uint32_t(kBlock / 32);  // FP64: spread_warps
     const uint32_t nwarps = gridDim.x * wpb;
     const uint32_t w = blockIdx.x * wpb + (threadIdx.x >> 5);

@@ -57,3 +57,25 @@ int tiles_per_step(uint32_t ntiles, uint32_t warps, int most) {
     if (even >= uint32_t(most)) return most;
     return even >= 2 ? 2 : 1;
 }
+
+// Launch with programmatic serialisation (chain): the kernel's blocks may start
+// while the previous launch drains; it waits for it (griddepcontrol.wait) before
+// it touches any memory.
+template <typename... K, typename... A>
+cudaError_t launch_chained_if(bool chain, void (*kernel)(K...), uint32_t blocks, int threads, cudaStream_t s, A... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(uint32_t(threads));
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, a...);
+}
+
+template <typename... K, typename... A>
+cudaError_t launch_chained(void (*kernel)(K...), uint32_t blocks, int threads, cudaStream_t s, A... a) {
+    return launch_chained_if(true, kernel, blocks, threads, s, a...);
+}

@@ -4,20 +4,10 @@
 #pragma once
 #include "spread.cuh"
 
-// With programmatic serialisation, as for the row passes.
 template <typename... K, typename... A>
 cudaError_t xtal_launch(void (*kernel)(K...), uint32_t ntiles, uint32_t cap, cudaStream_t s, A... a) {
     const Spread sp = spread_warps(ntiles, cap);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(sp.blocks);
-    cfg.blockDim = dim3(uint32_t(sp.threads));
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a...);
+    return launch_chained(kernel, sp.blocks, sp.threads, s, a...);
 }
 
 template <int TYPE, int J2>
