@@ -184,10 +184,12 @@ __device__ __forceinline__ bool brick_neighbours(const float* oth, const float4*
 
 // LAW 0: packed pairs (row kernels), 1: the general kernel's scalar law;
 // FACES: any boundaries (0: all periodic); ODD: rows of odd Lh (LAW 1);
-// MEASURE as in the row kernel.
-template <int LAW, int FACES, int ODD, int MEASURE>
+// MEASURE as in the row kernel; GROUP: the lattices of grp, each with blocks of
+// its own that know nothing of the others, instead of `one`.
+template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
 __global__ void __launch_bounds__(kBrickThreads, 1)
-    brick_sweep_kernel(const __grid_constant__ BrickArgs a, const float* __restrict__ cone) {
+    brick_sweep_kernel(const __grid_constant__ BrickArgs one, const __grid_constant__ BrickGroup grp,
+                       const float* __restrict__ cone) {
     constexpr int NS = MEASURE >= 2 ? kNumSums : kSumTux;  // sums sampled
     constexpr int NW = kBrickWarps;
     extern __shared__ __align__(16) float bsm[];
@@ -196,12 +198,23 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
     __shared__ long long cta_sums[kNumSums];   // fixed-point sample sums
     __shared__ float s_cone;                   // 1 - cos of the cone angle
     __shared__ int s_fail;
+    int lat = 0;
+    if (GROUP)
+        for (int hi = grp.n - 1; lat < hi;) {  // the last lattice whose first block is not above this one
+            const int mid = (lat + hi + 1) >> 1;
+            if (__ldg(&grp.first[mid]) <= blockIdx.x) lat = mid;
+            else hi = mid - 1;
+        }
+    const BrickArgs& a = GROUP ? grp.args[lat] : one;
+    const uint32_t key0 = a.key0, key1 = a.key1;  // launch constants of a lattice alone, and with them the round keys
+    const FastDiv div_half = a.div_half;
+    const int n_sweeps = GROUP ? grp.n_sweeps : a.n_sweeps;
     LatDev* const L = a.lat;
     const LatParams& p = L->p;
     BrickCtl* const ctl = a.ctl;
     const int tid = int(threadIdx.x), lane = tid & 31, warp = tid >> 5;
     const uint32_t Lh = uint32_t(p.Lh), Ly = uint32_t(p.Ly), Lz = uint32_t(p.Lz), stride = p.stride;
-    const uint32_t blk = blockIdx.x, G = gridDim.x;
+    const uint32_t G = a.nyc * a.nzc, blk = blockIdx.x - (GROUP ? __ldg(&grp.first[lat]) : 0u);
     float* const s = static_cast<float*>(p.spins);
     // this block's rows: a brick, or a run of rows
     uint32_t y0 = 0, ny = 1, z0 = 0, nr, r0 = 0;
@@ -298,8 +311,8 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         bool ok = true;
         long long acc = 0;
         unsigned long long before[2] = {0, 0};  // totals of the sweeps of either parity so far
-        for (int sw = 0; sw < a.n_sweeps && ok; ++sw) {
-            if (sw + 1 == a.n_sweeps && blk != 0) break;
+        for (int sw = 0; sw < n_sweeps && ok; ++sw) {
+            if (sw + 1 == n_sweeps && blk != 0) break;
             // every block's count of this sweep
             const uint32_t want = G * uint32_t(sw / 2 + 1) + uint32_t(a.inject);
             unsigned long long v = 0;
@@ -335,7 +348,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                 st.ml_lo += st.dml_lo;
                 st.dml_hi = 0;
                 st.dml_lo = 0;
-                st.sweep = sweep0 + uint32_t(a.n_sweeps);
+                st.sweep = sweep0 + uint32_t(n_sweeps);
             }
         }
         if (!ok && lane == 0) {
@@ -368,7 +381,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
     float cval = cone[theta];
     bool failed = false;
     bool alive = true;
-    for (int sw = 0; sw < a.n_sweeps && alive; ++sw) {
+    for (int sw = 0; sw < n_sweeps && alive; ++sw) {
         const uint32_t sweep = sweep0 + uint32_t(sw);
         unsigned nacc = 0;
         for (int c = 0; c < 2 && alive; ++c) {
@@ -394,7 +407,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                 uint32_t k1 = 0;
                 bool two = true;
                 if constexpr (!ODD) {
-                    const uint32_t i = fast_div(Pc, a.div_half);
+                    const uint32_t i = fast_div(Pc, div_half);
                     k = 2u * (Pc - i * (Lh >> 1));
                     e = tab[i];
                     const uint32_t xoff = (e.flags + uint32_t(c)) & 1u;
@@ -490,8 +503,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                     h = pack(hv);
                     O = pack(Ov);
                 }
-                // the key is a kernel parameter, so its round keys are launch constants
-                const uint4 w = philox(make_uint4(site0, sweep, tag_of(c, kPurposeMove), 0u), a.key0, a.key1);
+                const uint4 w = philox(make_uint4(site0, sweep, tag_of(c, kPurposeMove), 0u), key0, key1);
                 if (first) {  // the cone angle, now that everything else is at hand
                     first = false;
                     if (!mbar_wait(&tbar, uint32_t(sw - 1) & 1u) || *reinterpret_cast<volatile int*>(&s_fail)) failed = true;
@@ -620,9 +632,13 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
 // then adds those in the order of the sweeps (the additions of a sweep by
 // sweep close, so the same bits).
 template <int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(LatDev* L, BrickCtl* ctl, long long* record, int n) {
-    const LatParams& p = L->p;
-    LatState& st = L->st;
+__global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(const __grid_constant__ BrickArgs one,
+                                                                const BrickArgs* many, int n) {
+    const BrickArgs& a = many ? many[blockIdx.y] : one;
+    BrickCtl* const ctl = a.ctl;
+    long long* const record = a.record;
+    const LatParams& p = a.lat->p;
+    LatState& st = a.lat->st;
     const int lane = int(threadIdx.x & 31), w = int(blockIdx.x * WARPS + (threadIdx.x >> 5));
     if (*reinterpret_cast<volatile int*>(&ctl->abort)) return;
     const long long ring = st.ring_count;
@@ -658,6 +674,20 @@ __global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(LatDev* L, Bric
         st.moments[lane] = m;
     }
     if (lane == 0) st.ring_count = ring + n;
+}
+
+// Before a launch of several lattices: their control words (not the epochs) and
+// the records of n measured sweeps zeroed, as the memsets of a lattice alone do.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) brick_prep_kernel(const BrickArgs* many, int n) {
+    const BrickArgs& a = many[blockIdx.y];
+    const int i = int(blockIdx.x) * THREADS + int(threadIdx.x);
+    if (i < n * kRecordWords) a.record[i] = 0;
+    if (i == 0) {
+        a.ctl->abort = 0;
+        a.ctl->closed = 0;
+        a.ctl->count[0] = a.ctl->count[1] = 0;
+    }
 }
 
 }  // namespace mcgb

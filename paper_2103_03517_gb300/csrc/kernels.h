@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <vector>
+
 #include "mc_internal.h"
 
 namespace mcgb {
@@ -156,6 +158,9 @@ struct LaunchSet {
     // null; its Lh
     BrickArgs* brick = nullptr;
     uint32_t brick_lh = 0;
+    // a group whose unconstrained sweeps run as brick launches of all its
+    // lattices side by side, else null
+    struct BrickSet* brick_set = nullptr;
     int sample_level = 2;  // sample of a measured colour pass: 1 or 2 (torques)
     // a bcc / fcc / hcp lattice alone (xtal.lat, else null) and its sub-lattices
     XtalArgs xtal = {};
@@ -169,7 +174,21 @@ struct LaunchSet {
 // their shared memory.  Then n sweeps of a plan in cooperative launches of at
 // most kResMaxSweeps, measure as for colour_pass.
 bool brick_plan(const LatParams& p, BrickArgs* out);
+// The splits of several lattices swept side by side, each with blocks of its
+// own (splits only: out[i] keeps its pointers and key): the estimated us of a
+// sweep of the slowest, or 0 when they do not fit the SMs together.
+double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<BrickArgs>* out);
 cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, cudaStream_t s);
+// The same for lattices of one kernel instance (law, no faces, parity of Lh):
+// their plans and first blocks in device memory, blocks and shared memory of
+// the launch.
+struct BrickClass {
+    BrickArgs* args = nullptr;
+    uint32_t* first = nullptr;
+    int n = 0, law = 0, odd = 0;
+    uint32_t blocks = 0, smem = 0;
+};
+cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, cudaStream_t s);
 
 const KernelSet& kernels_f64();
 const KernelSet& kernels_f32();

@@ -1,6 +1,7 @@
 // kernels_brick.cu -- the brick sweeps of brick_pass.cuh: planner and launches.
 #include <algorithm>
 #include <cstddef>
+#include <vector>
 
 #include "kernels.h"
 #include "brick_pass.cuh"
@@ -8,89 +9,150 @@
 namespace mcgb {
 namespace {
 
-template <int LAW, int FACES, int ODD, int MEASURE>
-cudaError_t launch(const BrickArgs& a, const float* cone, cudaStream_t s) {
+template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
+cudaError_t launch(const BrickArgs& a, const BrickGroup& g, uint32_t blocks, uint32_t smem, const float* cone,
+                   cudaStream_t s) {
     static const bool ok = [] {
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        return cudaFuncSetAttribute(brick_sweep_kernel<LAW, FACES, ODD, MEASURE>,
+        return cudaFuncSetAttribute(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     optin - int(kResStaticSmem)) == cudaSuccess;
     }();
     if (!ok) return cudaErrorInvalidConfiguration;
     // cooperative: the launch fails rather than run with a block not resident
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.nyc * a.nzc);
+    cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kBrickThreads);
-    cfg.dynamicSmemBytes = a.smem;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, brick_sweep_kernel<LAW, FACES, ODD, MEASURE>, a, cone);
+    return cudaLaunchKernelEx(&cfg, brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>, a, g, cone);
 }
 
-template <int LAW, int FACES, int ODD>
-cudaError_t launch_m(const BrickArgs& a, const float* cone, int measure, cudaStream_t s) {
-    if (measure >= 2) return launch<LAW, FACES, ODD, 2>(a, cone, s);
-    if (measure == 1) return launch<LAW, FACES, ODD, 1>(a, cone, s);
-    return launch<LAW, FACES, ODD, 0>(a, cone, s);
+template <int LAW, int FACES, int ODD, int GROUP = 0>
+cudaError_t launch_m(const BrickArgs& a, const BrickGroup& g, uint32_t blocks, uint32_t smem, const float* cone,
+                     int measure, cudaStream_t s) {
+    if (measure >= 2) return launch<LAW, FACES, ODD, 2, GROUP>(a, g, blocks, smem, cone, s);
+    if (measure == 1) return launch<LAW, FACES, ODD, 1, GROUP>(a, g, blocks, smem, cone, s);
+    return launch<LAW, FACES, ODD, 0, GROUP>(a, g, blocks, smem, cone, s);
 }
 
 cudaError_t launch_any(const BrickArgs& a, uint32_t Lh, const float* cone, int measure, cudaStream_t s) {
-    if (a.law == 0) return a.faces ? launch_m<0, 1, 0>(a, cone, measure, s) : launch_m<0, 0, 0>(a, cone, measure, s);
-    if (Lh & 1u) return a.faces ? launch_m<1, 1, 1>(a, cone, measure, s) : launch_m<1, 0, 1>(a, cone, measure, s);
-    return a.faces ? launch_m<1, 1, 0>(a, cone, measure, s) : launch_m<1, 0, 0>(a, cone, measure, s);
+    const BrickGroup g{};
+    const uint32_t b = a.nyc * a.nzc;
+    if (a.law == 0)
+        return a.faces ? launch_m<0, 1, 0>(a, g, b, a.smem, cone, measure, s)
+                       : launch_m<0, 0, 0>(a, g, b, a.smem, cone, measure, s);
+    if (Lh & 1u)
+        return a.faces ? launch_m<1, 1, 1>(a, g, b, a.smem, cone, measure, s)
+                       : launch_m<1, 0, 1>(a, g, b, a.smem, cone, measure, s);
+    return a.faces ? launch_m<1, 1, 0>(a, g, b, a.smem, cone, measure, s)
+                   : launch_m<1, 0, 0>(a, g, b, a.smem, cone, measure, s);
+}
+
+struct Device {
+    uint32_t most, cap;  // blocks at once, shared memory of a block
+};
+
+Device device() {
+    int dev = 0, sms = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return Device{uint32_t(std::min(sms, kBrickMaxBlocks)), uint32_t(std::max(0, optin - int(kResStaticSmem)))};
+}
+
+// A split and its estimated us a pass, fitted to 8^3 ... 96^3 at 1 ... 152
+// blocks: the exchange and up to two tiles a scheduler 1.45 (one block 1.15),
+// 0.105 a tile beyond; among equals fewer rounds, face rows and blocks.
+struct Split {
+    uint32_t nyc = 0, nzc = 0, rows = 0, smem = 0;
+    double cost = 0;
+};
+
+// The best split of lattice p over exactly G blocks or fewer, for G = 1 ...
+// most (nyc = 0: none fits).
+std::vector<Split> splits(const LatParams& p, const Device& d) {
+    const uint32_t Lh = uint32_t(p.Lh), Ly = uint32_t(p.Ly), Lz = uint32_t(p.Lz);
+    std::vector<Split> best(d.most + 1);
+    auto consider = [&](uint32_t nyc, uint32_t nzc, uint32_t rows, uint32_t halo) {
+        const uint32_t smem = brick_smem_bytes(rows, Lh), G = nyc * nzc;
+        if (smem > d.cap) return;
+        const uint32_t tiles = ((rows * Lh + 1) / 2 + 31) / 32, rounds = (tiles + kBrickWarps - 1) / kBrickWarps;
+        const double cost = std::max(G > 1 ? 1.45 : 1.15, 0.3 + 0.105 * tiles) + 0.1 * rounds + 1e-3 * double(halo) +
+                            1e-3 * G;
+        if (best[G].nyc == 0 || cost < best[G].cost) best[G] = Split{nyc, nzc, rows, smem, cost};
+    };
+    if (Lh & 1u) {
+        const uint32_t pairs = (Ly * Lz + 1) / 2;
+        for (uint32_t G = 1; G <= d.most && G <= pairs; ++G) consider(G, 1, 2 * ((pairs + G - 1) / G), 0);
+    } else {
+        for (uint32_t nyc = 1; nyc <= Ly && nyc <= d.most; ++nyc)
+            for (uint32_t nzc = 1; nzc <= Lz && nyc * nzc <= d.most; ++nzc) {
+                const uint32_t by = (Ly + nyc - 1) / nyc, bz = (Lz + nzc - 1) / nzc;
+                consider(nyc, nzc, by * bz, (nyc > 1 ? 2 * bz : 0) + (nzc > 1 ? 2 * by : 0));
+            }
+    }
+    for (uint32_t G = 1; G <= d.most; ++G)
+        if (best[G - 1].nyc && (best[G].nyc == 0 || best[G - 1].cost <= best[G].cost)) best[G] = best[G - 1];
+    return best;
+}
+
+void take(const LatParams& p, const Split& b, BrickArgs* out) {
+    out->nyc = b.nyc;
+    out->nzc = b.nzc;
+    out->rows = b.rows;
+    out->smem = b.smem;
+    out->div_half = make_fastdiv(std::max(1u, uint32_t(p.Lh) / 2));
+    out->law = p.colour_kernel == kColourRow || p.colour_kernel == kColourRowFaces ? 0 : 1;
+    out->faces = p.bc[0] || p.bc[1] || p.bc[2] ? 1 : 0;
 }
 
 }  // namespace
 
 bool brick_plan(const LatParams& p, BrickArgs* out) {
-    int dev = 0, sms = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const uint32_t cap = uint32_t(std::max(0, optin - int(kResStaticSmem)));
-    const uint32_t most = uint32_t(std::min(sms, kBrickMaxBlocks));
-    const uint32_t Lh = uint32_t(p.Lh), Ly = uint32_t(p.Ly), Lz = uint32_t(p.Lz);
-    const bool odd = Lh & 1u;
-    bool found = false;
-    double best = 0;
-    auto consider = [&](uint32_t nyc, uint32_t nzc, uint32_t rows, uint32_t halo) {
-        const uint32_t smem = brick_smem_bytes(rows, Lh), G = nyc * nzc;
-        if (smem > cap) return;
-        const uint32_t tiles = ((rows * Lh + 1) / 2 + 31) / 32, rounds = (tiles + kBrickWarps - 1) / kBrickWarps;
-        // us a pass, fitted to 8^3 ... 96^3 at 1 ... 152 blocks: the exchange
-        // and up to two tiles a scheduler 1.45 (one block 1.15), 0.105 a tile
-        // beyond; among equals fewer rounds, face rows and blocks
-        const double cost = std::max(G > 1 ? 1.45 : 1.15, 0.3 + 0.105 * tiles) + 0.1 * rounds + 1e-3 * double(halo) +
-                            1e-3 * G;
-        if (found && cost >= best) return;
-        found = true;
-        best = cost;
-        out->nyc = nyc;
-        out->nzc = nzc;
-        out->rows = rows;
-        out->smem = smem;
-    };
-    if (odd) {
-        const uint32_t pairs = (Ly * Lz + 1) / 2;
-        for (uint32_t G = 1; G <= most && G <= pairs; ++G) consider(G, 1, 2 * ((pairs + G - 1) / G), 0);
-    } else {
-        for (uint32_t nyc = 1; nyc <= Ly && nyc <= most; ++nyc)
-            for (uint32_t nzc = 1; nzc <= Lz && nyc * nzc <= most; ++nzc) {
-                const uint32_t by = (Ly + nyc - 1) / nyc, bz = (Lz + nzc - 1) / nzc;
-                consider(nyc, nzc, by * bz, (nyc > 1 ? 2 * bz : 0) + (nzc > 1 ? 2 * by : 0));
-            }
-    }
-    if (!found) return false;
-    out->div_half = make_fastdiv(std::max(1u, Lh / 2));
-    out->law = p.colour_kernel == kColourRow || p.colour_kernel == kColourRowFaces ? 0 : 1;
-    out->faces = p.bc[0] || p.bc[1] || p.bc[2] ? 1 : 0;
+    const std::vector<Split> best = splits(p, device());
+    if (best.back().nyc == 0) return false;
+    take(p, best.back(), out);
     return true;
+}
+
+double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<BrickArgs>* out) {
+    const Device d = device();
+    const size_t n = lats.size();
+    if (n > d.most) return 0.0;
+    std::vector<std::vector<Split>> s;
+    std::vector<uint32_t> G(n);
+    uint32_t total = 0;
+    for (size_t i = 0; i < n; ++i) {
+        s.push_back(splits(*lats[i], d));
+        for (G[i] = 1; G[i] <= d.most && s[i][G[i]].nyc == 0;) ++G[i];
+        if (G[i] > d.most) return 0.0;
+        total += G[i];
+    }
+    if (total > d.most) return 0.0;
+    for (;;) {  // more blocks for the slowest, while they make it faster and there are any
+        size_t i = 0;
+        for (size_t j = 1; j < n; ++j)
+            if (s[j][G[j]].cost > s[i][G[i]].cost) i = j;
+        uint32_t g = G[i] + 1;
+        while (g <= d.most && s[i][g].cost >= s[i][G[i]].cost) ++g;
+        if (g > d.most || total + (g - G[i]) > d.most) break;
+        total += g - G[i];
+        G[i] = g;
+    }
+    double slowest = 0.0;
+    for (size_t i = 0; i < n; ++i) {
+        take(*lats[i], s[i][G[i]], &(*out)[i]);
+        slowest = std::max(slowest, s[i][G[i]].cost);
+    }
+    return 2.0 * slowest;
 }
 
 cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, cudaStream_t s) {
@@ -102,11 +164,34 @@ cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int 
             e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kRecordWords * sizeof(long long), s);
         if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
         if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a.lat, a.ctl, a.record, a.n_sweeps);
+            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, nullptr, a.n_sweeps);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) return e;
         done += a.n_sweeps;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, cudaStream_t s) {
+    const float* c32 = static_cast<const float*>(cone);
+    for (int done = 0; done < n;) {
+        const int m = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
+        const BrickGroup g{c.args, c.first, c.n, m};
+        const BrickArgs none{};
+        const int words = (measure ? m : 0) * kRecordWords;
+        brick_prep_kernel<256><<<dim3(uint32_t(words / 256 + 1), uint32_t(c.n)), 256, 0, s>>>(c.args, measure ? m : 0);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = c.law == 0 ? launch_m<0, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s)
+                : c.odd    ? launch_m<1, 0, 1, 1>(none, g, c.blocks, c.smem, c32, measure, s)
+                           : launch_m<1, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s);
+        if (e == cudaSuccess && measure) {
+            brick_close_kernel<4><<<dim3(uint32_t(m + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, c.args, m);
+            e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) return e;
+        done += m;
     }
     return cudaSuccess;
 }

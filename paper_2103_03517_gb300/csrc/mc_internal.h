@@ -285,4 +285,13 @@ struct BrickArgs {
     uint32_t key0, key1;  // the lattice's Philox key, a launch constant
 };
 
+// Brick sweeps of several lattices of one kernel instance in one launch: lattice
+// i has the blocks [first[i], first[i + 1]).
+struct BrickGroup {
+    const BrickArgs* args;
+    const uint32_t* first;
+    int n;
+    int n_sweeps;
+};
+
 }  // namespace mcgb

@@ -798,6 +798,68 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
     return true;
 }
 
+// The brick set of a group, on first use; false when it cannot be had.
+static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
+    if (b->failed) return false;
+    if (b->mem) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    b->failed = true;
+    const size_t n = b->lats.size();
+    std::vector<std::vector<BrickArgs>> args(3);  // by kernel instance: LAW 0, LAW 1, LAW 1 with odd rows
+    for (size_t i = 0; i < n; ++i) {
+        BrickArgs* own = b->lats[i]->brick;
+        if (!brick_memory(own, s)) return false;
+        BrickArgs a = *own;
+        const BrickArgs& plan = b->plans[i];
+        a.nyc = plan.nyc;
+        a.nzc = plan.nzc;
+        a.rows = plan.rows;
+        a.smem = plan.smem;
+        args[a.law == 0 ? 0 : 1 + b->lats[i]->hp.Lh % 2].push_back(a);
+    }
+    std::vector<char> host;
+    std::vector<size_t> at;
+    for (auto& v : args) {
+        at.push_back(host.size());
+        host.resize(host.size() + align256(v.size() * sizeof(BrickArgs)) + align256((v.size() + 1) * sizeof(uint32_t)));
+    }
+    void* mem = nullptr;
+    if (cudaMalloc(&mem, host.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    for (int k = 0; k < 3; ++k) {
+        const std::vector<BrickArgs>& v = args[k];
+        if (v.empty()) continue;
+        BrickClass c;
+        const size_t first = at[k] + align256(v.size() * sizeof(BrickArgs));
+        c.args = reinterpret_cast<BrickArgs*>(static_cast<char*>(mem) + at[k]);
+        c.first = reinterpret_cast<uint32_t*>(static_cast<char*>(mem) + first);
+        c.n = int(v.size());
+        c.law = k == 0 ? 0 : 1;
+        c.odd = k == 2;
+        uint32_t* f = reinterpret_cast<uint32_t*>(host.data() + first);
+        for (size_t i = 0; i < v.size(); ++i) {
+            std::memcpy(host.data() + at[k] + i * sizeof(BrickArgs), &v[i], sizeof(BrickArgs));
+            f[i] = c.blocks;
+            c.blocks += v[i].nyc * v[i].nzc;
+            c.smem = std::max(c.smem, v[i].smem);
+        }
+        f[v.size()] = c.blocks;
+        b->classes.push_back(c);
+    }
+    if (cudaMemcpyAsync(mem, host.data(), host.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess) {
+        cudaFree(mem);
+        b->classes.clear();
+        return false;
+    }
+    b->mem = mem;
+    b->failed = false;
+    return true;
+}
+
 // Enqueue n sweeps of the lattices of a launch set; with events != nullptr
 // every colour pass or pair pass is bracketed by a pair of events.
 int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, int n, int measure, bool constrained,
@@ -836,6 +898,18 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
             timed_kind(kTimedResident, [&] {
                 e = brick_sweeps(*ls.brick, ls.brick_lh, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
             });
+        if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
+        return MC_OK;
+    }
+    if (!constrained && ls.brick_set && n >= kResMinSweeps && brick_set_ready(ls.brick_set, s)) {
+        cudaError_t e = cudaSuccess;
+        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
+        for (int done = 0; done < n; done += most)
+            for (const BrickClass& c : ls.brick_set->classes)
+                timed_kind(kTimedResident, [&] {
+                    if (e == cudaSuccess)
+                        e = brick_group_sweeps(c, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
+                });
         if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
         return MC_OK;
     }
@@ -966,7 +1040,7 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
                bool constrained, cudaStream_t s) {
     const KernelSet& k = kernel_set(precision);
     // resident sweeps run many to a launch: nothing to capture
-    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && brick_memory(ls.brick, s))))
+    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && brick_memory(ls.brick, s)) || (ls.brick_set && brick_set_ready(ls.brick_set, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
     const int reps = n / kGraphSweeps;
     if (reps > 0) {

@@ -10,6 +10,8 @@
 #include "mc.h"
 #include "mc_internal.h"
 
+struct mc_lattice;
+
 namespace mcgb {
 // An NVTX range for the scope of the object (a no-op without a profiler).
 struct NvtxRange {
@@ -34,6 +36,25 @@ constexpr int kResMinSweeps = 3;
 constexpr long long kResGroupMinSpins = 1ll << 21;
 struct SweepGraphs {
     cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+};
+}  // namespace mcgb
+
+namespace mcgb {
+// The brick sweeps of a group's lattices side by side: made by the group's first
+// such call (the lattices' brick memory, then their plans on the device), or
+// given up then.
+struct BrickSet {
+    std::vector<mc_lattice*> lats;
+    std::vector<BrickArgs> plans;  // splits, one per lattice
+    std::vector<BrickClass> classes;
+    void* mem = nullptr;           // the classes' device arrays
+    bool failed = false;
+    BrickSet() = default;
+    BrickSet(const BrickSet&) = delete;
+    BrickSet& operator=(const BrickSet&) = delete;
+    ~BrickSet() {
+        if (mem) cudaFree(mem);
+    }
 };
 }  // namespace mcgb
 

@@ -79,6 +79,44 @@ def test_brick_samples_without_torques_and_with_a_fixed_cone(dims):
     _assert_same(_run(dims, kw, spins, plan, mc.MC_PATH_AUTO), _run(dims, kw, spins, plan, mc.MC_PATH_ROW), dims)
 
 
+@pytest.mark.parametrize("sizes", [(16, 16), (8, 16, 32, 64), (12, 18, 24, 50, 64), (2, 4), (32,) * 20])
+def test_group_of_small_lattices_side_by_side(sizes):
+    """A group whose lattices fit the SMs together: brick launches, one per
+    kernel instance, free and measured, mixed with constrained sweeps and calls
+    too short for them; every lattice equals the one swept alone by launches."""
+    def make(i, path):
+        L = sizes[i]
+        h = mc.mc_create_ex(mc.make_desc((L, L, L), K_u=0.03, T=0.5 + 0.05 * i, seed=30 + i, ring_capacity=16,
+                                         kernel_path=path, init_dir=(0.1 * (i % 5), 0.0, 1.0)))
+        mc.mc_set_spins(h, workloads.perturbed_spins(L ** 3, i, 0.3))
+        return h
+
+    def read(h, L):
+        return mc.mc_get_spins(h, L ** 3), mc.mc_get_theta(h), mc.mc_measure(h).asdict(), mc.mc_samples(h, 16)
+
+    n = len(sizes)
+    hs = [make(i, mc.MC_PATH_AUTO) for i in range(n)]
+    g = mc.mc_group_create(hs)
+    _, kinds = mc.mc_group_time_kernels(g, 5)
+    assert kinds[3] >= 1 and kinds[1] == 0, kinds
+    mc.mc_group_sweep(g, 4, True)
+    mc.mc_group_constrained_sweep(g, [10.0] * n, [0.0] * n, 3, True)
+    mc.mc_group_sweep(g, 2, True)
+    mc.mc_group_sweep(g, 20, True)
+    mc.mc_group_sweep(g, 18)
+    mc.mc_group_destroy(g)
+    for i, h in enumerate(hs):
+        one = make(i, mc.MC_PATH_ROW)
+        mc.mc_sweep(one, 5)
+        mc.mc_sweep(one, 4, True)
+        mc.mc_constrained_sweep(one, 10.0, 0.0, 3, True)
+        mc.mc_sweep(one, 22, True)
+        mc.mc_sweep(one, 18)
+        _assert_same(read(h, sizes[i]), read(one, sizes[i]), (i, sizes[i]))
+        mc.mc_destroy(one)
+        mc.mc_destroy(h)
+
+
 def test_brick_run_longer_than_one_launch():
     """2050 sweeps take two launches; tags and epochs go on across them."""
     dims = (16, 8, 12)
