@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         LatState& st = L->st;
         bool ok = true;
         long long acc = 0;
-        unsigned long long before[2] = {0, 0};  // totals of the sweeps of either parity so far
+        unsigned long long even = 0, odd = 0;  // totals of the sweeps of either parity so far
         for (int sw = 0; sw < n_sweeps && ok; ++sw) {
             if (sw + 1 == n_sweeps && blk != 0) break;
             // every block's count of this sweep
@@ -328,8 +328,9 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
             }
             ok = __shfl_sync(0xffffffffu, int(ok), 0) != 0;
             v = __shfl_sync(0xffffffffu, v, 0) & ((1ull << 40) - 1ull);
-            acc = (long long)(v - before[sw & 1]);
-            before[sw & 1] = v;
+            acc = (long long)(v - (sw & 1 ? odd : even));
+            if (sw & 1) odd = v;
+            else even = v;
             if (adapt) theta = cone_rule(theta, acc, p.n_mov);
             if (lane == 0) {
                 if (ok) s_cone = cone[theta];
@@ -625,55 +626,6 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
             const float* src = bsm + size_t(c) * half + e.own + comp * Lh;
             for (uint32_t k = uint32_t(lane); k < Lh; k += 32) dst[k] = src[k];
         }
-}
-
-// The samples of n measured sweeps from their records, one warp per sweep:
-// ring entries, and in each record what the moments grow by; the last block
-// then adds those in the order of the sweeps (the additions of a sweep by
-// sweep close, so the same bits).
-template <int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(const __grid_constant__ BrickArgs one,
-                                                                const BrickArgs* many, int n) {
-    const BrickArgs& a = many ? many[blockIdx.y] : one;
-    BrickCtl* const ctl = a.ctl;
-    long long* const record = a.record;
-    const LatParams& p = a.lat->p;
-    LatState& st = a.lat->st;
-    const int lane = int(threadIdx.x & 31), w = int(blockIdx.x * WARPS + (threadIdx.x >> 5));
-    if (*reinterpret_cast<volatile int*>(&ctl->abort)) return;
-    const long long ring = st.ring_count;
-    if (w < n) {
-        long long* r = record + size_t(w) * kRecordWords;
-        const long long sum = lane < kNumSums ? r[lane] : 0, theta = r[kRecTheta], acc = r[kRecAcc];
-        double inc, y;
-        sample_words(p, sum, p.sample_torque != 0, lane, p.N, &inc, &y);  // its shuffles end the reads
-        if (lane < kMomentWords) r[lane] = __double_as_longlong(inc);
-        if (p.ring && lane < kRingWords && w + p.ring_cap >= n)
-            p.ring[(ring + w) % p.ring_cap * kRingWords + lane] =
-                ring_word(lane, st.sweep - uint32_t(n) + uint32_t(w), int(theta), acc, y);
-    }
-    __threadfence();
-    __syncthreads();
-    __shared__ bool last;
-    if (threadIdx.x == 0) last = atomicAdd(&ctl->closed, 1u) + 1u == gridDim.x;
-    __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
-    __threadfence();
-    if (lane < kMomTq2 + 3) {
-        double m = st.moments[lane];
-        const double* r = reinterpret_cast<const double*>(record) + lane;
-        int i = 0;
-        for (; i + 16 <= n; i += 16) {
-            double x[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = __ldcg(r + size_t(i + j) * kRecordWords);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) m += x[j];
-        }
-        for (; i < n; ++i) m += __ldcg(r + size_t(i) * kRecordWords);
-        st.moments[lane] = m;
-    }
-    if (lane == 0) st.ring_count = ring + n;
 }
 
 // Before a launch of several lattices: their control words (not the epochs) and

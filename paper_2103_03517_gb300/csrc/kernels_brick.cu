@@ -164,7 +164,7 @@ cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int 
             e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kRecordWords * sizeof(long long), s);
         if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
         if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, nullptr, a.n_sweeps);
+            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, static_cast<const BrickArgs*>(nullptr), a.n_sweeps);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) return e;
@@ -187,7 +187,7 @@ cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int
                 : c.odd    ? launch_m<1, 0, 1, 1>(none, g, c.blocks, c.smem, c32, measure, s)
                            : launch_m<1, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s);
         if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<dim3(uint32_t(m + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, c.args, m);
+            brick_close_kernel<4><<<dim3(uint32_t(m + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, static_cast<const BrickArgs*>(c.args), m);
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) return e;

@@ -203,18 +203,15 @@ constexpr int kResMaxSweeps = 2048;  // sweeps per launch; longer runs take seve
 
 // Control words of one lattice's resident launch, in device memory, zeroed
 // before every launch: the abort flag a block sets when one of its waits
-// runs out; for sweep s, in slot s mod 3 (one slot fills, one is read, one
-// is cleared), the blocks that have completed their black pass (high 32
-// bits) and their accepted moves (low 32 bits) in one word, and the
-// fixed-point sample sums; per block, the passes whose face rows it has
-// written.
+// runs out; the blocks of the closing launch that are done; by the sweep's
+// parity, running totals of the blocks that have completed their black pass
+// (bits 40 up) and of their accepted moves; per block, the passes whose face
+// rows it has written.
 constexpr int kResMaxBlocks = 256;
-constexpr int kResSlots = 3;
 struct ResCtl {
     int abort;
-    int pad;
-    unsigned long long arrive_acc[kResSlots];
-    long long sums[kResSlots][kNumSums];
+    unsigned int closed;
+    unsigned long long count[2];
     unsigned int done[kResMaxBlocks];
 };
 
@@ -227,6 +224,7 @@ struct ResCtl {
 struct ResidentArgs {
     LatDev* lat;
     ResCtl* ctl;
+    long long* record;  // [kBrickMaxMeasured][kRecordWords]
     int nyc, nzc, by, bz;
     uint32_t smem;
     int n_sweeps;

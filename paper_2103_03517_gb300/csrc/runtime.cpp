@@ -159,7 +159,7 @@ bool wave_desc(const mc_desc* d) {
 // the automatic one and kResAutoSpins spins; whether its rows fit is decided
 // on the device (KernelSet::resident_plan).  Below that size the brick sweeps
 // (brick_desc) are faster, their exchange between blocks being shorter: us a
-// sweep resident / brick 10.3 / 5.9 for 128 x 64 x 64, 15.9 / 17.5 for 128^3.
+// sweep resident / brick 10.3 / 5.9 for 128 x 64 x 64, 15.7 / 17.5 for 128^3.
 constexpr uint64_t kResAutoSpins = 3ull << 19;
 
 bool resident_desc(const mc_desc* d, bool slab) {
@@ -219,7 +219,7 @@ size_t lattice_bytes(const mc_desc* d, bool slab) {
     // launch tables of the lattice alone: lattice pointer, site and pair starts
     b += align256(sizeof(void*)) + 2 * align256(2 * sizeof(uint32_t));
     if (slab) b += align256(kSlabWords * 8);
-    if (resident_desc(d, slab)) b += align256(sizeof(ResCtl));
+    if (resident_desc(d, slab)) b += align256(sizeof(ResCtl)) + align256(kBrickRecordBytes);
     return b;
 }
 
@@ -489,11 +489,13 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     if (slab) p.slab_counts = reinterpret_cast<long long*>(take(kSlabWords * 8));
     if (resident_desc(d, slab != nullptr)) {  // its control words, if its rows fit the SMs
         void* ctl = take(sizeof(ResCtl));
+        long long* record = reinterpret_cast<long long*>(take(kBrickRecordBytes));
         ResidentPlan* rp = new ResidentPlan();
         if (kernels_f32().resident_plan(p, rp)) {
             p.rctl = ctl;
             rp->args.lat = h->d_lat;
             rp->args.ctl = static_cast<ResCtl*>(ctl);
+            rp->args.record = record;
             rp->args.key0 = p.key0;
             rp->args.key1 = p.key1;
             // fault injection for the tests of the bounded waits: the wait for
@@ -882,8 +884,9 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     if (!constrained && ls.n_res && k.resident_sweeps && n >= kResMinSweeps) {
         cudaError_t e = cudaSuccess;
         for (int i = 0; i < ls.n_res && e == cudaSuccess; ++i)
-            for (int done = 0; done < n && e == cudaSuccess; done += kResMaxSweeps) {
-                const int m = std::min(n - done, kResMaxSweeps);
+            for (int done = 0, most = measure ? kBrickMaxMeasured : kResMaxSweeps; done < n && e == cudaSuccess;
+                 done += most) {
+                const int m = std::min(n - done, most);
                 timed_kind(kTimedResident, [&] {
                     e = k.resident_sweeps(*ls.res[i], cone, m, measure ? ls.sample_level : 0, ls.shape.row, s);
                 });
