@@ -149,7 +149,7 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
         g->ls.n_res = n;
     }
     if (n == 1) {
-        g->ls.brick = lattices[0]->brick;
+        g->ls.brick = brick_of(lattices[0]);
         g->ls.brick_lh = uint32_t(lattices[0]->hp.Lh);
     } else {
         // all side by side in shared memory, where that beats the launches: those
@@ -158,11 +158,11 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
         long long spins = 0;
         std::vector<const LatParams*> hp;
         for (int i = 0; i < n; ++i) {
-            all = all && lattices[i]->brick && !lattices[i]->brick->faces;
+            all = all && lattices[i]->brick && !lattices[i]->brick->off && !lattices[i]->brick->faces;
             spins += lattices[i]->hp.N;
             hp.push_back(&lattices[i]->hp);
         }
-        if (all) {
+        if (all && spins <= kBrickMaxSpins) {
             std::unique_ptr<BrickSet> b(new BrickSet());
             b->lats = g->lats;
             b->plans.resize(size_t(n));

@@ -127,12 +127,22 @@ double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<B
     const Device d = device();
     const size_t n = lats.size();
     if (n > d.most) return 0.0;
-    std::vector<std::vector<Split>> s;
+    std::vector<std::vector<Split>> s;  // of each size once
+    std::vector<size_t> kind(n);
+    std::vector<const LatParams*> seen;
     std::vector<uint32_t> G(n);
     uint32_t total = 0;
     for (size_t i = 0; i < n; ++i) {
-        s.push_back(splits(*lats[i], d));
-        for (G[i] = 1; G[i] <= d.most && s[i][G[i]].nyc == 0;) ++G[i];
+        const LatParams& p = *lats[i];
+        for (kind[i] = 0; kind[i] < seen.size(); ++kind[i]) {
+            const LatParams& q = *seen[kind[i]];
+            if (q.Lh == p.Lh && q.Ly == p.Ly && q.Lz == p.Lz) break;
+        }
+        if (kind[i] == seen.size()) {
+            seen.push_back(&p);
+            s.push_back(splits(p, d));
+        }
+        for (G[i] = 1; G[i] <= d.most && s[kind[i]][G[i]].nyc == 0;) ++G[i];
         if (G[i] > d.most) return 0.0;
         total += G[i];
     }
@@ -140,17 +150,17 @@ double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<B
     for (;;) {  // more blocks for the slowest, while they make it faster and there are any
         size_t i = 0;
         for (size_t j = 1; j < n; ++j)
-            if (s[j][G[j]].cost > s[i][G[i]].cost) i = j;
+            if (s[kind[j]][G[j]].cost > s[kind[i]][G[i]].cost) i = j;
         uint32_t g = G[i] + 1;
-        while (g <= d.most && s[i][g].cost >= s[i][G[i]].cost) ++g;
+        while (g <= d.most && s[kind[i]][g].cost >= s[kind[i]][G[i]].cost) ++g;
         if (g > d.most || total + (g - G[i]) > d.most) break;
         total += g - G[i];
         G[i] = g;
     }
     double slowest = 0.0;
     for (size_t i = 0; i < n; ++i) {
-        take(*lats[i], s[i][G[i]], &(*out)[i]);
-        slowest = std::max(slowest, s[i][G[i]].cost);
+        take(*lats[i], s[kind[i]][G[i]], &(*out)[i]);
+        slowest = std::max(slowest, s[kind[i]][G[i]].cost);
     }
     return 2.0 * slowest;
 }

@@ -274,8 +274,9 @@ struct BrickArgs {
     BrickCtl* ctl;
     void* packets;
     long long* record;    // [kBrickMaxMeasured][kRecordWords]
-    uint32_t nyc, nzc, rows, smem;
+    uint32_t nyc, nzc, rows, smem;  // nyc = 0: not planned yet
     FastDiv div_half;     // by Lh / 2
+    int off;              // it does not fit, or its launch was refused: swept by launches
     size_t bytes;         // of the lattice's brick memory: ctl (null until it is allocated), record, packets
     int law, faces;       // kernel instance: packed or scalar law, any boundaries
     int n_sweeps;

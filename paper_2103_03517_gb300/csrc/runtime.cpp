@@ -176,13 +176,12 @@ bool resident_desc(const mc_desc* d, bool slab) {
 // simple cubic without film tables, not a slab, the automatic or resident
 // kernel path, at most kBrickMaxSpins spins (whether its rows fit is decided
 // on the device, brick_plan); 128-wide periodic lattices take resident_pass.cuh.
-constexpr uint64_t kBrickMaxSpins = 3000000;
 
 bool brick_desc(const mc_desc* d, bool slab) {
     if (slab || d->precision != MC_FP32 || d->lattice != MC_SC || resident_desc(d, slab)) return false;
     if (d->kernel_path != MC_PATH_AUTO && d->kernel_path != MC_PATH_RESIDENT) return false;
     if (d->bond_mask || d->grain_id) return false;
-    return uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] <= kBrickMaxSpins;
+    return uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] <= uint64_t(kBrickMaxSpins);
 }
 
 // Device memory of the brick sweeps of such a lattice, allocated by its first
@@ -509,15 +508,14 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     }
     if (brick_desc(d, slab != nullptr)) {
         BrickArgs b{};
-        if (brick_plan(p, &b)) {
-            b.lat = h->d_lat;
-            b.key0 = p.key0;
-            b.key1 = p.key1;
-            b.bytes = brick_bytes(d);
-            const char* inj = std::getenv("MC_RESIDENT_INJECT_TIMEOUT");  // as for the resident sweeps
-            b.inject = inj && inj[0] == '1' ? 1 : 0;
-            h->brick = new BrickArgs(b);
-        }
+        b.lat = h->d_lat;
+        b.key0 = p.key0;
+        b.key1 = p.key1;
+        b.bytes = brick_bytes(d);
+        b.faces = p.bc[0] || p.bc[1] || p.bc[2] ? 1 : 0;
+        const char* inj = std::getenv("MC_RESIDENT_INJECT_TIMEOUT");  // as for the resident sweeps
+        b.inject = inj && inj[0] == '1' ? 1 : 0;
+        h->brick = new BrickArgs(b);
     }
     if (size_t(cur - static_cast<char*>(h->d_base)) > h->bytes) {
         cudaFree(h->d_base);
@@ -596,6 +594,14 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     return MC_OK;
 }
 
+// The lattice's brick sweeps, planned on first use; null if it has none.
+BrickArgs* brick_of(mc_lattice* h) {
+    BrickArgs* b = h->brick;
+    if (!b || b->off) return nullptr;
+    if (b->nyc == 0 && !brick_plan(h->hp, b)) b->off = 1;
+    return b->off ? nullptr : b;
+}
+
 // Lattices whose row-kernel passes take a block's tiles in turn (TURNS in
 // row_pass.cuh): long rows, and tiles enough that a block lies in one or two
 // lattices.
@@ -615,7 +621,7 @@ LaunchSet single_launch_set(mc_lattice* h) {
     }
     ls.sample_level = h->hp.sample_torque ? 2 : 1;
     ls.shape = h->shape;
-    ls.brick = h->brick;
+    ls.brick = brick_of(h);
     ls.brick_lh = uint32_t(h->hp.Lh);
     if (h->hp.nsub > 1) {
         const bool j2 = h->desc.lattice != MC_HCP && h->desc.J2 != 0.0;
@@ -818,6 +824,8 @@ static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
         a.nzc = plan.nzc;
         a.rows = plan.rows;
         a.smem = plan.smem;
+        a.div_half = plan.div_half;
+        a.law = plan.law;
         args[a.law == 0 ? 0 : 1 + b->lats[i]->hp.Lh % 2].push_back(a);
     }
     std::vector<char> host;
@@ -894,27 +902,42 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         return MC_OK;
     }
-    if (!constrained && ls.brick && n >= kResMinSweeps && brick_memory(ls.brick, s)) {
+    // a launch that the device refuses as too large for it (a context with fewer
+    // SMs) leaves the lattices as they were, and they are swept by launches
+    auto refused = [&](cudaError_t e, int done) {
+        if (e != cudaErrorCooperativeLaunchTooLarge || done) return false;
+        cudaGetLastError();
+        return true;
+    };
+    if (!constrained && ls.brick && !ls.brick->off && n >= kResMinSweeps && brick_memory(ls.brick, s)) {
         cudaError_t e = cudaSuccess;
         const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
-        for (int done = 0; done < n && e == cudaSuccess; done += most)
+        for (int done = 0; done < n && e == cudaSuccess && !ls.brick->off; done += most)
             timed_kind(kTimedResident, [&] {
                 e = brick_sweeps(*ls.brick, ls.brick_lh, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
+                if (refused(e, done)) ls.brick->off = 1;
             });
-        if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
-        return MC_OK;
+        if (!ls.brick->off) {
+            if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
+            return MC_OK;
+        }
     }
     if (!constrained && ls.brick_set && n >= kResMinSweeps && brick_set_ready(ls.brick_set, s)) {
         cudaError_t e = cudaSuccess;
         const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
+        int launches = 0;
         for (int done = 0; done < n; done += most)
             for (const BrickClass& c : ls.brick_set->classes)
-                timed_kind(kTimedResident, [&] {
-                    if (e == cudaSuccess)
+                if (e == cudaSuccess)
+                    timed_kind(kTimedResident, [&] {
                         e = brick_group_sweeps(c, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
-                });
-        if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
-        return MC_OK;
+                        if (refused(e, launches)) ls.brick_set->failed = true;
+                        ++launches;
+                    });
+        if (!ls.brick_set->failed) {
+            if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
+            return MC_OK;
+        }
     }
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
     auto kind_pass = [&](int kind, const GroupArgs& ga, uint32_t nt, int colour, int meas) {
@@ -1043,7 +1066,7 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
                bool constrained, cudaStream_t s) {
     const KernelSet& k = kernel_set(precision);
     // resident sweeps run many to a launch: nothing to capture
-    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && brick_memory(ls.brick, s)) || (ls.brick_set && brick_set_ready(ls.brick_set, s))))
+    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) || (ls.brick_set && brick_set_ready(ls.brick_set, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
     const int reps = n / kGraphSweeps;
     if (reps > 0) {

@@ -34,6 +34,9 @@ constexpr int kResMinSweeps = 3;
 // held in shared memory it sweeps faster than its share of a batched row
 // pass; smaller lattices sweep faster batched).
 constexpr long long kResGroupMinSpins = 1ll << 21;
+// Brick sweeps hold at most this many spins (12 bytes each in the SMs' shared
+// memory).
+constexpr long long kBrickMaxSpins = 3000000;
 struct SweepGraphs {
     cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
 };
@@ -121,6 +124,7 @@ int observables_from(const mc_lattice* h, const LatState& st, mc_observables* ou
 int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* cone, int n, int measure,
                bool constrained, cudaStream_t s);
 void destroy_graphs(SweepGraphs& gr);
+BrickArgs* brick_of(mc_lattice* h);
 bool long_rows(const LatParams& p);
 LaunchSet single_launch_set(mc_lattice* h);
 int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats, const void* cone, int sweeps,
