@@ -138,11 +138,21 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
                               int(sub[c].size())};
         *counts[c] = st[c].back();
     }
-    // resident lattices: alone, or a group made only of large ones (swept one
-    // after another, each held in shared memory)
-    bool all_res = true;
-    for (int i = 0; i < n; ++i)
-        all_res = all_res && lattices[i]->res && (n == 1 || lattices[i]->hp.N >= kResGroupMinSpins);
+    // lattices held in shared memory: one alone (resident or brick sweeps), or a
+    // group made only of large resident ones (one after another) or only of small
+    // ones (side by side as brick sweeps).  Both kinds in one group, held one kind
+    // after the other, lose to launches in calls of 20 sweeps: each large lattice
+    // is loaded and stored once a call (the 32-lattice batch 183 -> 193 us a sweep).
+    bool all_res = true, all_brick = n > 1;
+    long long spins = 0;
+    std::vector<const LatParams*> hp;
+    for (int i = 0; i < n; ++i) {
+        const mc_lattice* h = lattices[i];
+        all_res = all_res && h->res && (n == 1 || h->hp.N >= kResGroupMinSpins);
+        all_brick = all_brick && h->brick && !h->brick->off && !h->brick->faces;
+        spins += h->hp.N;
+        hp.push_back(&h->hp);
+    }
     if (all_res) {
         for (int i = 0; i < n; ++i) g->res_plans.push_back(lattices[i]->res);
         g->ls.res = g->res_plans.data();
@@ -151,26 +161,16 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
     if (n == 1) {
         g->ls.brick = brick_of(lattices[0]);
         g->ls.brick_lh = uint32_t(lattices[0]->hp.Lh);
-    } else {
-        // all side by side in shared memory, where that beats the launches: those
-        // take about 8 us a sweep and 10 ps a spin
-        bool all = true;
-        long long spins = 0;
-        std::vector<const LatParams*> hp;
-        for (int i = 0; i < n; ++i) {
-            all = all && lattices[i]->brick && !lattices[i]->brick->off && !lattices[i]->brick->faces;
-            spins += lattices[i]->hp.N;
-            hp.push_back(&lattices[i]->hp);
-        }
-        if (all && spins <= kBrickMaxSpins) {
-            std::unique_ptr<BrickSet> b(new BrickSet());
-            b->lats = g->lats;
-            b->plans.resize(size_t(n));
-            const double us = brick_group_plan(hp, &b->plans);
-            if (us > 0.0 && us < 8.0 + 1e-5 * double(spins)) {
-                g->ls.brick_set = b.get();
-                g->brick_set = std::move(b);
-            }
+    }
+    if (all_brick && spins <= kBrickMaxSpins) {
+        std::unique_ptr<BrickSet> b(new BrickSet());
+        b->lats = g->lats;
+        b->plans.resize(size_t(n));
+        const double us = brick_group_plan(hp, &b->plans);
+        // against launches: about 8 us a sweep and 10 ps a spin
+        if (us > 0.0 && us < 8.0 + 1e-5 * double(spins)) {
+            g->ls.brick_set = b.get();
+            g->brick_set = std::move(b);
         }
     }
     g->ls.sample_level = 1;

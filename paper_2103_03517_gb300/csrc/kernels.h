@@ -61,7 +61,7 @@ struct KernelSet {
     // gen = 1: any boundaries; gen = 2: film tables, any boundaries; turns: the
     // warps of a block share its tiles in turn (LaunchSet::turns).  Null in the FP64 set.  After a
     // black pass (colour 1) it also launches the close of the lattices' sweeps
-    // (row_close_kernel); of measured ones the samples are formed by
+    // (sweep_close_kernel); of measured ones the samples are formed by
     // sample_close.  Returns the status of the
     // launches (made with programmatic serialisation).
     cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law,
@@ -92,9 +92,8 @@ struct KernelSet {
     void (*profile)(LatDev* d, uint32_t Lh, uint32_t rows, cudaStream_t s);
     // The spins of a new lattice p (host copy): all along v, or a wall along x.
     void (*init_spins)(const LatParams& p, int wall, const double v[3], cudaStream_t s);
-    // The samples of the measured sweeps of row-kernel lattices since the last
-    // call (at most kSampleRecords), of every lattice of g.  Null in the FP64
-    // set.
+    // The samples of the measured launched sweeps since the last call (at most
+    // kSampleRecords), of every lattice of g.
     void (*sample_close)(const GroupArgs& g, cudaStream_t s);
     const char* name;
     // FP32 wavefront sweep (red and black pass in one launch) of the

@@ -47,7 +47,7 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
     const cudaError_t e =
         launch_chained(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, sp.blocks, sp.threads, s, g, ntiles, cone, colour);
     if (e != cudaSuccess || colour != 1) return e;  // the sweep's end
-    return launch_chained(row_close_kernel, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
+    return launch_chained(sweep_close_kernel<R>, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
 }
 
 // launch shape 0: the default blocks per SM of the instance (B0 of a pass
@@ -87,10 +87,6 @@ cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int 
     return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
 }
 
-void sample_close(const GroupArgs& g, cudaStream_t s) {
-    sample_close_kernel<<<uint32_t(g.n), 32 * kSampleRecords, 0, s>>>(g);
-}
-
 // the all-periodic instance samples red sites first and stores their field
 // (the next constrained sweep's red field); the other keeps black
 template <int GEN>
@@ -98,7 +94,7 @@ void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
     constexpr int B = GEN == 2 ? MINB_FILM_M : (GEN == 1 ? MINB_FACES_M : MINB);
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
     const Spread sp = spread_warps(ntiles, cap);
-    launch_chained_if(sp.blocks < cap, row_pass_kernel<B, 2, GEN, 0>, sp.blocks, sp.threads, s, g, ntiles,
+    launch_chained_if(chain_small(sp, cap), row_pass_kernel<B, 2, GEN, 0>, sp.blocks, sp.threads, s, g, ntiles,
                       static_cast<const R*>(nullptr), GEN ? 1 : 0);
 }
 
@@ -112,7 +108,7 @@ template <bool LEADER, int C, int B = LEADER ? MINB_PAIR_LEAD : MINB_PAIR, int N
 void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int sub, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B, C, LEADER, NT>, NT);
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap, NT);
-    launch_chained_if(sp.blocks < cap, pair_pass_kernel<R, B, C, LEADER, NT>, sp.blocks, sp.threads, s, g, ntiles,
+    launch_chained_if(chain_small(sp, cap), pair_pass_kernel<R, B, C, LEADER, NT>, sp.blocks, sp.threads, s, g, ntiles,
                       static_cast<const R*>(cone), colour, sub);
 }
 

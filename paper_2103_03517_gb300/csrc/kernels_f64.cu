@@ -19,7 +19,7 @@ template <int C>
 void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, int sub, uint32_t cap,
                  cudaStream_t s) {
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
-    launch_chained_if(sp.blocks < cap, pair_pass_kernel<R, 1, C, false>, sp.blocks, sp.threads, s, g, ntiles, cone, colour, sub);
+    launch_chained_if(chain_small(sp, cap), pair_pass_kernel<R, 1, C, false>, sp.blocks, sp.threads, s, g, ntiles, cone, colour, sub);
 }
 
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step; FP64
@@ -41,7 +41,7 @@ void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour
 const KernelSet& kernels_f64() {
     static const KernelSet k{colour_pass, nullptr,     pair_pass,   sweep_end,         pair_field,
                              ml_reset,    mlong,       measure,     nullptr,           grain_sample,
-                             profile,     init_spins,  nullptr,     "f64",
+                             profile,     init_spins,  sample_close, "f64",
                              nullptr,     nullptr,     nullptr,           nullptr,      nullptr,
                              nullptr,     nullptr,     nullptr};
     return k;

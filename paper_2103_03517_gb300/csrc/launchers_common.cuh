@@ -12,7 +12,9 @@ template <int MEASURE>
 void colour_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(colour_pass_kernel<R, V, MINB, MEASURE>);
     const Spread sp = spread_warps(ntiles, cap);
-    colour_pass_kernel<R, V, MINB, MEASURE><<<sp.blocks, sp.threads, 0, s>>>(g, ntiles, cone, colour);
+    const bool full = sp.threads == kBlock;  // FP64: the launch fills the SMs (64^3: 133 -> 127 us a sweep)
+    launch_chained_if(!kIsF64<R> || full || chain_small(sp, cap), colour_pass_kernel<R, V, MINB, MEASURE>, sp.blocks, sp.threads, s, g, ntiles, cone, colour);
+    if (colour == 1) launch_chained(sweep_close_kernel<R>, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
 }
 
 // measure: 0 none, 1 magnetisation and energies, 2 also torques
@@ -21,6 +23,10 @@ void colour_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
     if (measure >= 2) colour_pass_t<2>(g, ntiles, c, colour, s);
     else if (measure == 1) colour_pass_t<1>(g, ntiles, c, colour, s);
     else colour_pass_t<0>(g, ntiles, c, colour, s);
+}
+
+void sample_close(const GroupArgs& g, cudaStream_t s) {
+    sample_close_kernel<R><<<uint32_t(g.n), 32 * kSampleRecords, 0, s>>>(g);
 }
 
 void sweep_end(const GroupArgs& g, cudaStream_t s) {
@@ -33,7 +39,7 @@ void sweep_end(const GroupArgs& g, cudaStream_t s) {
 template <int C>
 void pair_field_t(const GroupArgs& g, uint32_t ntiles, int colour, uint32_t cap, cudaStream_t s) {
     const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
-    launch_chained_if(sp.blocks < cap, pair_field_kernel<R, V, C>, sp.blocks, sp.threads, s, g, ntiles, colour);
+    launch_chained_if(chain_small(sp, cap), pair_field_kernel<R, V, C>, sp.blocks, sp.threads, s, g, ntiles, colour);
 }
 
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step

@@ -108,7 +108,7 @@ struct LatParams {
     const uint8_t* bonds;   // [2][stride] or null
     const int32_t* grain;   // [2][stride] or null
     const void* gaxis;      // [n_grains][4] in the lattice precision, or null
-    long long* records;     // FP32: [kSampleRecords][kRecordWords]
+    long long* records;     // [kSampleRecords][kRecordWords]
     double* ring;           // [ring_cap][kRingWords]
     int ring_cap;
     long long* profile;     // [3][Lx] fixed-point sums

@@ -212,7 +212,7 @@ size_t lattice_bytes(const mc_desc* d, bool slab) {
         b += align256(3 * ng * 8) + align256(ng * 4) + align256((ng + 1) * 8);  // grain samples
     }
     const int cap = d->ring_capacity > 0 ? d->ring_capacity : 4096;
-    if (rs == 4) b += align256(size_t(kSampleRecords) * kRecordWords * 8);
+    b += align256(size_t(kSampleRecords) * kRecordWords * 8);
     b += align256(size_t(cap) * kRingWords * 8);
     b += align256(3 * size_t(d->dims[0]) * 8);
     // launch tables of the lattice alone: lattice pointer, site and pair starts
@@ -479,7 +479,7 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
         h->film_grain.assign(din->grain_id, din->grain_id + p.N);
         h->film_axes.assign(din->grain_axis, din->grain_axis + 3 * size_t(d->n_grains));
     }
-    if (rs == 4) p.records = reinterpret_cast<long long*>(take(size_t(kSampleRecords) * kRecordWords * 8));
+    p.records = reinterpret_cast<long long*>(take(size_t(kSampleRecords) * kRecordWords * 8));
     p.ring = reinterpret_cast<double*>(take(size_t(p.ring_cap) * kRingWords * 8));
     p.profile = reinterpret_cast<long long*>(take(3 * size_t(p.Lx) * 8));
     h->d_group_lats = reinterpret_cast<LatDev**>(take(sizeof(void*)));
@@ -891,14 +891,13 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     // all n sweeps held in shared memory, lattice after lattice (see kResMinSweeps)
     if (!constrained && ls.n_res && k.resident_sweeps && n >= kResMinSweeps) {
         cudaError_t e = cudaSuccess;
+        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
         for (int i = 0; i < ls.n_res && e == cudaSuccess; ++i)
-            for (int done = 0, most = measure ? kBrickMaxMeasured : kResMaxSweeps; done < n && e == cudaSuccess;
-                 done += most) {
-                const int m = std::min(n - done, most);
+            for (int done = 0; done < n && e == cudaSuccess; done += most)
                 timed_kind(kTimedResident, [&] {
-                    e = k.resident_sweeps(*ls.res[i], cone, m, measure ? ls.sample_level : 0, ls.shape.row, s);
+                    e = k.resident_sweeps(*ls.res[i], cone, std::min(n - done, most), measure ? ls.sample_level : 0,
+                                          ls.shape.row, s);
                 });
-            }
         if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         return MC_OK;
     }
@@ -1001,8 +1000,6 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     };
     bool rest_any = ls.nt_row_rest != 0;
     for (int c = 0; c < kColourKinds; ++c) rest_any = rest_any || (c != kColourRow && ls.nt_col[c]);
-    bool row_any = false;  // lattices whose samples sample_close forms
-    for (int c = kColourRow; c < kColourKinds; ++c) row_any = row_any || ls.nt_col[c];
     bool red_field_ready = false;  // the next constrained sweep's red field is stored
     for (int i = 0; i < n; ++i) {
         // wavefront lattices sweep two at a time, spins -> spins_alt -> spins,
@@ -1053,7 +1050,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
             }
         }
-        if (!constrained && measure && row_any && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
+        if (!constrained && measure && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
             k.sample_close(ls.all, s);
     }
     if (launch_err != cudaSuccess) return cuda_fail(launch_err, "row kernel launch");
@@ -1066,7 +1063,9 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
                bool constrained, cudaStream_t s) {
     const KernelSet& k = kernel_set(precision);
     // resident sweeps run many to a launch: nothing to capture
-    if (!constrained && n >= kResMinSweeps && (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) || (ls.brick_set && brick_set_ready(ls.brick_set, s))))
+    if (!constrained && n >= kResMinSweeps &&
+        (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) ||
+         (ls.brick_set && brick_set_ready(ls.brick_set, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
     const int reps = n / kGraphSweeps;
     if (reps > 0) {

@@ -30,13 +30,18 @@ struct Spread {
     int threads;
 };
 
-Spread spread_warps(uint32_t warps, uint32_t cap, int threads = kBlock) {
+uint32_t sm_count() {
     static const uint32_t sms = [] {
         int dev = 0, n = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         return uint32_t(n > 0 ? n : 1);
     }();
+    return sms;
+}
+
+Spread spread_warps(uint32_t warps, uint32_t cap, int threads = kBlock) {
+    const uint32_t sms = sm_count();
     const uint32_t wpb = uint32_t(threads / 32);
     if (warps == 0) warps = 1;
     if (warps >= cap * wpb) return Spread{cap, threads};
@@ -73,6 +78,13 @@ cudaError_t launch_chained_if(bool chain, void (*kernel)(K...), uint32_t blocks,
     cfg.attrs = attr;
     cfg.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, a...);
+}
+
+// Whether a pass that leaves room on the GPU is chained.  FP64: only where it
+// and the next fit the SMs side by side; blocks dealt out while the SMs are busy
+// pile up on some, and with them FP64 work (32^3: 39 -> 66 us a sweep).
+bool chain_small(const Spread& sp, uint32_t cap) {
+    return kIsF64<R> ? 2 * sp.blocks <= sm_count() : sp.blocks < cap;
 }
 
 template <typename... K, typename... A>

@@ -7,7 +7,7 @@
 template <typename... K, typename... A>
 cudaError_t xtal_launch(void (*kernel)(K...), uint32_t ntiles, uint32_t cap, cudaStream_t s, A... a) {
     const Spread sp = spread_warps(ntiles, cap);
-    return launch_chained(kernel, sp.blocks, sp.threads, s, a...);
+    return launch_chained_if(!kIsF64<R> || chain_small(sp, cap), kernel, sp.blocks, sp.threads, s, a...);
 }
 
 template <int TYPE, int J2>
