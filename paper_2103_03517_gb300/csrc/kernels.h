@@ -95,6 +95,9 @@ struct KernelSet {
     // The samples of the measured launched sweeps since the last call (at most
     // kSampleRecords), of every lattice of g.
     void (*sample_close)(const GroupArgs& g, cudaStream_t s);
+    // pair_field over all-periodic lattices in the row layout.  Null in the FP64
+    // set.
+    void (*row_field)(const GroupArgs& g, uint32_t ntiles, int colour, int shape, cudaStream_t s);
     const char* name;
     // FP32 wavefront sweep (red and black pass in one launch) of the
     // lattices of a, nblocks blocks; dir = 0 reads spins and writes

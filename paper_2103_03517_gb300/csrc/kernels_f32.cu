@@ -87,6 +87,22 @@ cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int 
     return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
 }
 
+template <int C>
+void row_field_t(const GroupArgs& g, uint32_t ntiles, int colour, uint32_t cap, cudaStream_t s) {
+    const Spread sp = spread_warps((ntiles + C - 1) / C, cap);
+    launch_chained_if(chain_small(sp, cap), row_field_kernel<C>, sp.blocks, sp.threads, s, g, ntiles, colour);
+}
+
+// launch shapes as for pair_field
+void row_field(const GroupArgs& g, uint32_t ntiles, int colour, int shape, cudaStream_t s) {
+    static const uint32_t cap = resident_blocks(row_field_kernel<kFieldChunk>);
+    const int c = tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : kFieldChunk);
+    if (c == 8) row_field_t<8>(g, ntiles, colour, cap, s);
+    else if (c == 4) row_field_t<4>(g, ntiles, colour, cap, s);
+    else if (c == 2) row_field_t<2>(g, ntiles, colour, cap, s);
+    else row_field_t<1>(g, ntiles, colour, cap, s);
+}
+
 // the all-periodic instance samples red sites first and stores their field
 // (the next constrained sweep's red field); the other keeps black
 template <int GEN>
@@ -366,7 +382,7 @@ cudaError_t slab_close_all(LatDev* const* lats, int n, int measure, cudaStream_t
 const KernelSet& kernels_f32() {
     static const KernelSet k{colour_pass, row_pass,    pair_pass,   sweep_end,         pair_field,
                              ml_reset,    mlong,       measure,     row_sample,        grain_sample,
-                             profile,     init_spins,  sample_close, "f32",
+                             profile,     init_spins,  sample_close, row_field, "f32",
                              wave_sweep,  wave_blocks, slab_export,       slab_close,   slab_halo,
                              slab_close_all, resident_sweeps, resident_plan};
     return k;

@@ -41,7 +41,7 @@ void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour
 const KernelSet& kernels_f64() {
     static const KernelSet k{colour_pass, nullptr,     pair_pass,   sweep_end,         pair_field,
                              ml_reset,    mlong,       measure,     nullptr,           grain_sample,
-                             profile,     init_spins,  sample_close, "f64",
+                             profile,     init_spins,  sample_close, nullptr, "f64",
                              nullptr,     nullptr,     nullptr,           nullptr,      nullptr,
                              nullptr,     nullptr,     nullptr};
     return k;

@@ -360,6 +360,47 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 }
 
 // ------------------------------------------------------------------------
+// The neighbour field of one colour (LatParams::pfield) of all-periodic lattices
+// in the row layout, as pair_field_kernel forms it for any lattice, from the
+// spins instead of the packed copy (the pair passes keep both in step): two
+// sites a lane, x neighbours by shuffle, so that 64 sites take 15 8-byte loads a
+// lane where the other takes 12 of 16 bytes, which kept L1 91% busy (80 x 64^3:
+// 85 us a colour).  The same terms in the same order (the -x, +x pair commutes):
+// the same bits.  Tiles in the same grid-stride order.
+// ------------------------------------------------------------------------
+template <int CHUNK>
+__global__ void __launch_bounds__(kBlock) row_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t nwarps = gridDim.x * uint32_t(kBlock / 32);
+    const uint32_t w = blockIdx.x * uint32_t(kBlock / 32) + (threadIdx.x >> 5);
+    const int lane = int(threadIdx.x & 31);
+    int l = 0;
+    for (uint32_t c0 = w * CHUNK; c0 < ntiles; c0 += nwarps * CHUNK) {
+        const uint32_t c1 = min(c0 + uint32_t(CHUNK), ntiles);
+        for (uint32_t tile = c0; tile < c1;) {
+            while (__ldg(&g.start[l + 1]) <= tile) ++l;  // tiles only move forward
+            const uint32_t t0 = __ldg(&g.start[l]);
+            const uint32_t t1 = min(__ldg(&g.start[l + 1]), c1);
+            const LatParams& p = g.lats[l]->p;
+            const float* s = static_cast<const float*>(p.spins);
+            Spin4<float>* fld = static_cast<Spin4<float>*>(p.pfield);
+            if (fld)
+                for (uint32_t t = tile; t < t1; ++t) {
+                    const uint32_t q0 = (t - t0) * 64u;
+                    P3 S, h, O;
+                    bool mov[2];
+                    row_pair_sums<0>(p, s, colour, q0, lane, 0u, S, h, O, mov);
+                    Spin4<float>* f = fld + q0 + 2u * uint32_t(lane);
+                    f[0] = Spin4<float>{h.x.x, h.y.x, h.z.x, 0.0f};
+                    f[1] = Spin4<float>{h.x.y, h.y.y, h.z.y, 0.0f};
+                }
+            tile = t1;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------
 // Slabs of one lattice split along z (the decomposition of Sec. 2's
 // multi-GPU projection).  A slab's passes publish their accepted moves and
 // sample sums but never close the sweep.  After the black pass each slab

@@ -1000,6 +1000,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
     };
     bool rest_any = ls.nt_row_rest != 0;
     for (int c = 0; c < kColourKinds; ++c) rest_any = rest_any || (c != kColourRow && ls.nt_col[c]);
+    const bool row_only = k.row_field && ls.nt_col[kColourRow] && ls.col[kColourRow].n == ls.all.n;
     bool red_field_ready = false;  // the next constrained sweep's red field is stored
     for (int i = 0; i < n; ++i) {
         // wavefront lattices sweep two at a time, spins -> spins_alt -> spins,
@@ -1027,7 +1028,10 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
             for (int colour = 0; colour < 2; ++colour) {
                 // a measured sweep of all-periodic row lattices leaves the red field
                 // behind in its sample (row_sample); otherwise sum it here
-                if (!(colour == 0 && red_field_ready)) k.pair_field(ls.all, ls.nt_all, colour, ls.shape.field, s);
+                if (!(colour == 0 && red_field_ready)) {
+                    if (row_only) k.row_field(ls.col[kColourRow], ls.nt_col[kColourRow], colour, ls.shape.field, s);
+                    else k.pair_field(ls.all, ls.nt_all, colour, ls.shape.field, s);
+                }
                 timed([&] {
                     if (ls.nt_pairs) k.pair_pass(ls.pairs, ls.nt_pairs, cone, colour, 0, ls.shape.pair, 0, s);
                     if (ls.nt_pairs_lead)
