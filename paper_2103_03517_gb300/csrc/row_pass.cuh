@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 // the same bits.  Tiles in the same grid-stride order.
 // ------------------------------------------------------------------------
 template <int CHUNK>
-__global__ void __launch_bounds__(kBlock) row_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
+__global__ void __launch_bounds__(kBlock, 4) row_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t nwarps = gridDim.x * uint32_t(kBlock / 32);
