@@ -47,7 +47,8 @@ typedef enum mc_status {
     MC_ERR_NOMEM = -2,      /* device memory exhausted / job can never fit       */
     MC_ERR_CUDA = -3,       /* a CUDA call failed (message in mc_last_error)     */
     MC_ERR_TIMEOUT = -4,    /* a bounded device wait gave up (the wavefront,     */
-                            /* resident and brick kernels' waits, about one second each;   */
+                            /* resident and brick kernels' waits, about one      */
+                            /* second each;                                      */
                             /* MC_WAVE_INJECT_TIMEOUT=1 or                       */
                             /* MC_RESIDENT_INJECT_TIMEOUT=1 in the environment   */
                             /* when a lattice is created makes its first wait    */
@@ -78,9 +79,11 @@ typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIP
  * 3 sweeps: a 128-wide all-periodic one of 1.5 million spins and more resident
  * (see RESIDENT), any other as brick sweeps, one cooperative launch per call of
  * up to 2048 sweeps (512 measured), for which it takes 16 bytes per spin of
- * device memory on first use (without them it sweeps by launches).  GENERAL always takes the
+ * device memory on first use (without them it sweeps by launches).  A group of
+ * such lattices with every axis periodic that together fit sweeps them side by
+ * side in one such launch.  GENERAL always takes the
  * general colour-pass kernel and the pairs in pair order.  ROW is AUTO
- * without the resident sweeps: the row kernels for every colour pass.
+ * without the resident and brick sweeps: a launch for every colour pass.
  * WAVE is ROW, except that on an all-periodic lattice with Lx = 128 and
  * Ly >= 16 (no film tables) the sweeps of each mc_sweep / mc_group_sweep
  * call run two at a time as single wavefront launches (red and black pass
@@ -95,10 +98,10 @@ typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIP
  * blocks between sweeps (each wait bounded; a wait that runs out gives
  * MC_ERR_TIMEOUT).  A group made only of such lattices of at least 2^21
  * spins each (128^3 and larger) sweeps them resident one after another.
- * Constrained sweeps, calls of fewer than 3 sweeps and other groups take
- * the row kernels.  The colour passes of AUTO, GENERAL,
+ * Constrained sweeps, calls of fewer than 3 sweeps and other groups sweep by
+ * launches.  The colour passes of AUTO, GENERAL,
  * WAVE and RESIDENT agree up to FP32 rounding (the draws are keyed to the
- * same sites; the wavefront, resident and row kernels bit for bit) and the
+ * same sites; the wavefront, resident, brick and row kernels bit for bit) and the
  * two pair orders exactly; GENERAL, ROW, WAVE and RESIDENT exist to compare
  * them.  FP64 lattices always take the general kernel and pair order. */
 typedef enum mc_kernel_path {
@@ -548,7 +551,8 @@ MC_API int mc_slab_sweep(const mc_handle* slabs, int n, int n_sweeps, int measur
  * libmc's kernels there, so make that first call before any stream
  * capture.  Every call rewrites the whole scratch
  * and clears its counters; calls that overlap on the GPU (on different
- * streams, or from different threads) race on it.
+ * streams, or from different threads) race on it: their results are undefined,
+ * and a call may end in MC_ERR_TIMEOUT.
  *
  * spins     device memory, FP32, colour-split layout of mc_export_state:
  *           6 * stride floats, stride = N/2 rounded up to a multiple of 64,

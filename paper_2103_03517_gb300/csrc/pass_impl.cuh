@@ -687,7 +687,9 @@ __device__ inline void finalize_sweep(const LatParams& p, LatState& st, int meas
 // warp tiles (a warp tile = 32 * V colour indices, or 32 pairs, of one
 // lattice; lattice l owns tiles [g.start[l], g.start[l+1])).  A warp walks
 // its chunk lattice by lattice and publishes each lattice's counts once per
-// run of tiles; no block-wide barrier is involved.
+// run of tiles; no block-wide barrier is involved.  (The TURNS instances of the
+// row kernel take a block's tiles in turn; FP64 launches that do not fill the GPU
+// take the smaller blocks of spread.cuh.)
 // ------------------------------------------------------------------------
 struct WarpChunk {
     uint32_t begin, end;

@@ -30,7 +30,9 @@
 // samples are those of the general kernel (scalar_move), whose chain it gives
 // bit for bit.  In the general kernel each of a lane's two sites found its own
 // neighbours and loaded them one float at a time: 750 warp instructions per 64
-// sites, 46% of them issued per cycle, 47 us a pass of 160^3.
+// sites, 46% of them issued per cycle, 47 us a pass of 160^3; here 373 and 24
+// us.  What bounds it is what bounds the other instances: issue (49% of the
+// cycles) and the latency of a tile's loads.
 #pragma once
 #include "pair_math.cuh"
 
@@ -365,8 +367,10 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 // spins instead of the packed copy (the pair passes keep both in step): two
 // sites a lane, x neighbours by shuffle, so that 64 sites take 15 8-byte loads a
 // lane where the other takes 12 of 16 bytes, which kept L1 91% busy (80 x 64^3:
-// 85 us a colour).  The same terms in the same order (the -x, +x pair commutes):
-// the same bits.  Tiles in the same grid-stride order.
+// 85 us a colour; here 62, L1 72% busy).  Four blocks per SM (64 registers, no
+// spills) take 0.6% off that workload's sweep against three.  The same terms in the
+// same order (the -x, +x pair commutes): the same bits.  Tiles in the same
+// grid-stride order.
 // ------------------------------------------------------------------------
 template <int CHUNK>
 __global__ void __launch_bounds__(kBlock, 4) row_field_kernel(GroupArgs g, uint32_t ntiles, int colour) {

@@ -12,8 +12,10 @@
 // site with their wraps) and three loads off a launch constant.  Walking a table
 // in shared memory instead, with the wraps and the address formed per entry,
 // cost 726 warp instructions per 32 sites of an fcc sub-set (25 us a pass of
-// 96^3 cells, 41% issued per cycle); the arithmetic on the spins, about 250, is
-// the rest.
+// 96^3 cells, 41% issued per cycle); here 360 to 440 and 17 to 21 us.  What bounds
+// it now is the latency of a site's 36 neighbour loads, which its draw and move
+// wait for (27 to 40% issued per cycle, 12 to 17 cycles of long-scoreboard stall
+// per instruction).
 #pragma once
 #include "kernels.h"
 #include "pass_impl.cuh"
