@@ -371,8 +371,10 @@ def gpu_arm(args, cfg):
         peak, peak_kind = measured_peak()
         traffic = read_traffic()
         # launches of the timed region: a wavefront pair is 2 x (1 + 2) launches;
-        # an odd last sweep runs every lattice on the two row passes
+        # an odd last sweep runs every lattice on the two row passes; one launch
+        # closes each sweep of the row lattices, one forms the samples of 16 sweeps
         launches = 3 * (args.steps - args.steps % 2) + 2 * (args.steps % 2) if kern_n[0] else 2 * args.steps
+        launches += args.steps + (args.steps + 15) // 16
 
         # end to end through the C ABI with host buffers: per step the whole
         # spin state goes host -> device from pinned memory, one measurement

@@ -783,13 +783,26 @@ int upload_wave_plan(const WavePlan& pl, const std::vector<LatDev*>& dev_lats, c
     return MC_OK;
 }
 
-// The device memory of a lattice's brick sweeps, on first use; false when it
-// cannot be had (none left, or the stream is being captured), and the sweeps
-// then run as launches.
-static bool brick_memory(BrickArgs* b, cudaStream_t s) {
-    if (b->ctl) return true;
+static bool capturing(cudaStream_t s) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    return cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
+// Allocations and waits of a sweep call are no part of a capture that another
+// thread has under way, and must not end it.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The device memory of a lattice's brick sweeps, on first use; false when it
+// cannot be had, or the stream is being captured, and the sweeps then run as
+// launches.
+static bool brick_memory(BrickArgs* b, cudaStream_t s) {
+    if (capturing(s)) return false;
+    if (b->ctl) return true;
+    RelaxedCapture relaxed;
     char* m = nullptr;
     if (cudaMalloc(reinterpret_cast<void**>(&m), b->bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -808,10 +821,9 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
 
 // The brick set of a group, on first use; false when it cannot be had.
 static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
-    if (b->failed) return false;
+    if (b->failed || capturing(s)) return false;
     if (b->mem) return true;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return false;
+    RelaxedCapture relaxed;
     b->failed = true;
     const size_t n = b->lats.size();
     std::vector<std::vector<BrickArgs>> args(3);  // by kernel instance: LAW 0, LAW 1, LAW 1 with odd rows
@@ -1071,7 +1083,11 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
         (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) ||
          (ls.brick_set && brick_set_ready(ls.brick_set, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
-    const int reps = n / kGraphSweeps;
+    // A call on a stream that the caller is capturing: a lattice that the resident
+    // sweeps can hold goes into the caller's graph whole, by launches where its
+    // sweeps are bricks; any other in calls of fewer than kGraphSweeps sweeps.
+    const bool whole = !constrained && ls.brick && ls.brick_lh == kResLh && !ls.brick->faces && capturing(s);
+    const int reps = whole ? 0 : n / kGraphSweeps;
     if (reps > 0) {
         cudaGraphExec_t& ex = gr.exec[constrained ? 1 : 0][measure ? 1 : 0];
         if (!ex) {

@@ -137,3 +137,40 @@ def test_brick_wait_that_runs_out_reports_timeout():
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=120,
                        env=dict(os.environ, MC_RESIDENT_INJECT_TIMEOUT="1", PYTHONPATH=ROOT))
     assert r.stdout.strip() == f"code {mc.MC_ERR_TIMEOUT}", r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("dims,n,used", [((128, 16, 16), 20, False), ((128, 16, 16), 5, True), ((32, 32, 32), 5, False),
+                                         ((48, 20, 24), 15, True)])
+def test_sweeps_captured_by_the_caller(dims, n, used):
+    """On a stream under capture the sweeps go into the caller's graph as
+    launches, whether the lattice has its brick memory (used) or not; a replay
+    is one more run of them.  Meanwhile another lattice's first brick launch,
+    on its own stream, neither fails nor ends the capture."""
+    torch = pytest.importorskip("torch")
+    st = torch.cuda.Stream()
+    kw = dict(K_u=0.03, T=0.7, seed=4)
+    spins = workloads.random_spins(dims[0] * dims[1] * dims[2], 8)
+    h = mc.mc_create_ex(mc.make_desc(dims, ring_capacity=64, stream=int(st.cuda_stream), **kw))
+    other = mc.mc_create_ex(mc.make_desc((16, 16, 16), T=0.5, seed=1))
+    ref = mc.mc_create_ex(mc.make_desc(dims, ring_capacity=64, kernel_path=mc.MC_PATH_ROW, **kw))
+    for x in (h, ref):
+        mc.mc_set_spins(x, spins)
+        mc.mc_sweep(x, 4 if used else 1)
+    mc.mc_sync(h)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(st):
+        graph.capture_begin()
+        mc.mc_sweep(h, n, measure=True)
+        mc.mc_sweep(other, 5)
+        graph.capture_end()
+        graph.replay()
+        graph.replay()
+    torch.cuda.synchronize()
+    mc.mc_sync(other)
+    mc.mc_sweep(ref, 2 * n, measure=True)
+    N = dims[0] * dims[1] * dims[2]
+    assert np.array_equal(mc.mc_get_spins(h, N), mc.mc_get_spins(ref, N))
+    assert mc.mc_measure(h).asdict() == mc.mc_measure(ref).asdict()
+    assert np.array_equal(mc.mc_samples(h, 64), mc.mc_samples(ref, 64))
+    for x in (h, other, ref):
+        mc.mc_destroy(x)
