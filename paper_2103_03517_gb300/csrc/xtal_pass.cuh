@@ -113,39 +113,60 @@ __device__ __forceinline__ XCell xtal_cell(const LatParams& p, int colour, uint3
     return c;
 }
 
-template <typename R, int TYPE, int J2, int SUB, bool HALF, int I>
-__device__ __forceinline__ void xtal_add(const XtalArgs& a, const XCell& c, int colour, V3<R>& h) {
+template <typename R, int TYPE, int J2, int SUB, bool HALF, int I = 0>
+__device__ __forceinline__ void xtal_load(const XtalArgs& a, const XCell& c, int colour, V3<R>* nb) {
     constexpr XtalEnt e = xtal_entry(TYPE, J2 != 0, SUB, I);
     if constexpr (!HALF || e.fwd) {
         const uint32_t q = c.kx[e.dx + 1] + c.ry[e.dy + 1] + c.rz[e.dz + 1];
         const R* b = static_cast<const R*>(a.spins) +
                      size_t(2 * e.t + ((colour + e.dx + e.dy + e.dz + 4) & 1)) * 3 * a.stride;
+        nb[I] = V3<R>{b[q], b[a.stride + q], b[2 * size_t(a.stride) + q]};
+    }
+    if constexpr (I + 1 < xtal_entries(TYPE, J2 != 0)) xtal_load<R, TYPE, J2, SUB, HALF, I + 1>(a, c, colour, nb);
+}
+
+template <typename R, int TYPE, int J2, int SUB, bool HALF, int I = 0>
+__device__ __forceinline__ void xtal_add(const XtalArgs& a, const V3<R>* nb, V3<R>& h) {
+    constexpr XtalEnt e = xtal_entry(TYPE, J2 != 0, SUB, I);
+    if constexpr (!HALF || e.fwd) {
         R J;
         if constexpr (kIsF64<R>) J = e.nn ? a.J : a.J2;
         else J = e.nn ? a.fJ : a.fJ2;
-        h.x = h.x + J * b[q];
-        h.y = h.y + J * b[a.stride + q];
-        h.z = h.z + J * b[2 * size_t(a.stride) + q];
+        h.x = h.x + J * nb[I].x;
+        h.y = h.y + J * nb[I].y;
+        h.z = h.z + J * nb[I].z;
     }
-    if constexpr (I + 1 < xtal_entries(TYPE, J2 != 0)) xtal_add<R, TYPE, J2, SUB, HALF, I + 1>(a, c, colour, h);
+    if constexpr (I + 1 < xtal_entries(TYPE, J2 != 0)) xtal_add<R, TYPE, J2, SUB, HALF, I + 1>(a, nb, h);
 }
 
 // h = sum over the neighbours of a site of sub-lattice SUB, colour `colour`, in
 // cell c, of J S_j.  HALF: the forward entries only (every bond once over the
-// lattice).
+// lattice).  Every neighbour is loaded before the first is added: taken entry by
+// entry, in the registers the compiler then chose, few of the 3 x 8 to 18 loads
+// were in flight and a site waited for L2 several times over.
 template <typename R, int TYPE, int J2, int SUB, bool HALF = false>
 __device__ __forceinline__ V3<R> xtal_field(const XtalArgs& a, const XCell& c, int colour) {
+    V3<R> nb[xtal_entries(TYPE, J2 != 0)];
+    xtal_load<R, TYPE, J2, SUB, HALF>(a, c, colour, nb);
     V3<R> h{R(0), R(0), R(0)};
-    xtal_add<R, TYPE, J2, SUB, HALF, 0>(a, c, colour, h);
+    xtal_add<R, TYPE, J2, SUB, HALF>(a, nb, h);
     return h;
 }
+
+// Blocks per SM that the kernels are compiled for: two in FP32, so that the loads
+// of a whole site fit the registers (80 to 128).  Blocks of 10 + 10 sweeps at two
+// / three / four: fcc 96^3 2310 / 2439, 64^3 1145 / 1341 / 1431, with J2 96^3 2650
+// / - / 2846 us, hcp 96^3 2297 / 2449, bcc 128^3 with J2 2493 / 2604, 64^3 774 / 777
+// / 800; without a bound (40 to 66 registers) fcc 96^3 2706.
+template <typename R>
+constexpr int kXtalMinb = kIsF64<R> ? 1 : 2;
 
 // ------------------------------------------------------------------- kernels
 // Pass over sub-set (SUB, colour); finalize != 0 closes the sweep (the last
 // sub-set of an unmeasured sweep).  Launched with programmatic serialisation:
 // its blocks start while the previous pass drains and wait for it here.
 template <typename R, int TYPE, int J2, int SUB>
-__global__ void __launch_bounds__(kBlock) xtal_pass_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
+__global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_pass_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
                                                            const R* __restrict__ cone, int colour, int finalize) {
     asm volatile("griddepcontrol.launch_dependents;");
     const LatParams& p = a.lat->p;
@@ -188,7 +209,7 @@ __global__ void __launch_bounds__(kBlock) xtal_pass_kernel(const __grid_constant
 // summed from the spins (which the pair passes keep in step; the sub-set's own
 // spins are not among its neighbours).
 template <typename R, int TYPE, int J2, int SUB>
-__global__ void __launch_bounds__(kBlock) xtal_field_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles, int colour) {
+__global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_field_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles, int colour) {
     const LatParams& p = a.lat->p;
     const WarpChunk wc = warp_chunk(ntiles);
     Spin4<R>* fld = static_cast<Spin4<R>*>(p.pfield);
@@ -216,7 +237,7 @@ __device__ __forceinline__ R xtal_dot(V3<R> S, V3<R> h) {
 // to fixed point on lane i (int64 in both precisions, so that large couplings
 // cannot overflow).  LEVEL 2: with the torques.
 template <typename R, int TYPE, int J2, int LEVEL>
-__global__ void __launch_bounds__(kBlock) xtal_sample_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
+__global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
                                                              uint32_t tiles_per_subset) {
     constexpr int NS = LEVEL >= 2 ? kNumSums : kSumTux;  // sums sampled
     asm volatile("griddepcontrol.launch_dependents;");
