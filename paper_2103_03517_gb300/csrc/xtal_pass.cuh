@@ -12,12 +12,12 @@
 // site with their wraps) and three loads off a launch constant.  Walking a table
 // in shared memory instead, with the wraps and the address formed per entry,
 // cost 726 warp instructions per 32 sites of an fcc sub-set (25 us a pass of
-// 96^3 cells, 41% issued per cycle); here 360 to 440 and 17 to 21 us.  What bounds
-// it now is the latency of a site's 36 neighbour loads, which its draw and move
-// wait for (27 to 40% issued per cycle, 12 to 17 cycles of long-scoreboard stall
-// per instruction).
+// 96^3 cells, 41% issued per cycle); here 342 and 14.5 us.  What bounds it now is
+// latency, of a site's loads and of its draw and move behind them: 38% issued per
+// cycle at 16 warps per SM.
 #pragma once
 #include "kernels.h"
+#include "pair_math.cuh"
 #include "pass_impl.cuh"
 
 namespace mcgb {
@@ -232,10 +232,12 @@ __device__ __forceinline__ R xtal_dot(V3<R> S, V3<R> h) {
 
 // Sample of the current state: M, the exchange sum over every bond once (sum_i
 // S_i . h_i over the forward entries), the uniaxial, cubic and torque sums;
-// tiles of 32 sites over the 2 nsub sub-sets; closes the sweep.  The warp sums
-// are reduced in the working precision in a fixed butterfly order and rounded
-// to fixed point on lane i (int64 in both precisions, so that large couplings
-// cannot overflow).  LEVEL 2: with the torques.
+// tiles of 32 sites over the 2 nsub sub-sets; closes the sweep.  FP64: the warp
+// sums of a tile are reduced in a fixed butterfly order and rounded to fixed
+// point on lane i (int64).  FP32: a lane adds its sites of 16 tiles in fixed
+// point before the warp adds the lanes, exact integers either way (a warp sum per
+// tile instead: bcc 48^3 591 against 551 us a block of 10 + 10 sweeps, fcc 32^3 748
+// against 704, 96^3 the same).  LEVEL 2: with the torques.
 template <typename R, int TYPE, int J2, int LEVEL>
 __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
                                                              uint32_t tiles_per_subset) {
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const
     const Par<R> par = load_par<R>(p);
     const V3<R> e_ax{par.e[0], par.e[1], par.e[2]};
     long long fix = 0;
+    int lf[NS] = {}, nparts = 0;
     for (uint32_t tile = wc.begin; tile < wc.end; ++tile) {
         const uint32_t set = tile / tiles_per_subset;  // 2 sub + colour
         const int sub = int(set >> 1), colour = int(set & 1u);
@@ -272,8 +275,16 @@ __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const
         if constexpr (kIsF64<R>) {
             fix += __double2ll_rn(warp_sums_f64<NS>(sums.v, lane) * kFixScale);
         } else {
-            fix += warp_tile_fix<R, NS>(sums, lane);  // per-lane fixed point, integer warp sums
+#pragma unroll
+            for (int i = 0; i < NS; ++i) lf[i] += __float2int_rn(sums.v[i] * float(kFixScaleF32));
+            if (++nparts == kPartTiles) {
+                fix += pair_parts_flush<NS>(lf, lane);
+                nparts = 0;
+            }
         }
+    }
+    if constexpr (!kIsF64<R>) {
+        if (nparts) fix += pair_parts_flush<NS>(lf, lane);
     }
     publish(a.lat->st, lane, 0, true, fix, 3, wc.end - wc.begin, ntiles, true,
             [&] { finalize_sweep(p, a.lat->st, 1, LEVEL >= 2, lane); });

@@ -42,3 +42,18 @@ def test_crystal_instances_equal_the_oracle(lattice, J2, cells):
         np.testing.assert_allclose([ob.ml, ob.e], [st["ml"], st["e"]], rtol=0, atol=1e-9)
     finally:
         mc.mc_destroy(h)
+
+
+@pytest.mark.parametrize("crystal,L", [(mc.MC_FCC, 80), (mc.MC_BCC, 100)])
+def test_sample_of_many_tiles_a_warp(crystal, L):
+    """More than 16 tiles a warp, so that the lanes' integer parts are summed over
+    several runs.  Each site's m_a is rounded once, at 2^-22: the mean is within
+    2^-23 of the mean of the spins."""
+    h = mc.mc_create_ex(mc.make_desc((L, L, L), K_u=0.02, T=1.2, seed=6, lattice=crystal, ring_capacity=4))
+    N = L ** 3 * (4 if crystal == mc.MC_FCC else 2)
+    mc.mc_sweep(h, 3)
+    mc.mc_sweep(h, 1, measure=True)
+    m = np.asarray(mc.mc_get_spins(h, N), dtype=np.float64).mean(axis=0)
+    o = mc.mc_measure(h)
+    mc.mc_destroy(h)
+    assert np.max(np.abs(np.asarray(o.m) - m)) <= 2.0 ** -23
