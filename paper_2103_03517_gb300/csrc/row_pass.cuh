@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 // spins instead of the packed copy (the pair passes keep both in step): two
 // sites a lane, x neighbours by shuffle, so that 64 sites take 15 8-byte loads a
 // lane where the other takes 12 of 16 bytes, which kept L1 91% busy (80 x 64^3:
-// 85 us a colour; here 62, L1 72% busy).  Four blocks per SM (64 registers, no
-// spills) take 0.6% off that workload's sweep against three.  The same terms in the
+// 85 us a colour; here 62, L1 72% busy).  Four blocks per SM (64 registers, 8
+// bytes spilled) take 0.6% off that workload's sweep against three.  The same terms in the
 // same order (the -x, +x pair commutes): the same bits.  Tiles in the same
 // grid-stride order.
 // ------------------------------------------------------------------------
