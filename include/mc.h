@@ -557,7 +557,9 @@ MC_API int mc_slab_sweep(const mc_handle* slabs, int n, int n_sweeps, int measur
  * spins     device memory, FP32, colour-split layout of mc_export_state:
  *           6 * stride floats, stride = N/2 rounded up to a multiple of 64,
  *           component a of colour c at spins[(3c + a) stride + q]; updated
- *           in place
+ *           in place.  Any float pointer: one that is not 8-byte aligned takes
+ *           the general kernel's arithmetic (see MC_PATH_GENERAL), whose chain
+ *           may differ in the last bits from the row kernels'
  * dims...   a periodic lattice as for mc_create (every size even)
  * first_sweep  sweep counter of the chain (0 for a new chain; a continuing
  *           chain passes the previous first_sweep + n_sweeps)
@@ -567,8 +569,9 @@ MC_API int mc_slab_sweep(const mc_handle* slabs, int n, int n_sweeps, int measur
  *           samples every sweep is a measurement sweep
  * stream    cudaStream_t (NULL = default stream); the call synchronises it
  *           before returning (to read theta back)
- * Errors: MC_ERR_ARG for invalid sizes or parameters, and for n_sweeps > 256
- * with samples (the scratch holds 256 samples per call); MC_ERR_CUDA. */
+ * Errors: MC_ERR_ARG for invalid sizes or parameters, spins not aligned to a
+ * float, and n_sweeps > 256 with samples (the scratch holds 256 samples per
+ * call); MC_ERR_CUDA; MC_ERR_TIMEOUT. */
 MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J, double K_u, const double axis[3],
                             double K_c, const double H[3], double T, uint64_t seed, int64_t first_sweep,
                             int n_sweeps, int* theta_deg, double* samples, void* stream);

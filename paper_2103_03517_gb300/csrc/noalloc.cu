@@ -7,6 +7,7 @@
 
 #include <cmath>
 #include <cstddef>
+#include <cstdint>
 #include <cstring>
 
 #include "runtime.h"
@@ -80,6 +81,8 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     int rc = validate_desc(&d);
     if (rc) return rc;
     if (n_sweeps == 0) return MC_OK;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(spins);
+    if (at % alignof(float)) return fail(MC_ERR_ARG, "spins must be aligned to a float");
 
     char* base = nullptr;
     rc = scratch_address(g_scratch, &base);
@@ -107,7 +110,9 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
     p.nblocks_pair = (p.n_pairs + 31) / 32 > 0 ? (p.n_pairs + 31) / 32 : 1;
     p.sample_torque = 1;
     p.row_fast = row_fast(p, false);
-    p.colour_kernel = colour_kernel(p, false, MC_PATH_AUTO);
+    // the row kernels move the caller's spins as float2; the general kernel, and
+    // brick sweeps by its law, take any float pointer
+    p.colour_kernel = colour_kernel(p, false, at % alignof(float2) ? MC_PATH_GENERAL : MC_PATH_AUTO);
     p.row_lanes = p.Lh / 2 < 32 ? (p.Lh / 2 > 0 ? p.Lh / 2 : 1) : 32;
     p.spins = spins;
     p.ring = reinterpret_cast<double*>(base + kOffRing);
