@@ -28,9 +28,11 @@
 //
 // Packets.  The packet of a site is rewritten two passes after it was read:
 // by then its writer has read the reader's own packet of the pass between,
-// which the reader stored after its read.  Tags are (epoch + 1) * 8192 + pass +
-// 1 (pass -1: the state at the start), the epoch counted up by every launch, so
-// no packet of an earlier launch, and none of zeroed memory, can match.
+// which the reader stored after its read.  Tags hold the pass and an epoch that
+// every launch counts up, so that no packet of an earlier launch, and none of
+// zeroed memory, can match (brick_tag0; before the epochs repeat the packets are
+// cleared, since a lattice swept alone, in a group, or in memory that several
+// sizes share does not write the same packets in every launch).
 //
 // Cone angle.  Every block adds its accepted count of a sweep and its arrival
 // to one word (running totals, one word per parity of the sweep: a block adds
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         }
     int theta = L->st.theta;
     const uint32_t sweep0 = L->st.sweep;
-    const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch), T0 = (epoch + 1u) << 13;
+    const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch), T0 = brick_tag0(epoch);
     const Par<float> par = load_par<float>(p);
     const bool adapt = MEASURE == 0 || p.adapt_in_measure;
     __syncthreads();
@@ -628,17 +630,23 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         }
 }
 
-// Before a launch of several lattices: their control words (not the epochs) and
-// the records of n measured sweeps zeroed, as the memsets of a lattice alone do.
+// Before a launch (of one lattice, or of many, by blockIdx.y): the control words
+// (not the epoch) and the records of n measured sweeps zeroed, and before a
+// launch whose epoch brick_clears all packets of the memory as well.
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS) brick_prep_kernel(const BrickArgs* many, int n) {
-    const BrickArgs& a = many[blockIdx.y];
-    const int i = int(blockIdx.x) * THREADS + int(threadIdx.x);
-    if (i < n * kRecordWords) a.record[i] = 0;
+__global__ void __launch_bounds__(THREADS) brick_prep_kernel(const __grid_constant__ BrickArgs one, const BrickArgs* many,
+                                                             int n) {
+    const BrickArgs& a = many ? many[blockIdx.y] : one;
+    const uint32_t i = blockIdx.x * uint32_t(THREADS) + threadIdx.x;
+    if (i < uint32_t(n * kRecordWords)) a.record[i] = 0;
     if (i == 0) {
         a.ctl->abort = 0;
         a.ctl->closed = 0;
         a.ctl->count[0] = a.ctl->count[1] = 0;
+    }
+    if (brick_clears(a.ctl->epoch)) {
+        float4* const p = static_cast<float4*>(a.packets);
+        for (uint32_t k = i; k < a.n_packets; k += gridDim.x * uint32_t(THREADS)) p[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 }
 

@@ -56,6 +56,13 @@ cudaError_t launch_any(const BrickArgs& a, uint32_t Lh, const float* cone, int m
                    : launch_m<1, 0, 0>(a, g, b, a.smem, cone, measure, s);
 }
 
+// What comes before a launch: brick_prep_kernel on lattice `one`, or on `many`;
+// n measured sweeps.
+cudaError_t prep(const BrickArgs& one, const BrickArgs* many, int lattices, int n, cudaStream_t s) {
+    brick_prep_kernel<256><<<dim3(uint32_t(n * kRecordWords / 256 + 1), uint32_t(lattices)), 256, 0, s>>>(one, many, n);
+    return cudaGetLastError();
+}
+
 struct Device {
     uint32_t most, cap;  // blocks at once, shared memory of a block
 };
@@ -169,9 +176,7 @@ cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int 
     for (int done = 0; done < n;) {
         BrickArgs a = b;
         a.n_sweeps = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
-        cudaError_t e = cudaMemsetAsync(a.ctl, 0, offsetof(BrickCtl, epoch), s);
-        if (e == cudaSuccess && measure)
-            e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kRecordWords * sizeof(long long), s);
+        cudaError_t e = prep(a, nullptr, 1, measure ? a.n_sweeps : 0, s);
         if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
         if (e == cudaSuccess && measure) {
             brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, static_cast<const BrickArgs*>(nullptr), a.n_sweeps);
@@ -189,9 +194,7 @@ cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int
         const int m = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
         const BrickGroup g{c.args, c.first, c.n, m};
         const BrickArgs none{};
-        const int words = (measure ? m : 0) * kRecordWords;
-        brick_prep_kernel<256><<<dim3(uint32_t(words / 256 + 1), uint32_t(c.n)), 256, 0, s>>>(c.args, measure ? m : 0);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = prep(none, c.args, c.n, measure ? m : 0, s);
         if (e == cudaSuccess)
             e = c.law == 0 ? launch_m<0, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s)
                 : c.odd    ? launch_m<1, 0, 1, 1>(none, g, c.blocks, c.smem, c32, measure, s)

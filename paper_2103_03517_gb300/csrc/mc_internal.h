@@ -11,6 +11,7 @@
 // k + xoff - 1 and k + xoff in the same row, and the -y/+y/-z/+z neighbours
 // share k in the adjacent rows.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 namespace mcgb {
@@ -266,6 +267,22 @@ struct BrickCtl {
 
 constexpr int kBrickMaxMeasured = 512;  // measured sweeps per launch
 
+// Tags of a brick launch's packets: brick_tag0(epoch) + pass + 1 (pass -1: the
+// state at the start).  Their low bits are 1 ... 4097, so zeroed memory never
+// carries a tag.  They repeat after 2^19 launches; a launch of an epoch that
+// brick_clears has its packets zeroed first (brick_prep_kernel), so that no
+// packet in memory is that old.
+#ifdef __CUDACC__
+#define MC_HD __host__ __device__
+#else
+#define MC_HD
+#endif
+constexpr int kBrickTagBits = 13;
+constexpr uint32_t kBrickEpochs = 1u << (32 - kBrickTagBits);
+static_assert(2 * kResMaxSweeps + 1 < 1 << kBrickTagBits, "a launch's tags are its epoch's");
+MC_HD inline uint32_t brick_tag0(uint32_t epoch) { return (epoch << kBrickTagBits) + 1u; }
+MC_HD inline bool brick_clears(uint32_t epoch) { return epoch % kBrickEpochs == kBrickEpochs - 1u; }
+
 // A brick launch: nyc x nzc bricks of rows (odd Lh: nyc blocks, runs of
 // rows), at most `rows` rows in a block; packets: 16 bytes per site, [2]
 // [stride]; inject as in ResidentArgs.
@@ -278,6 +295,8 @@ struct BrickArgs {
     FastDiv div_half;     // by Lh / 2
     int off;              // it does not fit, or its launch was refused: swept by launches
     size_t bytes;         // of the lattice's brick memory: ctl (null until it is allocated), record, packets
+    uint32_t n_packets;   // of that memory (of all sizes that share it)
+    uint32_t epoch0;      // first epoch (fault injection)
     int law, faces;       // kernel instance: packed or scalar law, any boundaries
     int n_sweeps;
     int inject;

@@ -161,6 +161,7 @@ extern "C" MC_API int mc_sweep_noalloc(float* spins, const int dims[3], double J
         brick.ctl = reinterpret_cast<BrickCtl*>(mem);
         brick.record = reinterpret_cast<long long*>(mem + kBrickOffRecord);
         brick.packets = mem + kBrickOffPackets;
+        brick.n_packets = uint32_t(kBrickSpins);
         brick.key0 = p.key0;
         brick.key1 = p.key1;
         ls.brick = &brick;

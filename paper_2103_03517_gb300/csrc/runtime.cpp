@@ -515,6 +515,9 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
         b.faces = p.bc[0] || p.bc[1] || p.bc[2] ? 1 : 0;
         const char* inj = std::getenv("MC_RESIDENT_INJECT_TIMEOUT");  // as for the resident sweeps
         b.inject = inj && inj[0] == '1' ? 1 : 0;
+        b.n_packets = 2 * p.stride;
+        const char* first = std::getenv("MC_BRICK_FIRST_EPOCH");  // for the tests of the epochs' wrap
+        b.epoch0 = first ? uint32_t(std::strtoul(first, nullptr, 10)) : 0u;
         h->brick = new BrickArgs(b);
     }
     if (size_t(cur - static_cast<char*>(h->d_base)) > h->bytes) {
@@ -809,7 +812,10 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
         return false;
     }
     // zero, so that no packet of uninitialised memory carries a tag
-    if (cudaMemsetAsync(m, 0, b->bytes, s) != cudaSuccess) {
+    cudaError_t e = cudaMemsetAsync(m, 0, b->bytes, s);
+    if (e == cudaSuccess && b->epoch0)
+        e = cudaMemcpyAsync(&reinterpret_cast<BrickCtl*>(m)->epoch, &b->epoch0, sizeof b->epoch0, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) {
         cudaFree(m);
         return false;
     }
