@@ -12,15 +12,8 @@ namespace {
 template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
 cudaError_t launch(const BrickArgs& a, const BrickGroup& g, uint32_t blocks, uint32_t smem, const float* cone,
                    cudaStream_t s) {
-    static const bool ok = [] {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        return cudaFuncSetAttribute(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin - int(kResStaticSmem)) == cudaSuccess;
-    }();
-    if (!ok) return cudaErrorInvalidConfiguration;
+    const cudaError_t opt = opt_in_smem(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>);
+    if (opt != cudaSuccess) return opt;
     // cooperative: the launch fails rather than run with a block not resident
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);

@@ -156,12 +156,10 @@ void pair_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour
 }
 
 // The wavefront kernel takes more than the default 48 KB of dynamic shared
-// memory: opt in once per instance.
+// memory (opt_in_smem).
 template <int MEASURE>
 bool wave_opt_in() {
-    static const bool ok = cudaFuncSetAttribute(wave_sweep_kernel<MEASURE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                int(kWaveSmemBytes)) == cudaSuccess;
-    return ok;
+    return opt_in_smem(wave_sweep_kernel<MEASURE>, int(kWaveSmemBytes)) == cudaSuccess;
 }
 
 template <int MEASURE>
@@ -204,14 +202,7 @@ uint32_t wave_blocks() {
 // largest brick.
 template <int NT, int MEASURE>
 bool resident_opt_in() {
-    static const bool ok = [] {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        return cudaFuncSetAttribute(resident_sweep_kernel<NT, MEASURE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin - int(kResStaticSmem)) == cudaSuccess;
-    }();
-    return ok;
+    return opt_in_smem(resident_sweep_kernel<NT, MEASURE>) == cudaSuccess;
 }
 
 template <int NT, int MEASURE>

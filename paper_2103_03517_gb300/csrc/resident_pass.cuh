@@ -54,6 +54,21 @@ constexpr int kResRow = 3 * kResLh;  // floats of one row of one colour: [3][64]
 constexpr long long kResWaitCycles = 1ll << 31;  // about one second at 2 GHz
 constexpr uint32_t kResStaticSmem = 1024;        // bound on the kernel's static shared memory
 
+// Lets launches of a kernel on the current device take `bytes` of dynamic shared
+// memory (0: all that the device allows).  The permission is the current device's,
+// so it is asked for before every launch and not once per process, whose other
+// devices would then refuse the launch.
+template <typename K>
+cudaError_t opt_in_smem(K kernel, int bytes = 0) {
+    if (bytes == 0) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        bytes -= int(kResStaticSmem);
+    }
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // Halo rows of a brick of at most by x bz rows: the rows beside its y faces
 // (2 bz, when y is split) and beside its z faces (2 by, when z is split).
 __host__ __device__ inline uint32_t resident_halo_rows(int by, int bz, int nyc, int nzc) {
