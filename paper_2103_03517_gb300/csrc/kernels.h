@@ -173,14 +173,16 @@ struct LaunchSet {
 // Brick sweeps (brick_pass.cuh; FP32 simple cubic lattices without film
 // tables): the split of lattice p (host copy) over the current device's SMs,
 // everything of out but its pointers and key; false when its rows do not fit
-// their shared memory.  Then n sweeps of a plan in cooperative launches of at
-// most kResMaxSweeps, measure as for colour_pass.
+// their shared memory.  Then n sweeps of a plan in one cooperative launch (at
+// most kResMaxSweeps, or kBrickMaxMeasured measured), measure as for colour_pass;
+// *ran: the launch was accepted (if not, nothing of it ran).
 bool brick_plan(const LatParams& p, BrickArgs* out);
 // The splits of several lattices swept side by side, each with blocks of its
 // own (splits only: out[i] keeps its pointers and key): the estimated us of a
 // sweep of the slowest, or 0 when they do not fit the SMs together.
 double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<BrickArgs>* out);
-cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, cudaStream_t s);
+cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, bool* ran,
+                         cudaStream_t s);
 // The same for lattices of one kernel instance (law, no faces, parity of Lh):
 // their plans and first blocks in device memory, blocks and shared memory of
 // the launch.
@@ -189,8 +191,9 @@ struct BrickClass {
     uint32_t* first = nullptr;
     int n = 0, law = 0, odd = 0;
     uint32_t blocks = 0, smem = 0;
+    int refuse = 0;  // the most of its lattices' (BrickArgs::refuse)
 };
-cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, cudaStream_t s);
+cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, bool* ran, cudaStream_t s);
 
 const KernelSet& kernels_f64();
 const KernelSet& kernels_f32();

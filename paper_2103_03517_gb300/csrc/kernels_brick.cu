@@ -12,6 +12,7 @@ namespace {
 template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
 cudaError_t launch(const BrickArgs& a, const BrickGroup& g, uint32_t blocks, uint32_t smem, const float* cone,
                    cudaStream_t s) {
+    if ((GROUP ? g.n_sweeps : a.n_sweeps) < a.refuse) return cudaErrorInvalidValue;
     const cudaError_t opt = opt_in_smem(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>);
     if (opt != cudaSuccess) return opt;
     // cooperative: the launch fails rather than run with a block not resident
@@ -165,41 +166,36 @@ double brick_group_plan(const std::vector<const LatParams*>& lats, std::vector<B
     return 2.0 * slowest;
 }
 
-cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, cudaStream_t s) {
-    for (int done = 0; done < n;) {
-        BrickArgs a = b;
-        a.n_sweeps = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
-        cudaError_t e = prep(a, nullptr, 1, measure ? a.n_sweeps : 0, s);
-        if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
-        if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, static_cast<const BrickArgs*>(nullptr), a.n_sweeps);
-            e = cudaGetLastError();
-        }
-        if (e != cudaSuccess) return e;
-        done += a.n_sweeps;
+cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int n, int measure, bool* ran,
+                         cudaStream_t s) {
+    BrickArgs a = b;
+    a.n_sweeps = n;
+    cudaError_t e = prep(a, nullptr, 1, measure ? n : 0, s);
+    if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
+    *ran = e == cudaSuccess;
+    if (*ran && measure) {
+        brick_close_kernel<4><<<(n + 3) / 4, 128, 0, s>>>(a, static_cast<const BrickArgs*>(nullptr), n);
+        e = cudaGetLastError();
     }
-    return cudaSuccess;
+    return e;
 }
 
-cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, cudaStream_t s) {
+cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int measure, bool* ran, cudaStream_t s) {
     const float* c32 = static_cast<const float*>(cone);
-    for (int done = 0; done < n;) {
-        const int m = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
-        const BrickGroup g{c.args, c.first, c.n, m};
-        const BrickArgs none{};
-        cudaError_t e = prep(none, c.args, c.n, measure ? m : 0, s);
-        if (e == cudaSuccess)
-            e = c.law == 0 ? launch_m<0, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s)
-                : c.odd    ? launch_m<1, 0, 1, 1>(none, g, c.blocks, c.smem, c32, measure, s)
-                           : launch_m<1, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s);
-        if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<dim3(uint32_t(m + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, static_cast<const BrickArgs*>(c.args), m);
-            e = cudaGetLastError();
-        }
-        if (e != cudaSuccess) return e;
-        done += m;
+    const BrickGroup g{c.args, c.first, c.n, n};
+    BrickArgs none{};
+    none.refuse = c.refuse;
+    cudaError_t e = prep(none, c.args, c.n, measure ? n : 0, s);
+    if (e == cudaSuccess)
+        e = c.law == 0 ? launch_m<0, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s)
+            : c.odd    ? launch_m<1, 0, 1, 1>(none, g, c.blocks, c.smem, c32, measure, s)
+                       : launch_m<1, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s);
+    *ran = e == cudaSuccess;
+    if (*ran && measure) {
+        brick_close_kernel<4><<<dim3(uint32_t(n + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, static_cast<const BrickArgs*>(c.args), n);
+        e = cudaGetLastError();
     }
-    return cudaSuccess;
+    return e;
 }
 
 }  // namespace mcgb

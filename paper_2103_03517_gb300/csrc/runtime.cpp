@@ -517,6 +517,8 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
         b.inject = inj && inj[0] == '1' ? 1 : 0;
         b.n_packets = 2 * p.stride;
         const char* first = std::getenv("MC_BRICK_FIRST_EPOCH");  // for the tests of the epochs' wrap
+        const char* ref = std::getenv("MC_BRICK_INJECT_REFUSAL");  // for the tests of refused launches
+        b.refuse = ref ? std::atoi(ref) : 0;
         b.epoch0 = first ? uint32_t(std::strtoul(first, nullptr, 10)) : 0u;
         h->brick = new BrickArgs(b);
     }
@@ -833,6 +835,7 @@ static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
     b->failed = true;
     const size_t n = b->lats.size();
     std::vector<std::vector<BrickArgs>> args(3);  // by kernel instance: LAW 0, LAW 1, LAW 1 with odd rows
+    std::vector<std::vector<mc_lattice*>> lats(3);
     for (size_t i = 0; i < n; ++i) {
         BrickArgs* own = b->lats[i]->brick;
         if (!brick_memory(own, s)) return false;
@@ -844,7 +847,9 @@ static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
         a.smem = plan.smem;
         a.div_half = plan.div_half;
         a.law = plan.law;
-        args[a.law == 0 ? 0 : 1 + b->lats[i]->hp.Lh % 2].push_back(a);
+        const int k = a.law == 0 ? 0 : 1 + b->lats[i]->hp.Lh % 2;
+        args[k].push_back(a);
+        lats[k].push_back(b->lats[i]);
     }
     std::vector<char> host;
     std::vector<size_t> at;
@@ -873,19 +878,41 @@ static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
             f[i] = c.blocks;
             c.blocks += v[i].nyc * v[i].nzc;
             c.smem = std::max(c.smem, v[i].smem);
+            c.refuse = std::max(c.refuse, v[i].refuse);
         }
         f[v.size()] = c.blocks;
         b->classes.push_back(c);
+        b->members.push_back(lats[k]);
     }
     if (cudaMemcpyAsync(mem, host.data(), host.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaFree(mem);
         b->classes.clear();
+        b->members.clear();
         return false;
     }
     b->mem = mem;
     b->failed = false;
     return true;
+}
+
+// Whether a cooperative launch that did not run was refused, for its size or by a
+// device or context that does not allow it: what it was to sweep is swept by
+// launches.
+static bool launch_refused(cudaError_t e) {
+    switch (e) {
+        case cudaErrorCooperativeLaunchTooLarge:
+        case cudaErrorInvalidValue:
+        case cudaErrorInvalidConfiguration:
+        case cudaErrorInvalidDeviceFunction:
+        case cudaErrorLaunchOutOfResources:
+        case cudaErrorMemoryAllocation:
+        case cudaErrorNotSupported:
+            cudaGetLastError();
+            return true;
+        default:
+            return false;
+    }
 }
 
 // Enqueue n sweeps of the lattices of a launch set; with events != nullptr
@@ -919,42 +946,52 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         return MC_OK;
     }
-    // a launch that the device refuses as too large for it (a context with fewer
-    // SMs) leaves the lattices as they were, and they are swept by launches
-    auto refused = [&](cudaError_t e, int done) {
-        if (e != cudaErrorCooperativeLaunchTooLarge || done) return false;
-        cudaGetLastError();
-        return true;
-    };
+    // brick launches; after a refused one (launch_refused) the remaining sweeps
+    // of its lattices go by launches, and so do later calls
+    const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
     if (!constrained && ls.brick && !ls.brick->off && n >= kResMinSweeps && brick_memory(ls.brick, s)) {
-        cudaError_t e = cudaSuccess;
-        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
-        for (int done = 0; done < n && e == cudaSuccess && !ls.brick->off; done += most)
+        for (int done = 0; done < n;) {
+            cudaError_t e = cudaSuccess;
+            bool ran = false;
+            const int m = std::min(n - done, most);
             timed_kind(kTimedResident, [&] {
-                e = brick_sweeps(*ls.brick, ls.brick_lh, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
-                if (refused(e, done)) ls.brick->off = 1;
+                e = brick_sweeps(*ls.brick, ls.brick_lh, cone, m, measure ? ls.sample_level : 0, &ran, s);
             });
-        if (!ls.brick->off) {
+            if (!ran && launch_refused(e)) {
+                ls.brick->off = 1;
+                n -= done;
+                break;
+            }
             if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
-            return MC_OK;
+            done += m;
         }
-    }
-    if (!constrained && ls.brick_set && n >= kResMinSweeps && brick_set_ready(ls.brick_set, s)) {
-        cudaError_t e = cudaSuccess;
-        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
-        int launches = 0;
-        for (int done = 0; done < n; done += most)
-            for (const BrickClass& c : ls.brick_set->classes)
-                if (e == cudaSuccess)
-                    timed_kind(kTimedResident, [&] {
-                        e = brick_group_sweeps(c, cone, std::min(n - done, most), measure ? ls.sample_level : 0, s);
-                        if (refused(e, launches)) ls.brick_set->failed = true;
-                        ++launches;
-                    });
-        if (!ls.brick_set->failed) {
-            if (e != cudaSuccess) return cuda_fail(e, "brick sweep launch");
-            return MC_OK;
-        }
+        if (!ls.brick->off) return MC_OK;
+    } else if (!constrained && ls.brick_set && n >= kResMinSweeps && brick_set_ready(ls.brick_set, s)) {
+        BrickSet& set = *ls.brick_set;
+        for (size_t c = 0; c < set.classes.size(); ++c)
+            for (int done = 0; done < n;) {
+                cudaError_t e = cudaSuccess;
+                bool ran = false;
+                int m = std::min(n - done, most);
+                timed_kind(kTimedResident, [&] {
+                    e = brick_group_sweeps(set.classes[c], cone, m, measure ? ls.sample_level : 0, &ran, s);
+                });
+                if (!ran && launch_refused(e)) {
+                    set.failed = true;
+                    m = n - done;
+                    for (mc_lattice* h : set.members[c]) {
+                        LaunchSet one = single_launch_set(h);
+                        one.brick = nullptr;
+                        one.n_res = 0;
+                        const int rc = enqueue_sweeps(k, one, cone, m, measure, constrained, s, events);
+                        if (rc) return rc;
+                    }
+                } else if (e != cudaSuccess) {
+                    return cuda_fail(e, "brick sweep launch");
+                }
+                done += m;
+            }
+        return MC_OK;
     }
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
     auto kind_pass = [&](int kind, const GroupArgs& ga, uint32_t nt, int colour, int meas) {

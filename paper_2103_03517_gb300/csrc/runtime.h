@@ -50,6 +50,7 @@ struct BrickSet {
     std::vector<mc_lattice*> lats;
     std::vector<BrickArgs> plans;  // splits, one per lattice
     std::vector<BrickClass> classes;
+    std::vector<std::vector<mc_lattice*>> members;  // of each class
     void* mem = nullptr;           // the classes' device arrays
     bool failed = false;
     BrickSet() = default;
