@@ -300,6 +300,7 @@ struct BrickArgs {
     int law, faces;       // kernel instance: packed or scalar law, any boundaries
     int n_sweeps;
     int inject;
+    int nomem;            // requests for memory that are still to fail (fault injection)
     int refuse;           // launches of fewer sweeps than this are refused (fault injection)
     uint32_t key0, key1;  // the lattice's Philox key, a launch constant
 };

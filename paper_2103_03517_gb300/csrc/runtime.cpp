@@ -519,6 +519,8 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
         const char* first = std::getenv("MC_BRICK_FIRST_EPOCH");  // for the tests of the epochs' wrap
         const char* ref = std::getenv("MC_BRICK_INJECT_REFUSAL");  // for the tests of refused launches
         b.refuse = ref ? std::atoi(ref) : 0;
+        const char* nomem = std::getenv("MC_BRICK_INJECT_NOMEM");  // for the tests without their memory
+        b.nomem = nomem ? std::atoi(nomem) : 0;
         b.epoch0 = first ? uint32_t(std::strtoul(first, nullptr, 10)) : 0u;
         h->brick = new BrickArgs(b);
     }
@@ -801,16 +803,18 @@ struct RelaxedCapture {
     ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-// The device memory of a lattice's brick sweeps, on first use; false when it
-// cannot be had, or the stream is being captured, and the sweeps then run as
-// launches.
+// The device memory of a lattice's brick sweeps, on first use; false when the
+// stream is being captured, and the sweeps then run as launches, or when it
+// cannot be had: they then run as launches from now on, with no further request.
 static bool brick_memory(BrickArgs* b, cudaStream_t s) {
-    if (capturing(s)) return false;
+    if (b->off || capturing(s)) return false;
     if (b->ctl) return true;
     RelaxedCapture relaxed;
     char* m = nullptr;
-    if (cudaMalloc(reinterpret_cast<void**>(&m), b->bytes) != cudaSuccess) {
-        cudaGetLastError();
+    if (b->nomem > 0 || cudaMalloc(reinterpret_cast<void**>(&m), b->bytes) != cudaSuccess) {
+        if (b->nomem > 0) --b->nomem;
+        else cudaGetLastError();
+        b->off = 1;
         return false;
     }
     // zero, so that no packet of uninitialised memory carries a tag
@@ -819,6 +823,7 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
         e = cudaMemcpyAsync(&reinterpret_cast<BrickCtl*>(m)->epoch, &b->epoch0, sizeof b->epoch0, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) {
         cudaFree(m);
+        b->off = 1;
         return false;
     }
     b->ctl = reinterpret_cast<BrickCtl*>(m);
