@@ -376,7 +376,8 @@ MC_API int mc_group_sync(mc_group_handle g);
  *   row:   FP32 row kernel, minimum resident blocks per SM (so registers per
  *          thread): {3, 2} (boundaries and films: 2 in passes with a sample);
  *          a lattice swept resident (MC_PATH_RESIDENT): threads per block
- *          {512, 640};
+ *          {512, 640}; lattices that sweep as bricks: the launches that their
+ *          calls of one or two sweeps take;
  *   field: constrained neighbour-field kernel, tiles per grid-stride step
  *          {4, 8, 2};
  *   pair:  constrained pair pass, the same {4, 8, 2}, then 4 tiles per step

@@ -61,6 +61,11 @@ int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats,
     if (sweeps < 1 || !(what & (MC_TUNE_SWEEP | MC_TUNE_CONSTRAINED))) return fail(MC_ERR_ARG, "invalid argument");
     bool row_kernel = false;
     for (int c = kColourRow; c < kColourKinds; ++c) row_kernel = row_kernel || ls.nt_col[c];
+    // the knobs are those of launches: sweeps that would run as bricks are timed as
+    // the launches that their calls of one or two sweeps take
+    LaunchSet lt = ls;
+    lt.brick = nullptr;
+    lt.brick_set = nullptr;
     const bool tune_free = (what & MC_TUNE_SWEEP) && row_kernel;
     const bool tune_cons = (what & MC_TUNE_CONSTRAINED) && (ls.nt_pairs || ls.nt_pairs_lead);
     for (mc_lattice* h : lats) {
@@ -100,10 +105,10 @@ int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats,
         const KernelSet& k = kernel_set(precision);
         // mean ms per sweep of `sweeps` sweeps after one untimed, then restore
         auto trial = [&](bool constrained, double& ms) -> int {
-            int r = enqueue_sweeps(k, ls, cone, 1, 0, constrained, s, nullptr);
+            int r = enqueue_sweeps(k, lt, cone, 1, 0, constrained, s, nullptr);
             if (!r) {
                 cudaEventRecord(a, s);
-                r = enqueue_sweeps(k, ls, cone, sweeps, 0, constrained, s, nullptr);
+                r = enqueue_sweeps(k, lt, cone, sweeps, 0, constrained, s, nullptr);
                 cudaEventRecord(b, s);
             }
             if (!r) {
@@ -135,14 +140,15 @@ int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats,
             choice = pick;
             return MC_OK;
         };
-        if (!rc && tune_free) rc = knob(ls.shape.row, kRowShapes, rep.row_ms, false);
-        if (!rc && tune_cons) rc = knob(ls.shape.field, kFieldShapes, rep.field_ms, true);
-        if (!rc && tune_cons) rc = knob(ls.shape.pair, kPairShapes, rep.pair_ms, true);
+        if (!rc && tune_free) rc = knob(lt.shape.row, kRowShapes, rep.row_ms, false);
+        if (!rc && tune_cons) rc = knob(lt.shape.field, kFieldShapes, rep.field_ms, true);
+        if (!rc && tune_cons) rc = knob(lt.shape.pair, kPairShapes, rep.pair_ms, true);
         const cudaError_t es = cudaStreamSynchronize(s);
         cudaEventDestroy(a);
         cudaEventDestroy(b);
         if (rc) return rc;
         if (es != cudaSuccess) return cuda_fail(es, "autotune sync");
+        ls.shape = lt.shape;
         rep.row = ls.shape.row;
         rep.field = ls.shape.field;
         rep.pair = ls.shape.pair;
