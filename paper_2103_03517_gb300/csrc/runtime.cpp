@@ -155,33 +155,34 @@ bool wave_desc(const mc_desc* d) {
 
 // Lattices whose sweeps may run held in shared memory (resident_pass.cuh):
 // FP32 simple cubic, every axis periodic, no film tables, rows of 64 sites
-// per colour (Lx = 128), not a slab, and either the resident kernel path or
-// the automatic one and kResAutoSpins spins; whether its rows fit is decided
-// on the device (KernelSet::resident_plan).  Below that size the brick sweeps
-// (brick_desc) are faster, their exchange between blocks being shorter: us a
-// sweep resident / brick 10.3 / 5.9 for 128 x 64 x 64, 15.7 / 17.5 for 128^3.
-constexpr uint64_t kResAutoSpins = 3ull << 19;
-
+// per colour (Lx = 128), not a slab, the automatic or resident kernel path;
+// whether its rows fit is decided on the device (KernelSet::resident_plan).
 bool resident_desc(const mc_desc* d, bool slab) {
     if (slab || d->precision != MC_FP32 || d->lattice != MC_SC) return false;
     if (d->kernel_path != MC_PATH_AUTO && d->kernel_path != MC_PATH_RESIDENT) return false;
     if (d->bond_mask || d->grain_id) return false;
     for (int a = 0; a < 3; ++a)
         if (d->boundary[a] != MC_PERIODIC) return false;
-    if (d->kernel_path == MC_PATH_AUTO && uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] < kResAutoSpins) return false;
     return d->dims[0] == 2 * kResLh;
 }
 
 // Lattices whose sweeps may run as brick launches (brick_pass.cuh): FP32
 // simple cubic without film tables, not a slab, the automatic or resident
 // kernel path, at most kBrickMaxSpins spins (whether its rows fit is decided
-// on the device, brick_plan); 128-wide periodic lattices take resident_pass.cuh.
+// on the device, brick_plan).  Of those that can be swept resident, the ones
+// below kResAutoSpins on the automatic path, where the bricks' shorter exchange
+// between blocks makes them faster: us a sweep resident / brick 10.3 / 5.9 for
+// 128 x 64 x 64, 15.7 / 17.5 for 128^3.  Captured by the caller, which takes no
+// brick launch, those are swept resident too.
+constexpr uint64_t kResAutoSpins = 3ull << 19;
 
 bool brick_desc(const mc_desc* d, bool slab) {
-    if (slab || d->precision != MC_FP32 || d->lattice != MC_SC || resident_desc(d, slab)) return false;
+    if (slab || d->precision != MC_FP32 || d->lattice != MC_SC) return false;
     if (d->kernel_path != MC_PATH_AUTO && d->kernel_path != MC_PATH_RESIDENT) return false;
     if (d->bond_mask || d->grain_id) return false;
-    return uint64_t(d->dims[0]) * d->dims[1] * d->dims[2] <= uint64_t(kBrickMaxSpins);
+    const uint64_t spins = uint64_t(d->dims[0]) * d->dims[1] * d->dims[2];
+    if (resident_desc(d, slab) && (d->kernel_path == MC_PATH_RESIDENT || spins >= kResAutoSpins)) return false;
+    return spins <= uint64_t(kBrickMaxSpins);
 }
 
 // Device memory of the brick sweeps of such a lattice, allocated by its first
@@ -938,19 +939,6 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         }
     };
     auto timed = [&](auto&& launch) { timed_kind(constrained ? kTimedPair : kTimedPass, launch); };
-    // all n sweeps held in shared memory, lattice after lattice (see kResMinSweeps)
-    if (!constrained && ls.n_res && k.resident_sweeps && n >= kResMinSweeps) {
-        cudaError_t e = cudaSuccess;
-        const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
-        for (int i = 0; i < ls.n_res && e == cudaSuccess; ++i)
-            for (int done = 0; done < n && e == cudaSuccess; done += most)
-                timed_kind(kTimedResident, [&] {
-                    e = k.resident_sweeps(*ls.res[i], cone, std::min(n - done, most), measure ? ls.sample_level : 0,
-                                          ls.shape.row, s);
-                });
-        if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
-        return MC_OK;
-    }
     // brick launches; after a refused one (launch_refused) the remaining sweeps
     // of its lattices go by launches, and so do later calls
     const int most = measure ? kBrickMaxMeasured : kResMaxSweeps;
@@ -996,6 +984,18 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
                 done += m;
             }
+        return MC_OK;
+    }
+    // or all n sweeps held in shared memory, lattice after lattice (see kResMinSweeps)
+    if (!constrained && ls.n_res && k.resident_sweeps && n >= kResMinSweeps) {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < ls.n_res && e == cudaSuccess; ++i)
+            for (int done = 0; done < n && e == cudaSuccess; done += most)
+                timed_kind(kTimedResident, [&] {
+                    e = k.resident_sweeps(*ls.res[i], cone, std::min(n - done, most), measure ? ls.sample_level : 0,
+                                          ls.shape.row, s);
+                });
+        if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         return MC_OK;
     }
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
@@ -1131,11 +1131,7 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
         (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) ||
          (ls.brick_set && brick_set_ready(ls.brick_set, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
-    // A call on a stream that the caller is capturing: a lattice that the resident
-    // sweeps can hold goes into the caller's graph whole, by launches where its
-    // sweeps are bricks; any other in calls of fewer than kGraphSweeps sweeps.
-    const bool whole = !constrained && ls.brick && ls.brick_lh == kResLh && !ls.brick->faces && capturing(s);
-    const int reps = whole ? 0 : n / kGraphSweeps;
+    const int reps = n / kGraphSweeps;
     if (reps > 0) {
         cudaGraphExec_t& ex = gr.exec[constrained ? 1 : 0][measure ? 1 : 0];
         if (!ex) {

@@ -66,6 +66,7 @@ int autotune(int precision, LaunchSet& ls, const std::vector<mc_lattice*>& lats,
     LaunchSet lt = ls;
     lt.brick = nullptr;
     lt.brick_set = nullptr;
+    if (ls.brick) lt.n_res = 0;
     const bool tune_free = (what & MC_TUNE_SWEEP) && row_kernel;
     const bool tune_cons = (what & MC_TUNE_CONSTRAINED) && (ls.nt_pairs || ls.nt_pairs_lead);
     for (mc_lattice* h : lats) {
