@@ -53,7 +53,8 @@ struct KernelSet {
     // Table A1 colour pass over the lattices of g (ntiles = warp tiles of the
     // launch; the launcher sizes a persistent grid from the occupancy).
     // measure: 0 none, 1 magnetisation and energies, 2 also torques.
-    void (*colour_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure,
+    // now: see row_pass.
+    void (*colour_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, bool now,
                         cudaStream_t s);
     // FP32 colour pass over lattices in the row layout (adjacent site pairs
     // per lane; law = 0) or outside it with rows of even Lh (law = 1: the
@@ -61,11 +62,11 @@ struct KernelSet {
     // gen = 1: any boundaries; gen = 2: film tables, any boundaries; turns: the
     // warps of a block share its tiles in turn (LaunchSet::turns).  Null in the FP64 set.  After a
     // black pass (colour 1) it also launches the close of the lattices' sweeps
-    // (sweep_close_kernel); of measured ones the samples are formed by
-    // sample_close.  Returns the status of the
+    // (sweep_close_kernel); of measured ones the samples are formed there (now) or
+    // by sample_close.  Returns the status of the
     // launches (made with programmatic serialisation).
     cudaError_t (*row_pass)(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law,
-                            int gen, int shape, bool turns, cudaStream_t s);
+                            int gen, int shape, bool turns, bool now, cudaStream_t s);
     // Table A2 pair pass over sub-set (sub, colour) (sub = 0 for simple cubic
     // lattices); leader != 0 takes the pairs in site order
     // (LatParams::pair_leader).

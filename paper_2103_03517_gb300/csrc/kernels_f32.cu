@@ -41,50 +41,50 @@ constexpr int V = kSitesPerThreadF32;
 #include "launchers_common.cuh"
 
 template <int B, int MEASURE, int GEN, int LAW, int TURNS = 0>
-cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
+cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, bool now, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>);
     const Spread sp = spread_warps(ntiles, cap);
     const cudaError_t e =
         launch_chained(row_pass_kernel<B, MEASURE, GEN, 1, LAW, TURNS>, sp.blocks, sp.threads, s, g, ntiles, cone, colour);
     if (e != cudaSuccess || colour != 1) return e;  // the sweep's end
-    return launch_chained(sweep_close_kernel<R>, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
+    return sweep_close(g, MEASURE > 0, now, s);
 }
 
 // launch shape 0: the default blocks per SM of the instance (B0 of a pass
 // without a sample, B0M of one with it); 1: the other candidate, B1
 template <int GEN, int B0, int B0M, int B1, int LAW, int TURNS>
 cudaError_t row_pass_s(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape,
-                       cudaStream_t s) {
+                       bool now, cudaStream_t s) {
     if constexpr (!TURNS) {
         if (shape == 1) {
-            if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, s);
-            if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, s);
-            return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, s);
+            if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, now, s);
+            if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, now, s);
+            return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, now, s);
         }
     }
-    if (measure >= 2) return row_pass_t<B0M, 2, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
-    if (measure == 1) return row_pass_t<B0M, 1, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
-    return row_pass_t<B0, 0, GEN, LAW, TURNS>(g, ntiles, c, colour, s);
+    if (measure >= 2) return row_pass_t<B0M, 2, GEN, LAW, TURNS>(g, ntiles, c, colour, now, s);
+    if (measure == 1) return row_pass_t<B0M, 1, GEN, LAW, TURNS>(g, ntiles, c, colour, now, s);
+    return row_pass_t<B0, 0, GEN, LAW, TURNS>(g, ntiles, c, colour, now, s);
 }
 
 template <int GEN, int B0, int B0M, int B1, int LAW>
 cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape, bool turns,
-                       cudaStream_t s) {
-    if (turns && shape == 0) return row_pass_s<GEN, B0, B0M, B1, LAW, 1>(g, ntiles, c, colour, measure, shape, s);
-    return row_pass_s<GEN, B0, B0M, B1, LAW, 0>(g, ntiles, c, colour, measure, shape, s);
+                       bool now, cudaStream_t s) {
+    if (turns && shape == 0) return row_pass_s<GEN, B0, B0M, B1, LAW, 1>(g, ntiles, c, colour, measure, shape, now, s);
+    return row_pass_s<GEN, B0, B0M, B1, LAW, 0>(g, ntiles, c, colour, measure, shape, now, s);
 }
 
 cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law, int gen,
-                     int shape, bool turns, cudaStream_t s) {
+                     int shape, bool turns, bool now, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
     if (law) {
-        if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
-        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
-        return row_pass_g<0, MINB, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, s);
+        if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
+        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
+        return row_pass_g<0, MINB, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
     }
-    if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
-    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
-    return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, s);
+    if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
+    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
+    return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
 }
 
 template <int C>

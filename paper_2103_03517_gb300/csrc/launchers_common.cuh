@@ -8,25 +8,41 @@
 
 #include "spread.cuh"
 
+// Lattices up to which a launch that forms samples, a block per lattice, is chained
+// as it is: blocks dealt out while the SMs are busy pile up on some, and with
+// them their FP64 chains.  Above it, sweep_close takes blocks of kCloseThreads
+// threads, all but one warp idle, of which an SM holds four, and sample_close is
+// not chained.  A measured sweep by itself, us, one warp chained / one warp not
+// chained / spread blocks chained: 40 x 24^3 40 / 29.5 / 26.6, 8 x 32^3 18.5 /
+// 20.0 / -, 32 lattices of 16^3 ... 128^3 211 / 209 / 206.
+constexpr int kChainedSamples = 16;
+
+// The end of a sweep after its black pass (sweep_close_kernel).
+cudaError_t sweep_close(const GroupArgs& g, bool measure, bool now, cudaStream_t s) {
+    const int threads = measure && now && g.n > kChainedSamples ? kCloseThreads : 32;
+    return launch_chained(sweep_close_kernel<R>, uint32_t(g.n), threads, s, g, measure ? (now ? 2 : 1) : 0);
+}
+
 template <int MEASURE>
-void colour_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, cudaStream_t s) {
+void colour_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int colour, bool now, cudaStream_t s) {
     static const uint32_t cap = resident_blocks(colour_pass_kernel<R, V, MINB, MEASURE>);
     const Spread sp = spread_warps(ntiles, cap);
     const bool full = sp.threads == kBlock;  // FP64: the launch fills the SMs (64^3: 133 -> 127 us a sweep)
     launch_chained_if(!kIsF64<R> || full || chain_small(sp, cap), colour_pass_kernel<R, V, MINB, MEASURE>, sp.blocks, sp.threads, s, g, ntiles, cone, colour);
-    if (colour == 1) launch_chained(sweep_close_kernel<R>, uint32_t(g.n), 32, s, g, MEASURE > 0 ? 1 : 0);
+    if (colour == 1) sweep_close(g, MEASURE > 0, now, s);
 }
 
 // measure: 0 none, 1 magnetisation and energies, 2 also torques
-void colour_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, cudaStream_t s) {
+void colour_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, bool now,
+                 cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
-    if (measure >= 2) colour_pass_t<2>(g, ntiles, c, colour, s);
-    else if (measure == 1) colour_pass_t<1>(g, ntiles, c, colour, s);
-    else colour_pass_t<0>(g, ntiles, c, colour, s);
+    if (measure >= 2) colour_pass_t<2>(g, ntiles, c, colour, now, s);
+    else if (measure == 1) colour_pass_t<1>(g, ntiles, c, colour, now, s);
+    else colour_pass_t<0>(g, ntiles, c, colour, now, s);
 }
 
 void sample_close(const GroupArgs& g, cudaStream_t s) {
-    sample_close_kernel<R><<<uint32_t(g.n), 32 * kSampleRecords, 0, s>>>(g);
+    launch_chained_if(g.n <= kChainedSamples, sample_close_kernel<R>, uint32_t(g.n), 32 * kSampleRecords, s, g);
 }
 
 void sweep_end(const GroupArgs& g, cudaStream_t s) {

@@ -979,8 +979,13 @@ __global__ void __launch_bounds__(kBlock, MINB) colour_pass_kernel(GroupArgs g, 
 // kSampleRecords sweeps at once.  Formed at the end of each pass instead, by its
 // last warp, a sample's FP64 chain stood between two sweeps: a lone 64^3 lattice
 // swept by launches took 20.5 us a measured sweep against 10.7 unmeasured.
+// measure = 2: the sample is formed here, in a call of one sweep (kSamplesNow),
+// which the other launch would only delay (16^3 17.7 -> 13.9 us, 64^3 24.8 ->
+// 21.7, 40 x 24^3 32.3 -> 26.6).
+constexpr int kCloseThreads = 512;
 template <typename R>
-__global__ void sweep_close_kernel(GroupArgs g, int measure) {
+__global__ void __launch_bounds__(kCloseThreads) sweep_close_kernel(GroupArgs g, int measure) {
+    if (threadIdx.x >= 32) return;  // blocks of more threads than one warp only to spread them
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int l = int(blockIdx.x), lane = int(threadIdx.x & 31);
@@ -988,7 +993,7 @@ __global__ void sweep_close_kernel(GroupArgs g, int measure) {
     const LatParams& p = g.lats[l]->p;
     LatState& st = g.lats[l]->st;
     if (p.slab) return;
-    if (measure) {
+    if (measure == 1) {
         long long* r = p.records + size_t(st.nrec) * kRecordWords;
         if (lane < kNumSums)
             r[lane] = (long long)atomicExch(reinterpret_cast<unsigned long long*>(&st.sums[lane]), 0ull);
@@ -999,6 +1004,8 @@ __global__ void sweep_close_kernel(GroupArgs g, int measure) {
             st.nrec += 1;
             st.sweep += 1;
         }
+    } else if (measure) {
+        finalize_sweep(p, st, 1, p.sample_torque != 0, lane);
     } else {
         finalize_sweep(p, st, 0, false, lane);
     }
@@ -1010,6 +1017,7 @@ __global__ void sweep_close_kernel(GroupArgs g, int measure) {
 template <typename R>
 __global__ void __launch_bounds__(32 * kSampleRecords) sample_close_kernel(GroupArgs g) {
     __shared__ double incs[kSampleRecords][kMomentWords];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const LatParams& p = g.lats[blockIdx.x]->p;
     LatState& st = g.lats[blockIdx.x]->st;
     const int lane = int(threadIdx.x & 31), w = int(threadIdx.x >> 5), n = st.nrec;

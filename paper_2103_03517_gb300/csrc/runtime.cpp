@@ -998,15 +998,16 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
         if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
         return MC_OK;
     }
+    const bool now = n <= kSamplesNow;  // samples formed as their sweeps end
     cudaError_t launch_err = cudaSuccess;  // first failed launch of the row kernels
     auto kind_pass = [&](int kind, const GroupArgs& ga, uint32_t nt, int colour, int meas) {
         if (!nt) return;
         if (kind == kColourGeneral) {
-            k.colour_pass(ga, nt, cone, colour, meas, s);
+            k.colour_pass(ga, nt, cone, colour, meas, now, s);
             return;
         }
         const cudaError_t e = k.row_pass(ga, nt, cone, colour, meas, kind >= kColourEven ? 1 : 0,
-                                         (kind - kColourRow) % 3, ls.shape.row, ls.turns[kind], s);
+                                         (kind - kColourRow) % 3, ls.shape.row, ls.turns[kind], now, s);
         if (launch_err == cudaSuccess) launch_err = e;
     };
     auto colour_pass = [&](int colour, int meas) {
@@ -1114,7 +1115,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
                 }
             }
         }
-        if (!constrained && measure && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
+        if (!constrained && measure && !now && (i % kSampleRecords == kSampleRecords - 1 || i + 1 == n))
             k.sample_close(ls.all, s);
     }
     if (launch_err != cudaSuccess) return cuda_fail(launch_err, "row kernel launch");

@@ -25,6 +25,9 @@ struct NvtxRange {
 // [constrained][measure]; built on first use and replayed.
 constexpr int kGraphSweeps = 16;
 static_assert(kGraphSweeps <= kSampleRecords, "a graph's measured sweeps fit a lattice's records");
+// Launched calls of at most this many measured sweeps form each sample in the
+// launch that closes its sweep, instead of all in one more launch.
+constexpr int kSamplesNow = 1;
 // A resident lattice (LatParams::rctl) sweeps held in shared memory in calls
 // of at least this many sweeps; shorter calls, which would not pay for the
 // lattice's load and store, take the row passes (the same chain).

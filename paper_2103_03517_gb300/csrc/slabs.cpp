@@ -89,7 +89,7 @@ MC_API int mc_slab_pass(mc_handle h, int colour, int measure) {
     const LaunchSet ls = single_launch_set(h);
     const int level = measure ? (h->hp.sample_torque ? 2 : 1) : 0;
     const cudaError_t e = kernels_f32().row_pass(ls.col[kColourRowFaces], ls.nt_col[kColourRowFaces], h->cone, colour ^ h->hp.cflip, level, 0, 1,
-                                                 ls.shape.row, ls.turns[kColourRowFaces], h->stream);
+                                                 ls.shape.row, ls.turns[kColourRowFaces], false, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "slab pass");
     return MC_OK;
 }
