@@ -184,6 +184,66 @@ __device__ __forceinline__ bool brick_neighbours(const float* oth, const float4*
     }
 }
 
+// The block's nr rows, both colours, from the lattice (LOAD) or back into it, by
+// WARPS warps.  A unit is 32 sites of a row, or short rows that make up at most
+// 32; a lane moves the six floats of its site index, those of two units (LOAD)
+// before it waits for the first.  A component of a row at a time, each waited for
+// and each with its address formed anew, a block of 192 rows of 32 took 14 us to
+// load and 7.5 to store: 3 sweeps of 8 x 64^3 took 107 us a call that way (75 by
+// launches), 78 this way; 3 of 256 x 100 x 100 100 (92), 86.  Odd rows stay with
+// that way: compiled with the other, their sweeps are slower (138^3 37.1 -> 38.1 us).
+template <bool LOAD, int ODD, int WARPS>
+__device__ __forceinline__ void brick_rows(float* bsm, float* s, const BrickRow* tab, uint32_t nr, uint32_t Lh,
+                                           uint32_t half, uint32_t stride, int warp, int lane) {
+    if constexpr (ODD) {
+        for (int c = 0; c < 2; ++c)
+            for (uint32_t i = uint32_t(warp); i < 3u * nr; i += uint32_t(WARPS)) {
+                const BrickRow& e = tab[i / 3u];
+                const uint32_t comp = i % 3u;
+                float* g = s + size_t(3 * c + int(comp)) * stride + size_t(e.row) * Lh;
+                float* b = bsm + size_t(c) * half + e.own + comp * Lh;
+                const float* src = LOAD ? g : b;
+                float* dst = LOAD ? b : g;
+                for (uint32_t k = uint32_t(lane); k < Lh; k += 32) dst[k] = src[k];
+            }
+        return;
+    }
+    constexpr int U = LOAD ? 2 : 1;
+    const uint32_t segs = (Lh + 31u) / 32u;
+    const uint32_t lg = Lh > 16u ? 5u : 32u - uint32_t(__clz(int(Lh - 1u)));  // lanes of a row: 1 << lg
+    const uint32_t per = 32u >> lg, units = (nr + per - 1u) / per * segs;
+    for (uint32_t u0 = uint32_t(warp); u0 < units; u0 += uint32_t(U * WARPS)) {
+        float v[U][6];
+        float* g[U];
+        float* b[U];
+        bool has[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t u = u0 + uint32_t(j * WARPS);
+            const uint32_t r0 = segs == 1u ? u : u / segs;
+            const uint32_t i = r0 * per + (uint32_t(lane) >> lg);
+            const uint32_t k = 32u * (u - r0 * segs) + (uint32_t(lane) & ((1u << lg) - 1u));
+            has[j] = u < units && i < nr && k < Lh;
+            if (has[j]) {
+                g[j] = s + size_t(tab[i].row) * Lh + k;
+                b[j] = bsm + tab[i].own + k;
+                if (LOAD)
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) v[j][c] = g[j][size_t(c) * stride];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (has[j])
+#pragma unroll
+                for (int c = 0; c < 6; ++c) {
+                    float* const at = b[j] + (c >= 3 ? half : 0u) + uint32_t(c % 3) * Lh;
+                    if (LOAD) *at = v[j][c];
+                    else g[j][size_t(c) * stride] = *at;
+                }
+    }
+}
+
 // LAW 0: packed pairs (row kernels), 1: the general kernel's scalar law;
 // FACES: any boundaries (0: all periodic); ODD: rows of odd Lh (LAW 1);
 // MEASURE as in the row kernel; GROUP: the lattices of grp, each with blocks of
@@ -241,66 +301,61 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         s_fail = 0;
     }
     if (tid < kNumSums) cta_sums[tid] = 0;
-    // the row table: face rows first (ODD: in order), by warp 0
+    // the row table, by warp 0: face rows from its front, the others from its end
+    // (ODD: in order)
     if (warp == 0) {
-        uint32_t at = 0;
-        for (int phase = 0; phase < (ODD ? 1 : 2); ++phase)
-            for (uint32_t i0 = 0; i0 < nr; i0 += 32) {
-                const uint32_t i = i0 + uint32_t(lane);
-                BrickRow e{};
-                bool mine = false;
-                if (i < nr) {
-                    const uint32_t f = ODD ? r0 + i : y0 + i % ny + Ly * (z0 + i / ny);
-                    const uint32_t y = f % Ly, z = f / Ly;
-                    e.own = int(i * rowf);
-                    e.row = f;
-                    bool face = false;
+        uint32_t front = 0, end = nr;
+        for (uint32_t i0 = 0; i0 < nr; i0 += 32) {
+            const uint32_t i = i0 + uint32_t(lane);
+            BrickRow e{};
+            bool mine = false, first = false;
+            if (i < nr) {
+                const uint32_t f = ODD ? r0 + i : y0 + i % ny + Ly * (z0 + i / ny);
+                const uint32_t y = f % Ly, z = f / Ly;
+                e.own = int(i * rowf);
+                e.row = f;
+                bool face = false;
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) {
-                        const bool isz = d >= 2, plus = d & 1;
-                        const uint32_t n = isz ? Lz : Ly, w = isz ? z : y;
-                        const bool cross = plus ? w + 1 == n : w == 0;
-                        const uint32_t w2 = cross ? (plus ? 0 : n - 1) : (plus ? w + 1 : w - 1);
-                        const int bc = isz ? p.bc[2] : p.bc[1];
-                        const bool absent = cross && (bc == 1 || bc == 2);
-                        const uint32_t yn = isz ? y : w2, zn = isz ? w2 : z, fn = yn + Ly * zn;
-                        uint32_t j = 0;  // its place in the block
-                        bool in;
-                        if (ODD) {
-                            in = fn >= r0 && fn < r0 + nr;
-                            j = fn - r0;
-                        } else {
-                            in = yn >= y0 && yn < y0 + ny && zn >= z0 && (zn - z0) * ny < nr;
-                            j = (yn - y0) + ny * (zn - z0);
-                        }
-                        if (absent) {
-                            e.nb[d] = e.own;  // read and multiplied by zero
-                            e.flags |= 1u << (8 + 2 * d);
-                        } else {
-                            e.nb[d] = in ? int(j * rowf) : ~int(fn * Lh);
-                            face = face || !in;
-                            if (cross && bc == 3) e.flags |= 2u << (8 + 2 * d);
-                        }
+                for (int d = 0; d < 4; ++d) {
+                    const bool isz = d >= 2, plus = d & 1;
+                    const uint32_t n = isz ? Lz : Ly, w = isz ? z : y;
+                    const bool cross = plus ? w + 1 == n : w == 0;
+                    const uint32_t w2 = cross ? (plus ? 0 : n - 1) : (plus ? w + 1 : w - 1);
+                    const int bc = isz ? p.bc[2] : p.bc[1];
+                    const bool absent = cross && (bc == 1 || bc == 2);
+                    const uint32_t yn = isz ? y : w2, zn = isz ? w2 : z, fn = yn + Ly * zn;
+                    uint32_t j = 0;  // its place in the block
+                    bool in;
+                    if (ODD) {
+                        in = fn >= r0 && fn < r0 + nr;
+                        j = fn - r0;
+                    } else {
+                        in = yn >= y0 && yn < y0 + ny && zn >= z0 && (zn - z0) * ny < nr;
+                        j = (yn - y0) + ny * (zn - z0);
                     }
-                    e.flags |= ((y + z) & 1u) | (face ? 2u : 0u);
-                    if ((p.bc[1] == 2 && (y == 0 || y + 1 == Ly)) || (p.bc[2] == 2 && (z == 0 || z + 1 == Lz))) e.flags |= 4u;
-                    mine = ODD || face == (phase == 0);
+                    if (absent) {
+                        e.nb[d] = e.own;  // read and multiplied by zero
+                        e.flags |= 1u << (8 + 2 * d);
+                    } else {
+                        e.nb[d] = in ? int(j * rowf) : ~int(fn * Lh);
+                        face = face || !in;
+                        if (cross && bc == 3) e.flags |= 2u << (8 + 2 * d);
+                    }
                 }
-                const uint32_t m = __ballot_sync(0xffffffffu, mine);
-                if (mine) tab[at + uint32_t(__popc(m & ((1u << lane) - 1u)))] = e;
-                at += uint32_t(__popc(m));
+                e.flags |= ((y + z) & 1u) | (face ? 2u : 0u);
+                if ((p.bc[1] == 2 && (y == 0 || y + 1 == Ly)) || (p.bc[2] == 2 && (z == 0 || z + 1 == Lz))) e.flags |= 4u;
+                mine = true;
+                first = ODD || face;
             }
+            const uint32_t below = (1u << lane) - 1u;
+            const uint32_t f = __ballot_sync(0xffffffffu, first), o = __ballot_sync(0xffffffffu, mine && !first);
+            if (mine) tab[first ? front + uint32_t(__popc(f & below)) : end - 1u - uint32_t(__popc(o & below))] = e;
+            front += uint32_t(__popc(f));
+            end -= uint32_t(__popc(o));
+        }
     }
     __syncthreads();
-    // the rows, both colours
-    for (int c = 0; c < 2; ++c)
-        for (uint32_t i = uint32_t(warp); i < 3u * nr; i += uint32_t(NW + 1)) {
-            const BrickRow& e = tab[i / 3u];
-            const uint32_t comp = i % 3u;
-            const float* src = s + size_t(3 * c + int(comp)) * stride + size_t(e.row) * Lh;
-            float* dst = bsm + size_t(c) * half + e.own + comp * Lh;
-            for (uint32_t k = uint32_t(lane); k < Lh; k += 32) dst[k] = src[k];
-        }
+    brick_rows<true, ODD, NW + 1>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
     int theta = L->st.theta;
     const uint32_t sweep0 = L->st.sweep;
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch), T0 = brick_tag0(epoch);
@@ -620,14 +675,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         return;
     }
     // the rows back into the lattice
-    for (int c = 0; c < 2; ++c)
-        for (uint32_t i = uint32_t(warp); i < 3u * nr; i += uint32_t(NW)) {
-            const BrickRow& e = tab[i / 3u];
-            const uint32_t comp = i % 3u;
-            float* dst = s + size_t(3 * c + int(comp)) * stride + size_t(e.row) * Lh;
-            const float* src = bsm + size_t(c) * half + e.own + comp * Lh;
-            for (uint32_t k = uint32_t(lane); k < Lh; k += 32) dst[k] = src[k];
-        }
+    brick_rows<false, ODD, NW>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
 }
 
 // Before a launch (of one lattice, or of many, by blockIdx.y): the control words

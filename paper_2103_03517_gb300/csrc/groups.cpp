@@ -167,8 +167,13 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
         b->lats = g->lats;
         b->plans.resize(size_t(n));
         const double us = brick_group_plan(hp, &b->plans);
-        // against launches: about 8 us a sweep and 10 ps a spin
-        if (us > 0.0 && us < 8.0 + 1e-5 * double(spins)) {
+        // against launches: about 8 us a sweep and 10 ps a spin; where the gain is
+        // below a tenth it takes one sweep more to pay for the lattices' load and
+        // store (8 x 64^3 26.2 us a sweep in calls of 3, 24.3 in calls of 4, 24.9 by
+        // launches)
+        const double launched = 8.0 + 1e-5 * double(spins);
+        if (us > 0.0 && us < launched) {
+            b->min_sweeps = us < 0.9 * launched ? kResMinSweeps : kResMinSweeps + 1;
             g->ls.brick_set = b.get();
             g->brick_set = std::move(b);
         }

@@ -833,9 +833,10 @@ static bool brick_memory(BrickArgs* b, cudaStream_t s) {
     return true;
 }
 
-// The brick set of a group, on first use; false when it cannot be had.
-static bool brick_set_ready(BrickSet* b, cudaStream_t s) {
-    if (b->failed || capturing(s)) return false;
+// The brick set of a group, on first use; false when it cannot be had, or for
+// calls of fewer sweeps than it pays for.
+static bool brick_set_ready(BrickSet* b, int sweeps, cudaStream_t s) {
+    if (sweeps < b->min_sweeps || b->failed || capturing(s)) return false;
     if (b->mem) return true;
     RelaxedCapture relaxed;
     b->failed = true;
@@ -959,7 +960,7 @@ int enqueue_sweeps(const KernelSet& k, const LaunchSet& ls, const void* cone, in
             done += m;
         }
         if (!ls.brick->off) return MC_OK;
-    } else if (!constrained && ls.brick_set && n >= kResMinSweeps && brick_set_ready(ls.brick_set, s)) {
+    } else if (!constrained && ls.brick_set && brick_set_ready(ls.brick_set, n, s)) {
         BrickSet& set = *ls.brick_set;
         for (size_t c = 0; c < set.classes.size(); ++c)
             for (int done = 0; done < n;) {
@@ -1130,7 +1131,7 @@ int run_sweeps(SweepGraphs& gr, int precision, const LaunchSet& ls, const void* 
     // resident sweeps run many to a launch: nothing to capture
     if (!constrained && n >= kResMinSweeps &&
         (ls.n_res || (ls.brick && !ls.brick->off && brick_memory(ls.brick, s)) ||
-         (ls.brick_set && brick_set_ready(ls.brick_set, s))))
+         (ls.brick_set && brick_set_ready(ls.brick_set, n, s))))
         return enqueue_sweeps(k, ls, cone, n, measure, constrained, s, nullptr);
     const int reps = n / kGraphSweeps;
     if (reps > 0) {

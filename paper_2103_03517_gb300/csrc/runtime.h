@@ -54,6 +54,7 @@ struct BrickSet {
     std::vector<BrickArgs> plans;  // splits, one per lattice
     std::vector<BrickClass> classes;
     std::vector<std::vector<mc_lattice*>> members;  // of each class
+    int min_sweeps = kResMinSweeps;  // calls of fewer go by launches
     void* mem = nullptr;           // the classes' device arrays
     bool failed = false;
     BrickSet() = default;
