@@ -128,6 +128,18 @@ void pair_pass_t(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
                       static_cast<const R*>(cone), colour, sub);
 }
 
+// Consecutive pair tiles a warp takes per step: the fewest of 1, 2 and `most` with
+// which about one step a warp does the launch.  Fewer leave a warp a second step
+// when others have none, more leave warps without work; constrained sweeps of
+// periodic lattices alone, us a sweep at 1 / 2 / 4 tiles: 64^3 (0.8 tiles a
+// warp) 25.1 / 27.8 / 35.3, 128 x 128 x 32 (1.7) 40.3 / 30.5 / 38.2, 88^3 (2.2)
+// 63.6 / 55.3 / 58.3, 128 x 96 x 64 (2.5) 65.5 / 54.2 / 52.7, 96^3 (2.8) 72.9 /
+// 59.1 / 53.1, 256 x 64 x 64 (3.4) 75.9 / 57.4 / 45.5.
+int pair_tiles_per_step(uint32_t ntiles, uint32_t warps, int most) {
+    if (ntiles <= warps) return 1;
+    return 5 * ntiles <= 11 * warps ? 2 : most;
+}
+
 // launch shapes: at most {default, 8, 2} tiles per grid-stride step, and the
 // default step with more resident warps per SM: pair order one more block
 // of 256 threads (fewer registers, some spilled), site order blocks of 128
@@ -139,7 +151,7 @@ void pair_pass_s(const GroupArgs& g, uint32_t ntiles, const void* cone, int colo
     constexpr int C0 = LEADER ? kPairChunkLead : kPairChunk;
     constexpr int B0 = LEADER ? MINB_PAIR_LEAD : MINB_PAIR;
     static const uint32_t cap = resident_blocks(pair_pass_kernel<R, B0, C0, LEADER>);
-    const int c = tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : C0);
+    const int c = pair_tiles_per_step(ntiles, cap * (kBlock / 32), shape == 1 ? 8 : shape == 2 ? 2 : C0);
     if (c == 1) pair_pass_t<LEADER, 1>(g, ntiles, cone, colour, sub, s);
     else if (c == 2) pair_pass_t<LEADER, 2>(g, ntiles, cone, colour, sub, s);
     else if (c == 8) pair_pass_t<LEADER, 8>(g, ntiles, cone, colour, sub, s);
