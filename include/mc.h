@@ -374,7 +374,8 @@ MC_API int mc_group_sync(mc_group_handle g);
 /* Launch-shape autotuning of the batched sweeps (the block and tile shapes of
  * a persistent launch).  Candidates, in the order of the report's arrays:
  *   row:   FP32 row kernel, minimum resident blocks per SM (so registers per
- *          thread): {3, 2} (boundaries and films: 2 in passes with a sample);
+ *          thread): {3, 2} (boundaries: 2 in passes with a sample), with film
+ *          tables {2, 3} (2 in passes with a sample);
  *          a lattice swept resident (MC_PATH_RESIDENT): threads per block
  *          {512, 640}; lattices that sweep as bricks: the launches that their
  *          calls of one or two sweeps take;

@@ -12,7 +12,8 @@ namespace mcgb {
 // Launch shapes the autotuner chooses among: an index into each kernel's
 // candidate list (0 = the default, measured best on the batched workloads).
 //   row:   FP32 row kernel, minimum resident blocks per SM (registers per
-//          thread): {3, 2} (boundaries and films: 2 in passes with a sample);
+//          thread): {3, 2} (boundaries: 2 in passes with a sample), with film
+//          tables {2, 3} (2 in passes with a sample);
 //          for a resident lattice, threads per block {512, 640};
 //   pair:  pair pass, consecutive tiles per grid-stride step {4, 8, 2}, and
 //          4 with one more resident block per SM;

@@ -26,11 +26,16 @@ namespace {
 
 using R = float;
 constexpr int MINB = MC_MINB_F32;  // minimum resident blocks per SM of the colour pass
-// The same for the row kernel with faces (GEN 1) and with film tables (GEN 2):
-// three blocks without a sample, two with one, whose sums would spill 160 to
-// 380 bytes a thread at 80 registers.  Film 1024 x 1024 x 15, at two / three
-// blocks: 278 / 253 us a sweep unmeasured, 278 / 347 measured.
-constexpr int MINB_FACES = 3, MINB_FACES_M = 2, MINB_FILM = 3, MINB_FILM_M = 2;
+// The same for the row kernel with faces (GEN 1): three blocks without a sample,
+// two with one, whose sums would spill 160 to 380 bytes a thread at 80 registers.
+constexpr int MINB_FACES = 3, MINB_FACES_M = 2;
+// With film tables (GEN 2) two blocks: at three an unmeasured pass spills too,
+// and most sizes lose.  Unmeasured us a sweep, two / three blocks / three with the
+// warps in turn and a tile's tables read one tile ahead: 128 x 128 x 8 9.5 /
+// 11.7 / 12.2, 256 x 256 x 8 13.6 / 17.6 / 18.1, 512 x 512 x 8 32.7 / 35.5 /
+// 36.6, 500 x 500 x 20 66.8 / 74.6 / 79.9, 1024 x 1024 x 15 224 / 237 / 234
+// (measured 256 / 263 / 280); 768 x 768 x 24 208 / 201 / 201 (236 / 233 / 249).
+constexpr int MINB_FILM = 2;
 constexpr int MINB_PAIR = MC_MINB_PAIR_F32;  // the same for the pair pass
 constexpr int MINB_PAIR_LEAD = 2;            // the same for the pair pass in site order
 constexpr int kPairChunk = MC_PAIR_CHUNK;    // consecutive pair tiles per grid-stride step
@@ -51,14 +56,14 @@ cudaError_t row_pass_t(const GroupArgs& g, uint32_t ntiles, const R* cone, int c
 }
 
 // launch shape 0: the default blocks per SM of the instance (B0 of a pass
-// without a sample, B0M of one with it); 1: the other candidate, B1
-template <int GEN, int B0, int B0M, int B1, int LAW, int TURNS>
+// without a sample, B0M of one with it); 1: the other candidate (B1, B1M)
+template <int GEN, int B0, int B0M, int B1, int B1M, int LAW, int TURNS>
 cudaError_t row_pass_s(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape,
                        bool now, cudaStream_t s) {
     if constexpr (!TURNS) {
         if (shape == 1) {
-            if (measure >= 2) return row_pass_t<B1, 2, GEN, LAW>(g, ntiles, c, colour, now, s);
-            if (measure == 1) return row_pass_t<B1, 1, GEN, LAW>(g, ntiles, c, colour, now, s);
+            if (measure >= 2) return row_pass_t<B1M, 2, GEN, LAW>(g, ntiles, c, colour, now, s);
+            if (measure == 1) return row_pass_t<B1M, 1, GEN, LAW>(g, ntiles, c, colour, now, s);
             return row_pass_t<B1, 0, GEN, LAW>(g, ntiles, c, colour, now, s);
         }
     }
@@ -67,24 +72,25 @@ cudaError_t row_pass_s(const GroupArgs& g, uint32_t ntiles, const R* c, int colo
     return row_pass_t<B0, 0, GEN, LAW, TURNS>(g, ntiles, c, colour, now, s);
 }
 
-template <int GEN, int B0, int B0M, int B1, int LAW>
-cudaError_t row_pass_g(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int shape, bool turns,
-                       bool now, cudaStream_t s) {
-    if (turns && shape == 0) return row_pass_s<GEN, B0, B0M, B1, LAW, 1>(g, ntiles, c, colour, measure, shape, now, s);
-    return row_pass_s<GEN, B0, B0M, B1, LAW, 0>(g, ntiles, c, colour, measure, shape, now, s);
+template <int LAW>
+cudaError_t row_pass_l(const GroupArgs& g, uint32_t ntiles, const R* c, int colour, int measure, int gen, int shape,
+                       bool turns, bool now, cudaStream_t s) {
+    const bool t = turns && shape == 0;
+    if (gen == 2)
+        return row_pass_s<2, MINB_FILM, MINB_FILM, MINB_FILM + 1, MINB_FILM, LAW, 0>(g, ntiles, c, colour, measure, shape, now, s);
+    if (gen == 1) {
+        if (t) return row_pass_s<1, MINB_FACES, MINB_FACES_M, 2, 2, LAW, 1>(g, ntiles, c, colour, measure, shape, now, s);
+        return row_pass_s<1, MINB_FACES, MINB_FACES_M, 2, 2, LAW, 0>(g, ntiles, c, colour, measure, shape, now, s);
+    }
+    if (t) return row_pass_s<0, MINB, MINB, MINB - 1, MINB - 1, LAW, 1>(g, ntiles, c, colour, measure, shape, now, s);
+    return row_pass_s<0, MINB, MINB, MINB - 1, MINB - 1, LAW, 0>(g, ntiles, c, colour, measure, shape, now, s);
 }
 
 cudaError_t row_pass(const GroupArgs& g, uint32_t ntiles, const void* cone, int colour, int measure, int law, int gen,
                      int shape, bool turns, bool now, cudaStream_t s) {
     const R* c = static_cast<const R*>(cone);
-    if (law) {
-        if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
-        if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
-        return row_pass_g<0, MINB, MINB, MINB - 1, 1>(g, ntiles, c, colour, measure, shape, turns, now, s);
-    }
-    if (gen == 2) return row_pass_g<2, MINB_FILM, MINB_FILM_M, MINB_FILM - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
-    if (gen == 1) return row_pass_g<1, MINB_FACES, MINB_FACES_M, MINB_FACES - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
-    return row_pass_g<0, MINB, MINB, MINB - 1, 0>(g, ntiles, c, colour, measure, shape, turns, now, s);
+    if (law) return row_pass_l<1>(g, ntiles, c, colour, measure, gen, shape, turns, now, s);
+    return row_pass_l<0>(g, ntiles, c, colour, measure, gen, shape, turns, now, s);
 }
 
 template <int C>
@@ -107,7 +113,7 @@ void row_field(const GroupArgs& g, uint32_t ntiles, int colour, int shape, cudaS
 // (the next constrained sweep's red field); the other keeps black
 template <int GEN>
 void row_sample_g(const GroupArgs& g, uint32_t ntiles, cudaStream_t s) {
-    constexpr int B = GEN == 2 ? MINB_FILM_M : (GEN == 1 ? MINB_FACES_M : MINB);
+    constexpr int B = GEN == 2 ? MINB_FILM : (GEN == 1 ? MINB_FACES_M : MINB);
     static const uint32_t cap = resident_blocks(row_pass_kernel<B, 2, GEN, 0>);
     const Spread sp = spread_warps(ntiles, cap);
     launch_chained_if(chain_small(sp, cap), row_pass_kernel<B, 2, GEN, 0>, sp.blocks, sp.threads, s, g, ntiles,

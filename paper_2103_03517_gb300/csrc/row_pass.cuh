@@ -198,9 +198,9 @@ __device__ __forceinline__ P3 grain_axes(const LatParams& p, int2 g) {
 // moment they work on neighbouring rows and find each other's rows in L1.  It
 // pays where a row is long (Lh >= 128: the rows a warp alone comes back to have
 // left L1 by then): wall 1024 x 128 x 128 217 -> 186 us a sweep, 256^3 164 ->
-// 158, film 1024 x 1024 x 15 267 -> 253; it does not for the batch of 16^3 ...
-// 128^3 (168 -> 184, where a block also publishes many small lattices once per
-// warp).
+// 158; it does not for the batch of 16^3 ... 128^3 (168 -> 184, where a block also
+// publishes many small lattices once per warp), nor for films, which take more
+// registers (MINB_FILM).
 // MOVE = 0: no moves; the sample of the current state, closing the lattice's
 // sweep as the standalone sample does after a constrained sweep: with colour
 // c, each site of colour c, the site of the other colour with its index, and
@@ -258,29 +258,24 @@ __global__ void __launch_bounds__(kBlock, MINB) row_pass_kernel(GroupArgs g, uin
 #pragma unroll
         for (int i = 0; i < NS; ++i) lf[i] = 0;
         uint32_t nparts = 0;
-        // films: the tables of a tile are read one tile ahead, since its axes hang
-        // on its grains
-        FilmPair ahead{};
-        auto film_at = [&](uint32_t t) {
-            const uint32_t q = (t - t0) * 64u + 2u * uint32_t(lane);
-            return film_pair<(MEASURE > 0)>(p, colour, LAW == 1 ? min(q, p.Nc - 2u) : q);
-        };
-        if constexpr (GEN == 2) ahead = film_at(tile);
         for (; tile < t1; tile += kStep) {
             const uint32_t q0 = (tile - t0) * 64u;
             P3 S, h, O;
             P3 e, eo;  // per-site easy axes (films with grain axes)
             const bool grains = GEN == 2 && p.grain;
-            const FilmPair film = ahead;
+            FilmPair film{};
             if constexpr (GEN == 2) {
+                const uint32_t q = q0 + 2u * uint32_t(lane);
+                film = film_pair<(MEASURE > 0)>(p, colour, LAW == 1 ? min(q, p.Nc - 2u) : q);
+            }
+            bool mov[2];
+            const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, film.bonds, S, h, O, mov);
+            if constexpr (GEN == 2) {  // after the spins' loads, so that these do not wait for the grains
                 if (grains) {
                     e = grain_axes(p, film.g);
                     if (MEASURE > 0) eo = grain_axes(p, film.go);
                 }
-                if (tile + kStep < t1) ahead = film_at(tile + kStep);
             }
-            bool mov[2];
-            const uint32_t site0 = row_pair_sums<GEN, LAW>(p, s, colour, q0, lane, film.bonds, S, h, O, mov);
             const bool valid = LAW == 0 || q0 + 2u * uint32_t(lane) < p.Nc;
             if (!grains) e = eo = P3{p2(e_ax.x), p2(e_ax.y), p2(e_ax.z)};
             P3 Sf = S;

@@ -611,8 +611,8 @@ BrickArgs* brick_of(mc_lattice* h) {
 }
 
 // Lattices whose row-kernel passes take a block's tiles in turn (TURNS in
-// row_pass.cuh): long rows, and tiles enough that a block lies in one or two
-// lattices.
+// row_pass.cuh; films never do): long rows, and tiles enough that a block lies in
+// one or two lattices.
 bool long_rows(const LatParams& p) { return p.Lh >= 128 && p.nblocks_site >= 1024; }
 
 // Launch tables of the lattice alone (one colour-pass kernel).
