@@ -174,8 +174,7 @@ cudaError_t brick_sweeps(const BrickArgs& b, uint32_t Lh, const void* cone, int 
     if (e == cudaSuccess) e = launch_any(a, Lh, static_cast<const float*>(cone), measure, s);
     *ran = e == cudaSuccess;
     if (*ran && measure) {
-        brick_close_kernel<4><<<(n + 3) / 4, 128, 0, s>>>(a, static_cast<const BrickArgs*>(nullptr), n);
-        e = cudaGetLastError();
+        e = brick_close(a, static_cast<const BrickArgs*>(nullptr), 1, n, s);
     }
     return e;
 }
@@ -192,8 +191,7 @@ cudaError_t brick_group_sweeps(const BrickClass& c, const void* cone, int n, int
                        : launch_m<1, 0, 0, 1>(none, g, c.blocks, c.smem, c32, measure, s);
     *ran = e == cudaSuccess;
     if (*ran && measure) {
-        brick_close_kernel<4><<<dim3(uint32_t(n + 3) / 4, uint32_t(c.n)), 128, 0, s>>>(none, static_cast<const BrickArgs*>(c.args), n);
-        e = cudaGetLastError();
+        e = brick_close(none, static_cast<const BrickArgs*>(c.args), c.n, n, s);
     }
     return e;
 }

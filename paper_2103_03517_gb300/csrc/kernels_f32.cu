@@ -257,15 +257,15 @@ cudaError_t resident_sweeps(const ResidentPlan& r, const void* cone, int n, int 
     for (int done = 0; done < n;) {
         ResidentArgs a = r.args;
         a.n_sweeps = std::min(n - done, measure ? kBrickMaxMeasured : kResMaxSweeps);
-        cudaError_t e = cudaMemsetAsync(a.ctl, 0, sizeof(ResCtl), s);
-        if (e == cudaSuccess && measure)
-            e = cudaMemsetAsync(a.record, 0, size_t(a.n_sweeps) * kRecordWords * sizeof(long long), s);
+        // the records lie behind the control words (create_lattice): one memset
+        const size_t clear = measure ? size_t(reinterpret_cast<char*>(a.record + size_t(a.n_sweeps) * kRecordWords) -
+                                              reinterpret_cast<char*>(a.ctl))
+                                     : sizeof(ResCtl);
+        cudaError_t e = cudaMemsetAsync(a.ctl, 0, clear, s);
         if (e == cudaSuccess)
             e = shape == 1 ? resident_m<640>(r, a, c, measure, s) : resident_m<512>(r, a, c, measure, s);
         if (e == cudaSuccess && measure) {
-            brick_close_kernel<4><<<(a.n_sweeps + 3) / 4, 128, 0, s>>>(a, static_cast<const ResidentArgs*>(nullptr),
-                                                                       a.n_sweeps);
-            e = cudaGetLastError();
+            e = brick_close(a, static_cast<const ResidentArgs*>(nullptr), 1, a.n_sweeps, s);
         }
         if (e != cudaSuccess) return e;
         done += a.n_sweeps;

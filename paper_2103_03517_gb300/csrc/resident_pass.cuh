@@ -436,6 +436,7 @@ __global__ void __launch_bounds__(NT, 1)
 template <int WARPS, typename Args>
 __global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(const __grid_constant__ Args one, const Args* many,
                                                                 int n) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const Args& a = many ? many[blockIdx.y] : one;
     auto* const ctl = a.ctl;
     long long* const record = a.record;
@@ -476,6 +477,21 @@ __global__ void __launch_bounds__(32 * WARPS) brick_close_kernel(const __grid_co
         st.moments[lane] = m;
     }
     if (lane == 0) st.ring_count = ring + n;
+}
+
+// Its launch, chained to the sweeps' launch.
+template <typename Args>
+cudaError_t brick_close(const Args& one, const Args* many, int lattices, int n, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(uint32_t(n + 3) / 4, uint32_t(lattices));
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, brick_close_kernel<4, Args>, one, many, n);
 }
 
 }  // namespace mcgb

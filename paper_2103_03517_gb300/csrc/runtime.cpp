@@ -488,7 +488,7 @@ int create_lattice(const mc_desc* din, mc_handle* out, const SlabSpec* slab) {
     h->d_group_start_pair = reinterpret_cast<uint32_t*>(take(2 * sizeof(uint32_t)));
     if (slab) p.slab_counts = reinterpret_cast<long long*>(take(kSlabWords * 8));
     if (resident_desc(d, slab != nullptr)) {  // its control words, if its rows fit the SMs
-        void* ctl = take(sizeof(ResCtl));
+        void* ctl = take(sizeof(ResCtl));  // and the records behind it: resident_sweeps clears both at once
         long long* record = reinterpret_cast<long long*>(take(kBrickRecordBytes));
         ResidentPlan* rp = new ResidentPlan();
         if (kernels_f32().resident_plan(p, rp)) {
