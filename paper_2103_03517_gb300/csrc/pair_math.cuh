@@ -211,8 +211,8 @@ __device__ __forceinline__ long long pair_tile_sample(const Par<float>& par, con
 // instead of reduced per tile: the sums are exact integers, so reducing the
 // accumulators once per run of tiles (pair_parts_flush) gives the totals of
 // pair_tile_sample's per-tile reductions.  A lane's part of a tile is below
-// 2^26 in magnitude (at most 12 at scale 2^22), so an int32 holds the parts
-// of kPartTiles = 16 tiles.
+// 2^26 in magnitude (at most 12 at scale 2^22, with couplings of 1 as the sums of a
+// simple cubic lattice have), so an int32 holds the parts of kPartTiles = 16 tiles.
 constexpr int kPartTiles = 16;
 
 template <int MEASURE, int NS>

@@ -237,7 +237,10 @@ __device__ __forceinline__ R xtal_dot(V3<R> S, V3<R> h) {
 // point on lane i (int64).  FP32: a lane adds its sites of 16 tiles in fixed
 // point before the warp adds the lanes, exact integers either way (a warp sum per
 // tile instead: bcc 48^3 591 against 551 us a block of 10 + 10 sweeps, fcc 32^3 748
-// against 704, 96^3 the same).  LEVEL 2: with the torques.
+// against 704, 96^3 the same); of fewer tiles where |S . h|, whose couplings are
+// inside the sum, could take 16 of them out of an int32, and for couplings that take
+// one site out of it the exchange sum is formed in 64 bits.  LEVEL 2: with the
+// torques.
 template <typename R, int TYPE, int J2, int LEVEL>
 __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const __grid_constant__ XtalArgs a, uint32_t ntiles,
                                                              uint32_t tiles_per_subset) {
@@ -252,6 +255,10 @@ __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const
     const V3<R> e_ax{par.e[0], par.e[1], par.e[2]};
     long long fix = 0;
     int lf[NS] = {}, nparts = 0;
+    // tiles whose parts fit an int32 at scale 2^22: |S . h| is at most `most` (up to
+    // the rounding of a unit spin)
+    const float most = 1.01f * (float(TYPE == 1 ? 8 : 12) * fabsf(a.fJ) + (J2 ? 6.0f * fabsf(a.fJ2) : 0.0f));
+    const int parts = most < 512.0f / kPartTiles ? kPartTiles : most < 512.0f ? int(512.0f / most) : 0;
     for (uint32_t tile = wc.begin; tile < wc.end; ++tile) {
         const uint32_t set = tile / tiles_per_subset;  // 2 sub + colour
         const int sub = int(set >> 1), colour = int(set & 1u);
@@ -275,9 +282,16 @@ __global__ void __launch_bounds__(kBlock, kXtalMinb<R>) xtal_sample_kernel(const
         if constexpr (kIsF64<R>) {
             fix += __double2ll_rn(warp_sums_f64<NS>(sums.v, lane) * kFixScale);
         } else {
+            if (parts == 0) {
+                long long ex = __float2ll_rn(sums.v[kSumEx] * float(kFixScaleF32));
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
+                if (lane == kSumEx) fix += ex;
+                sums.v[kSumEx] = 0.0f;
+            }
 #pragma unroll
             for (int i = 0; i < NS; ++i) lf[i] += __float2int_rn(sums.v[i] * float(kFixScaleF32));
-            if (++nparts == kPartTiles) {
+            if (++nparts >= max(parts, 1)) {
                 fix += pair_parts_flush<NS>(lf, lane);
                 nparts = 0;
             }
