@@ -15,6 +15,7 @@ Usage:  python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 Under torchrun (N > 1) the ranks split the batch: each lattice runs on one
 rank, shares balanced by spins (strong scaling, no collective on the data
 path); the time is the max over ranks and the value the batch's updates.
+The result is one JSON line on stdout; the side measurements are one on stderr.
 `--impl reference` times the serial FP64 CPU oracle on the host cores instead.
 """
 from __future__ import annotations
@@ -288,6 +289,20 @@ def reference_arm(args, cfg):
     print(json.dumps(line), flush=True)
 
 
+def print_result(line, side):
+    """The result: one JSON line on stdout, short enough to be read whole by what
+    collects it (with the serving rates and latencies, which the metric names); the
+    side measurements, some 25 KB, are one JSON line on stderr."""
+    served = side.get("serving")
+    if served:
+        steady = served["steady_state"]
+        line = dict(line, serving={"capacity_req_per_s": served["capacity_req_per_s"],
+                                   "steady_state": {k: v for k, v in steady.items() if isinstance(v, (int, float))}})
+    print(json.dumps(line), flush=True)
+    if side:
+        print(json.dumps({"side": side}), file=sys.stderr, flush=True)
+
+
 # ------------------------------------------------------------ GPU arm
 def gpu_arm(args, cfg):
     import torch
@@ -462,8 +477,7 @@ def gpu_arm(args, cfg):
             "gpu_launches": launches,
             "clocks": clk.summary(),
         }
-        line.update(extra)
-        print(json.dumps(line), flush=True)
+        print_result(line, extra)
     if world > 1:
         torch.distributed.destroy_process_group()
 
@@ -1102,7 +1116,7 @@ def main():
     ap.add_argument("--side", default="all",
                     choices=["all", "none", "fp64", "constrained", "anisotropy", "cubes", "general", "stiffness", "films",
                              "precision", "serving", "torque", "wall", "wave", "slabs", "paper"],
-                    help="which side measurements to add to the line")
+                    help="which side measurements to take (printed as a JSON line on stderr)")
     args = ap.parse_args()
     if args.warmup < 3:
         ap.error("--warmup must be >= 3")
