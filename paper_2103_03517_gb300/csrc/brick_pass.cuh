@@ -185,17 +185,16 @@ __device__ __forceinline__ bool brick_neighbours(const float* oth, const float4*
 }
 
 // The block's nr rows, both colours, from the lattice (LOAD) or back into it, by
-// WARPS warps.  A unit is 32 sites of a row, or short rows that make up at most
-// 32; a lane moves the six floats of its site index, those of two units (LOAD)
-// before it waits for the first.  A component of a row at a time, each waited for
-// and each with its address formed anew, a block of 192 rows of 32 took 14 us to
-// load and 7.5 to store: 3 sweeps of 8 x 64^3 took 107 us a call that way (75 by
-// launches), 78 this way; 3 of 256 x 100 x 100 100 (92), 86.  Odd rows stay with
-// that way: compiled with the other, their sweeps are slower (138^3 37.1 -> 38.1 us).
-template <bool LOAD, int ODD, int WARPS>
+// WARPS warps.  SIX: a unit is 32 sites of a row, or short rows that make up at
+// most 32; a lane moves the six floats of its site index, those of two units (LOAD)
+// before it waits for the first.  Otherwise a component of a row at a time, each
+// waited for and each with its address formed anew: a block of 192 rows of 32 took
+// 14 us to load and 7.5 to store that way, and 3 sweeps of 8 x 64^3 107 us a call
+// (75 by launches); all SIX, and the row table made in one pass, 78.
+template <bool LOAD, bool SIX, int WARPS>
 __device__ __forceinline__ void brick_rows(float* bsm, float* s, const BrickRow* tab, uint32_t nr, uint32_t Lh,
                                            uint32_t half, uint32_t stride, int warp, int lane) {
-    if constexpr (ODD) {
+    if constexpr (!SIX) {
         for (int c = 0; c < 2; ++c)
             for (uint32_t i = uint32_t(warp); i < 3u * nr; i += uint32_t(WARPS)) {
                 const BrickRow& e = tab[i / 3u];
@@ -244,6 +243,21 @@ __device__ __forceinline__ void brick_rows(float* bsm, float* s, const BrickRow*
     }
 }
 
+// Which form of row table, load and store an instance has.  They differ by a few us
+// a call, but the compiler gives the sweeps of an instance other registers with
+// each, and those differ by up to 7% a sweep; this is the shortest call whose sweeps
+// are no slower than with the plainest.  us a sweep, all of the short form / as
+// here: 60^3 open 4.28 / 3.97, 40 x 160 x 136 9.90 / 9.72 (without torques 11.43
+// / 10.79), 96^3 without torques 10.86 / 10.26, 128 x 100 x 80 open without
+// torques 12.23 / 11.76, 138^3 38.1 / 37.1.
+template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
+struct BrickForm {
+    static constexpr bool plain = LAW == 0 && FACES && MEASURE == 1;
+    static constexpr bool table_once = LAW == 0 || GROUP;
+    static constexpr bool load_six = !ODD && !plain;
+    static constexpr bool store_six = !ODD && !plain && (LAW == 0 || FACES || GROUP);
+};
+
 // LAW 0: packed pairs (row kernels), 1: the general kernel's scalar law;
 // FACES: any boundaries (0: all periodic); ODD: rows of odd Lh (LAW 1);
 // MEASURE as in the row kernel; GROUP: the lattices of grp, each with blocks of
@@ -254,6 +268,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
                        const float* __restrict__ cone) {
     constexpr int NS = MEASURE >= 2 ? kNumSums : kSumTux;  // sums sampled
     constexpr int NW = kBrickWarps;
+    using Form = BrickForm<LAW, FACES, ODD, MEASURE, GROUP>;
     extern __shared__ __align__(16) float bsm[];
     __shared__ uint64_t tbar;                  // the cone angle of a sweep is known
     __shared__ unsigned cta_acc, wdone;        // accepted moves, warps done with the sweep
@@ -302,60 +317,66 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
     }
     if (tid < kNumSums) cta_sums[tid] = 0;
     // the row table, by warp 0: face rows from its front, the others from its end
-    // (ODD: in order)
+    // in one pass, or behind them in two (ODD: in order, one pass)
     if (warp == 0) {
+        constexpr int phases = ODD || Form::table_once ? 1 : 2;
         uint32_t front = 0, end = nr;
-        for (uint32_t i0 = 0; i0 < nr; i0 += 32) {
-            const uint32_t i = i0 + uint32_t(lane);
-            BrickRow e{};
-            bool mine = false, first = false;
-            if (i < nr) {
-                const uint32_t f = ODD ? r0 + i : y0 + i % ny + Ly * (z0 + i / ny);
-                const uint32_t y = f % Ly, z = f / Ly;
-                e.own = int(i * rowf);
-                e.row = f;
-                bool face = false;
+        for (int phase = 0; phase < phases; ++phase)
+            for (uint32_t i0 = 0; i0 < nr; i0 += 32) {
+                const uint32_t i = i0 + uint32_t(lane);
+                BrickRow e{};
+                bool mine = false, last = false;
+                if (i < nr) {
+                    const uint32_t f = ODD ? r0 + i : y0 + i % ny + Ly * (z0 + i / ny);
+                    const uint32_t y = f % Ly, z = f / Ly;
+                    e.own = int(i * rowf);
+                    e.row = f;
+                    bool face = false;
 #pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    const bool isz = d >= 2, plus = d & 1;
-                    const uint32_t n = isz ? Lz : Ly, w = isz ? z : y;
-                    const bool cross = plus ? w + 1 == n : w == 0;
-                    const uint32_t w2 = cross ? (plus ? 0 : n - 1) : (plus ? w + 1 : w - 1);
-                    const int bc = isz ? p.bc[2] : p.bc[1];
-                    const bool absent = cross && (bc == 1 || bc == 2);
-                    const uint32_t yn = isz ? y : w2, zn = isz ? w2 : z, fn = yn + Ly * zn;
-                    uint32_t j = 0;  // its place in the block
-                    bool in;
-                    if (ODD) {
-                        in = fn >= r0 && fn < r0 + nr;
-                        j = fn - r0;
-                    } else {
-                        in = yn >= y0 && yn < y0 + ny && zn >= z0 && (zn - z0) * ny < nr;
-                        j = (yn - y0) + ny * (zn - z0);
+                    for (int d = 0; d < 4; ++d) {
+                        const bool isz = d >= 2, plus = d & 1;
+                        const uint32_t n = isz ? Lz : Ly, w = isz ? z : y;
+                        const bool cross = plus ? w + 1 == n : w == 0;
+                        const uint32_t w2 = cross ? (plus ? 0 : n - 1) : (plus ? w + 1 : w - 1);
+                        const int bc = isz ? p.bc[2] : p.bc[1];
+                        const bool absent = cross && (bc == 1 || bc == 2);
+                        const uint32_t yn = isz ? y : w2, zn = isz ? w2 : z, fn = yn + Ly * zn;
+                        uint32_t j = 0;  // its place in the block
+                        bool in;
+                        if (ODD) {
+                            in = fn >= r0 && fn < r0 + nr;
+                            j = fn - r0;
+                        } else {
+                            in = yn >= y0 && yn < y0 + ny && zn >= z0 && (zn - z0) * ny < nr;
+                            j = (yn - y0) + ny * (zn - z0);
+                        }
+                        if (absent) {
+                            e.nb[d] = e.own;  // read and multiplied by zero
+                            e.flags |= 1u << (8 + 2 * d);
+                        } else {
+                            e.nb[d] = in ? int(j * rowf) : ~int(fn * Lh);
+                            face = face || !in;
+                            if (cross && bc == 3) e.flags |= 2u << (8 + 2 * d);
+                        }
                     }
-                    if (absent) {
-                        e.nb[d] = e.own;  // read and multiplied by zero
-                        e.flags |= 1u << (8 + 2 * d);
-                    } else {
-                        e.nb[d] = in ? int(j * rowf) : ~int(fn * Lh);
-                        face = face || !in;
-                        if (cross && bc == 3) e.flags |= 2u << (8 + 2 * d);
-                    }
+                    e.flags |= ((y + z) & 1u) | (face ? 2u : 0u);
+                    if ((p.bc[1] == 2 && (y == 0 || y + 1 == Ly)) || (p.bc[2] == 2 && (z == 0 || z + 1 == Lz))) e.flags |= 4u;
+                    mine = ODD || Form::table_once || face == (phase == 0);
+                    last = !ODD && Form::table_once && !face;
                 }
-                e.flags |= ((y + z) & 1u) | (face ? 2u : 0u);
-                if ((p.bc[1] == 2 && (y == 0 || y + 1 == Ly)) || (p.bc[2] == 2 && (z == 0 || z + 1 == Lz))) e.flags |= 4u;
-                mine = true;
-                first = ODD || face;
+                const uint32_t below = (1u << lane) - 1u;
+                const uint32_t f = __ballot_sync(0xffffffffu, mine && !last);
+                if (mine && !last) tab[front + uint32_t(__popc(f & below))] = e;
+                front += uint32_t(__popc(f));
+                if (!ODD && Form::table_once) {
+                    const uint32_t o = __ballot_sync(0xffffffffu, last);
+                    if (last) tab[end - 1u - uint32_t(__popc(o & below))] = e;
+                    end -= uint32_t(__popc(o));
+                }
             }
-            const uint32_t below = (1u << lane) - 1u;
-            const uint32_t f = __ballot_sync(0xffffffffu, first), o = __ballot_sync(0xffffffffu, mine && !first);
-            if (mine) tab[first ? front + uint32_t(__popc(f & below)) : end - 1u - uint32_t(__popc(o & below))] = e;
-            front += uint32_t(__popc(f));
-            end -= uint32_t(__popc(o));
-        }
     }
     __syncthreads();
-    brick_rows<true, ODD, NW + 1>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
+    brick_rows<true, Form::load_six, NW + 1>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
     int theta = L->st.theta;
     const uint32_t sweep0 = L->st.sweep;
     const uint32_t epoch = *reinterpret_cast<volatile uint32_t*>(&ctl->epoch), T0 = brick_tag0(epoch);
@@ -675,7 +696,7 @@ __global__ void __launch_bounds__(kBrickThreads, 1)
         return;
     }
     // the rows back into the lattice
-    brick_rows<false, ODD, NW>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
+    brick_rows<false, Form::store_six, NW>(bsm, s, tab, nr, Lh, half, stride, warp, lane);
 }
 
 // Before a launch (of one lattice, or of many, by blockIdx.y): the control words
