@@ -13,8 +13,10 @@ template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
 cudaError_t launch(const BrickArgs& a, const BrickGroup& g, uint32_t blocks, uint32_t smem, const float* cone,
                    cudaStream_t s) {
     if ((GROUP ? g.n_sweeps : a.n_sweeps) < a.refuse) return cudaErrorInvalidValue;
-    const cudaError_t opt = opt_in_smem(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>);
-    if (opt != cudaSuccess) return opt;
+    if (smem + kResStaticSmem > 48u * 1024u) {  // what any kernel may take
+        const cudaError_t opt = opt_in_smem(brick_sweep_kernel<LAW, FACES, ODD, MEASURE, GROUP>);
+        if (opt != cudaSuccess) return opt;
+    }
     // cooperative: the launch fails rather than run with a block not resident
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
