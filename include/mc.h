@@ -48,8 +48,8 @@ typedef enum mc_status {
     MC_ERR_CUDA = -3,       /* a CUDA call failed (message in mc_last_error)     */
     MC_ERR_TIMEOUT = -4,    /* a bounded device wait gave up (the wavefront,     */
                             /* resident and brick kernels' waits, about one      */
-                            /* second each;                                      */
-                            /* MC_WAVE_INJECT_TIMEOUT=1 or                       */
+                            /* second each); the lattice's spins are undefined   */
+                            /* then (MC_WAVE_INJECT_TIMEOUT=1 or                 */
                             /* MC_RESIDENT_INJECT_TIMEOUT=1 in the environment   */
                             /* when a lattice is created makes its first wait    */
                             /* run out: a test hook)                             */
@@ -70,8 +70,9 @@ typedef enum mc_precision { MC_FP32 = 0, MC_FP64 = 1 } mc_precision;
 typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIPERIODIC = 3 } mc_boundary;
 
 /* Kernels of an FP32 lattice.  AUTO takes a row kernel for the colour
- * passes where the row layout applies (Lh = Lx/2 a power of two <= 64 or a
- * multiple of 64, Nc a multiple of 64) and the general kernel otherwise,
+ * passes where Lh = Lx/2 is even (in the row layout, Lh a power of two <= 64
+ * or a multiple of 64 and Nc a multiple of 64, with packed arithmetic; else
+ * with the general kernel's, bit for bit) and the general kernel otherwise,
  * and walks the constrained pairs in site order (each pair led by the
  * member whose shuffled position is even); a lattice without film tables
  * whose rows fit the SMs' shared memory (up to about 2.8 million spins) runs
@@ -79,9 +80,17 @@ typedef enum mc_boundary { MC_PERIODIC = 0, MC_OPEN = 1, MC_PINNED = 2, MC_ANTIP
  * 3 sweeps: a 128-wide all-periodic one of 1.5 million spins and more resident
  * (see RESIDENT), any other as brick sweeps, one cooperative launch per call of
  * up to 2048 sweeps (512 measured), for which it takes 16 bytes per spin of
- * device memory on first use (without them it sweeps by launches).  A group of
+ * device memory on first use (asked for once: without them, or when the device
+ * refuses the launch, it sweeps by launches from then on).  A group of
  * such lattices with every axis periodic that together fit sweeps them side by
- * side in one such launch.  GENERAL always takes the
+ * side in one such launch.  Under a caller's stream capture no brick launch is
+ * made: a lattice that can be swept resident goes into the graph as one launch
+ * of any number of sweeps, any other by launches, in calls of fewer than 16
+ * sweeps (MC_ERR_CUDA above).  (Test hooks in the environment when a lattice is
+ * created: MC_BRICK_INJECT_REFUSAL=k refuses its brick launches of fewer than k
+ * sweeps, MC_BRICK_INJECT_NOMEM=k fails its first k requests for brick memory,
+ * MC_BRICK_FIRST_EPOCH=n starts the count of its brick launches at n.)  GENERAL
+ * always takes the
  * general colour-pass kernel and the pairs in pair order.  ROW is AUTO
  * without the resident and brick sweeps: a launch for every colour pass.
  * WAVE is ROW, except that on an all-periodic lattice with Lx = 128 and
@@ -347,8 +356,8 @@ MC_API int mc_group_time_passes(mc_group_handle g, int n_sweeps, int measure, do
 /* The same, by kind: avg_ms[0] / launches[0] for the wavefront launches
  * (one sweep of the lattices that take them), [1] for the colour passes of
  * the row and general kernels, [2] for the pair passes of Table A2, [3] for
- * the resident launches (MC_PATH_RESIDENT: each runs up to 2048 of the
- * n_sweeps sweeps, so a launch's time per sweep is avg_ms[3] times
+ * the resident and brick launches (MC_PATH_AUTO: each runs up to 2048 of the
+ * n_sweeps sweeps, 512 measured, so a launch's time per sweep is avg_ms[3] times
  * launches[3] over n_sweeps).  With
  * constrained != 0 the sweeps are constrained sweeps about each lattice's
  * last constraint direction (MC_ERR_STATE before any constrained sweep of

@@ -49,9 +49,12 @@
 // round trips, which every block then waited for: 6.1 us a measured sweep of
 // 32^3 against 3.1 us unmeasured.
 //
-// Every wait is bounded (about one second): the block then raises the abort
-// flag and its workers leave together at the next barrier (a reduction of
-// their fail flags), without writing the lattice back.
+// Every wait is bounded (a count of polls that takes about one second): the block
+// then raises the abort flag, its workers leave together at the next barrier (a
+// reduction of their fail flags) without writing their rows back, and the lattice's
+// error is set.  Its spins are undefined then: until the barrier a lane whose wait
+// ran out still publishes what it computed, and a block that has finished its last
+// pass writes back.
 #pragma once
 #include "resident_pass.cuh"
 
@@ -261,7 +264,9 @@ struct BrickForm {
 // LAW 0: packed pairs (row kernels), 1: the general kernel's scalar law;
 // FACES: any boundaries (0: all periodic); ODD: rows of odd Lh (LAW 1);
 // MEASURE as in the row kernel; GROUP: the lattices of grp, each with blocks of
-// its own that know nothing of the others, instead of `one`.
+// its own that know nothing of the others, instead of `one` (plan and keys then come
+// from memory: these instances spill 22 to 72 bytes a thread at 96 registers, the
+// others at most 24).
 template <int LAW, int FACES, int ODD, int MEASURE, int GROUP>
 __global__ void __launch_bounds__(kBrickThreads, 1)
     brick_sweep_kernel(const __grid_constant__ BrickArgs one, const __grid_constant__ BrickGroup grp,

@@ -141,8 +141,9 @@ MC_API int mc_group_create(const mc_handle* lattices, int n, mc_group_handle* ou
     // lattices held in shared memory: one alone (resident or brick sweeps), or a
     // group made only of large resident ones (one after another) or only of small
     // ones (side by side as brick sweeps).  Both kinds in one group, held one kind
-    // after the other, lose to launches in calls of 20 sweeps: each large lattice
-    // is loaded and stored once a call (the 32-lattice batch 183 -> 193 us a sweep).
+    // after the other, lost to launches in calls of 20 sweeps (the 32-lattice batch
+    // 183 -> 193 us a sweep): each large lattice is loaded and stored once a call.
+    // Longer calls, over which that is spread, have not been measured.
     bool all_res = true, all_brick = n > 1;
     long long spins = 0;
     std::vector<const LatParams*> hp;

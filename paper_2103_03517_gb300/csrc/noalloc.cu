@@ -35,7 +35,10 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 // Memory of the brick sweeps of calls of at least kResMinSweeps sweeps on a
 // lattice of up to kBrickSpins (64^3): control words, records, packets.  Zero at
-// load; the epoch in its control words then counts the calls.
+// load; the epoch in its control words then counts the calls.  The array is there on
+// every device that loads the library, used or not, at 16 bytes a spin, which is what
+// sets the limit: 4 MiB here, 45 MiB for every size that could sweep as bricks (at
+// 80^3 a call of 20 sweeps takes 300 us by launches).
 constexpr long long kBrickSpins = 1 << 18;
 constexpr size_t kBrickOffRecord = 256;
 constexpr size_t kBrickOffPackets = kBrickOffRecord + size_t(kMaxSamples) * kRecordWords * sizeof(long long);

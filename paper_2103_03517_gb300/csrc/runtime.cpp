@@ -171,9 +171,12 @@ bool resident_desc(const mc_desc* d, bool slab) {
 // kernel path, at most kBrickMaxSpins spins (whether its rows fit is decided
 // on the device, brick_plan).  Of those that can be swept resident, the ones
 // below kResAutoSpins on the automatic path, where the bricks' shorter exchange
-// between blocks makes them faster: us a sweep resident / brick 10.3 / 5.9 for
-// 128 x 64 x 64, 15.7 / 17.5 for 128^3.  Captured by the caller, which takes no
-// brick launch, those are swept resident too.
+// between blocks makes them faster: us a sweep resident / brick, long calls, 9.7 /
+// 5.9 for 128 x 64 x 64, 11.8 / 9.3 for 128 x 128 x 64, 10.5 / 10.7 for 128 x 96 x
+// 96 (1.18M spins; calls of 3 sweeps 16.6 / 15.5), 11.8 / 11.5 for 128 x 112 x 96,
+// 13.2 / 13.5 for 128 x 128 x 96 (1.57M), 12.8 / 13.7 for 128 x 112 x 112, 15.7 /
+// 17.5 for 128^3.  Captured by the caller, which takes no brick launch, those below
+// are swept resident too.
 constexpr uint64_t kResAutoSpins = 3ull << 19;
 
 bool brick_desc(const mc_desc* d, bool slab) {
